@@ -143,6 +143,13 @@ unsigned long long kernel_launches() { return g_kernel_launches.load(std::memory
 }  // namespace
 void note_launch() { g_kernel_launches.fetch_add(1, std::memory_order_relaxed); }
 namespace {
+int sm_count() {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
+
 uint32_t *error_word() {
     static std::mutex mu;
     static uint32_t *addr[64] = {nullptr};
@@ -466,6 +473,11 @@ int preprocess_impl(const void *W_dev, bool w16, int m, int K, const pvmvmd_para
         ctx_alloc(c, &c->status, scan_status_words(c->Nx, c->sb)) != cudaSuccess ||
         ctx_alloc(c, &c->status_y, scan_status_words(c->Ny, c->ell)) != cudaSuccess)
         return fail(PVMVMD_E_NOMEM);
+    // the tiled syndrome finds its status words zero and leaves them zero
+    if (cudaMemsetAsync(c->status, 0, scan_status_words(c->Nx, c->sb) * sizeof(unsigned long long), s) != cudaSuccess ||
+        cudaMemsetAsync(c->status_y, 0, scan_status_words(c->Ny, c->ell) * sizeof(unsigned long long), s) !=
+            cudaSuccess)
+        return fail(PVMVMD_E_CUDA);
     // the challenge kernels are few and short; at the highest priority their
     // blocks take SMs as the decrypt's blocks drain instead of queueing
     // behind the rest of the decrypt's grid
@@ -595,11 +607,8 @@ int encode_batch(pvmvmd_ctx *ctx, const uint32_t *X_dev, int B, const pvmvmd_key
     if (!err) return PVMVMD_E_CUDA;
     uint32_t *stp = static_cast<uint32_t *>(st_dev);
     const CodeDev &d = ctx->gx;
-    int C;
-    uint32_t slice;
-    size_t smem;
-    const bool fused = syndrome_fused_plan(ctx->Nx, ctx->t_x, &C, &slice, &smem);
-    if (B >= kLaneMinBatch && ctx->laux && !(fused && C == 1)) {
+    const bool fits = syndrome_fused_fits(ctx->Nx, ctx->t_x);
+    if (B >= kLaneMinBatch && ctx->laux && !fits) {
         // vectors as lanes: every permutation step moves whole rows (a code
         // that fits one CTA's shared memory stays on chip in the fused kernel)
         for (int b0 = 0; b0 < B; b0 += ctx->sb) {
@@ -612,11 +621,30 @@ int encode_batch(pvmvmd_ctx *ctx, const uint32_t *X_dev, int B, const pvmvmd_key
         }
         return PVMVMD_OK;
     }
-    if (fused) {
+    // A code of more than four tiles and a batch of at most one tile per SM:
+    // small CTAs, one per tile, finish sooner than a CTA per vector.  Measured
+    // (one encode and a field add, graph replay, about 8 us of it launches):
+    // K = 4096, B = 8: 16.8 against 25.2 us; K = 2560, B = 8: 17.6 against
+    // 21.4; K = 1001 (four tiles), B = 1: 13.7 and 13.7; back to back the two
+    // tie at one tile per SM (K = 4096, B = 8: 7.1 against 6.7 us a call) and
+    // beyond it the CTA per vector wins (B = 16: 12.1 against 6.7).
+    const bool tiles = syndrome_tiles_eligible((uint32_t)ctx->t_x);
+    const uint32_t ntiles = scan_tiles((uint32_t)ctx->Nx);
+    if (fits && !(tiles && ntiles > 4 && (uint64_t)B * ntiles <= (uint64_t)sm_count())) {
         // sample, scan and gather in one launch per batch, no scratch
-        PV_CUDA(launch_syndrome_fused(*key, kTagMask, 0, ctx->Nx, ctx->t_x, (uint32_t)B, d.pi2inv,
-                                      d.v2p, d.v1, d.pi1inv, d.pi2, d.v2m, d.v1pm, ctx->K, ctx->rate,
-                                      stp, X_dev, Xhat_dev, s, /*pdl=*/true, kSpreadEncode));
+        PV_CUDA(launch_syndrome_fused(*key, kTagMask, 0, ctx->Nx, ctx->t_x, (uint32_t)B, d.pi1inv, d.pi2,
+                                      d.v2m, d.v1pm, ctx->K, ctx->rate, stp, X_dev, Xhat_dev, s));
+        return PVMVMD_OK;
+    }
+    if (tiles) {
+        for (int b0 = 0; b0 < B; b0 += ctx->sb) {
+            const uint32_t nb = (uint32_t)(B - b0 < ctx->sb ? B - b0 : ctx->sb);
+            PV_CUDA(launch_syndrome_tiles(*key, kTagMask, (uint64_t)b0, ctx->Nx, ctx->t_x, nb, d.pi2inv, d.v2p,
+                                          d.v1m, d.pi1inv, ctx->K, ctx->rate, stp + (size_t)b0 * 2 * ctx->t_x,
+                                          ctx->F, ctx->status, err,
+                                          X_dev ? X_dev + (size_t)b0 * ctx->K : nullptr,
+                                          Xhat_dev + (size_t)b0 * ctx->K, s, /*pdl=*/true));
+        }
         return PVMVMD_OK;
     }
     for (int b0 = 0; b0 < B; b0 += ctx->sb) {
@@ -725,23 +753,15 @@ namespace {
 // The verification of a call: challenges e_q <- E_{t_y}^{N_y} shared by the
 // B vectors, g_q = G_y e_q, u_q = e_q^T Q, and accept_b from x_hat_b and
 // y_hat_b, all on stream cs.
-// beside_decrypt: a decrypt of t_x rows per vector runs beside the chain
-// (standard mode), so a large batch keeps its challenge clusters small; in
-// boost mode the chain is the whole decode and gets the wider clusters.
 int verify_chain(pvmvmd_ctx *ctx, const pvmvmd_key *challenge_key, const uint32_t *Xhat_dev,
-                 const uint32_t *Yhat_dev, int B, int32_t *accept_dev, cudaStream_t cs, bool beside_decrypt) {
+                 const uint32_t *Yhat_dev, int B, int32_t *accept_dev, cudaStream_t cs) {
     uint32_t *err = error_word();
     if (!err) return PVMVMD_E_CUDA;
     const CodeDev &d = ctx->gy;
-    int C;
-    uint32_t slice;
-    size_t smem;
-    if (syndrome_fused_plan(ctx->Ny, ctx->t_y, &C, &slice, &smem)) {
-        PV_CUDA(launch_syndrome_fused(*challenge_key, kTagChallenge, 0, ctx->Ny, ctx->t_y,
-                                      (uint32_t)ctx->ell, d.pi2inv, d.v2p, d.v1, d.pi1inv, d.pi2,
-                                      d.v2m, d.v1pm, ctx->m, ctx->rate, ctx->chal, nullptr, ctx->g, cs, false,
-                                      beside_decrypt && B >= kChallengeLargeBatch ? kSpreadChallenge
-                                                                                 : kSpreadChallengeSmallBatch));
+    if (syndrome_tiles_eligible((uint32_t)ctx->t_y)) {
+        PV_CUDA(launch_syndrome_tiles(*challenge_key, kTagChallenge, 0, ctx->Ny, ctx->t_y, (uint32_t)ctx->ell,
+                                      d.pi2inv, d.v2p, d.v1m, d.pi1inv, ctx->m, ctx->rate, nullptr, ctx->Fy,
+                                      ctx->status_y, err, nullptr, ctx->g, cs, false, ctx->Q, ctx->K, ctx->u));
     } else {
         PV_CUDA(launch_sample_sparse(*challenge_key, kTagChallenge, 0, ctx->Ny, ctx->t_y, ctx->ell,
                                      ctx->chal, ctx->status_y, scan_status_words(ctx->Ny, ctx->ell), cs));
@@ -749,8 +769,8 @@ int verify_chain(pvmvmd_ctx *ctx, const pvmvmd_key *challenge_key, const uint32_
                                      ctx->Fy, ctx->status_y, err, cs));
         PV_CUDA(launch_syndrome_gather(d.pi1inv, ctx->m, ctx->rate, ctx->Fy, ctx->Ny, nullptr, ctx->g,
                                        ctx->ell, cs));
+        PV_CUDA(launch_verify_u(ctx->Q, ctx->K, ctx->chal, ctx->t_y, ctx->ell, ctx->u, cs));
     }
-    PV_CUDA(launch_verify_u(ctx->Q, ctx->K, ctx->chal, ctx->t_y, ctx->ell, ctx->u, cs));
     PV_CUDA(launch_check(Xhat_dev, ctx->K, Yhat_dev, ctx->m, ctx->g, ctx->u, (uint32_t)ctx->ell, B,
                          accept_dev, cs));
     return PVMVMD_OK;
@@ -777,7 +797,7 @@ int decode_verify_batch(pvmvmd_ctx *ctx, const void *st_dev, const uint32_t *mas
         PV_CUDA(cudaEventRecord(ctx->fork, s));
         PV_CUDA(cudaStreamWaitEvent(ctx->side, ctx->fork, 0));
     }
-    int st = verify_chain(ctx, challenge_key, Xhat_dev, Yhat_dev, B, accept_dev, cs, mask_out_dev == nullptr);
+    int st = verify_chain(ctx, challenge_key, Xhat_dev, Yhat_dev, B, accept_dev, cs);
     if (st) return st;
     PV_CUDA(launch_decrypt(ctx->PT, ctx->m, static_cast<const uint32_t *>(st_dev), ctx->t_x, (uint32_t)ctx->Nx,
                            Yhat_dev, B, Y_dev, s, mask_out_dev));
@@ -959,6 +979,9 @@ int pvmvmd_bv_preprocess(const int8_t *W_dev, int B, int m, int n, const pvmvmd_
         ctx_alloc(c, &c->eticket, 1) != cudaSuccess ||
         ctx_alloc(c, &c->status, scan_status_words((uint32_t)N2, (uint32_t)ell2)) != cudaSuccess)
         return fail(PVMVMD_E_NOMEM);
+    if (cudaMemsetAsync(c->status, 0, scan_status_words((uint32_t)N2, (uint32_t)ell2) * sizeof(unsigned long long),
+                        s) != cudaSuccess)
+        return fail(PVMVMD_E_CUDA);
     // Q_b = G^T M_b into the column block b n of Qs (the lanes are M_b's columns)
     for (int b = 0; b < B; ++b) {
         st = encode_lanes(c->g, (uint32_t)m, (uint32_t)rate, W_dev + (size_t)b * m * n, true, (size_t)n,
@@ -1014,13 +1037,11 @@ int pvmvmd_bv_check(pvmvmd_bv_ctx *ctx, const uint32_t *X_dev, const uint32_t *Y
     if (st) return st;
     // secondary challenges, drawn after the responses, and r^(j) = G' e'^(j)
     const CodeDev &d = ctx->g2;
-    int C;
-    uint32_t slice;
-    size_t smem;
-    if (syndrome_fused_plan((uint32_t)ctx->N2, (uint32_t)ctx->t2, &C, &slice, &smem)) {
-        PV_CUDA(launch_syndrome_fused(*key2, kTagBvSecondary, 0, (uint32_t)ctx->N2, (uint32_t)ctx->t2,
-                                      (uint32_t)ctx->ell2, d.pi2inv, d.v2p, d.v1, d.pi1inv, d.pi2, d.v2m,
-                                      d.v1pm, Bn, (uint32_t)ctx->rate, ctx->chal2, nullptr, ctx->R, s));
+    if (syndrome_tiles_eligible((uint32_t)ctx->t2)) {
+        PV_CUDA(launch_syndrome_tiles(*key2, kTagBvSecondary, 0, (uint32_t)ctx->N2, (uint32_t)ctx->t2,
+                                      (uint32_t)ctx->ell2, d.pi2inv, d.v2p, d.v1m, d.pi1inv, Bn,
+                                      (uint32_t)ctx->rate, ctx->chal2, ctx->F2, ctx->status, err, nullptr, ctx->R,
+                                      s, false));
     } else {
         PV_CUDA(launch_sample_sparse(*key2, kTagBvSecondary, 0, (uint32_t)ctx->N2, (uint32_t)ctx->t2,
                                      (uint32_t)ctx->ell2, ctx->chal2, ctx->status,

@@ -17,8 +17,12 @@
 #include <map>
 #include <mutex>
 
+#include <cooperative_groups.h>
+
 #include "common.cuh"
 #include "launch.h"
+
+namespace cg = cooperative_groups;
 
 namespace pv {
 namespace {
@@ -226,30 +230,37 @@ __global__ void __launch_bounds__(kDecThreads) k_decrypt(const uint32_t *__restr
 // ---------------------------------------------------------------------------
 // Verify: accept_b = AND_q [ L_q == R_q ] with L_q = u_q . x_hat_b and
 // R_q = g_q . y_hat_b (= e_q^T (G_y^T y_hat_b) by transposition), u_q =
-// e_q^T Q and g_q = G_y e_q from the challenge kernels.  One CTA per vector;
-// the repetitions run one after the other over the (cached) vectors.
+// e_q^T Q and g_q = G_y e_q from the challenge kernels.  One cluster of up to
+// eight CTAs per vector; the repetitions run one after the other over the (cached) vectors.
 // ---------------------------------------------------------------------------
-// 512 threads with eight loads of each operand in flight (1024 threads with
-// four, an SM's whole register file per CTA, waited longer for SMs beside
-// the decrypts: 8B layer 0.500 -> 0.492 ms, 70B layer 2.218 -> 2.191 ms per
-// step, the batch-1 workload unchanged at 0.320 ms; 256 threads were
-// slower)
-constexpr int kCheckThreads = 512;
-constexpr int kCheckBatch = 8;  // loads in flight per operand and thread
+// The S CTAs of a cluster (256 threads, four loads of each operand in flight
+// per thread) take one slice of the columns each and add their sums through
+// distributed shared memory: small CTAs find room beside a decrypt's (one CTA
+// of 512 threads per vector took 15.5 us cold for 14336 x 4096, 64 vectors).
+constexpr int kCheckThreads = 256;
+constexpr int kCheckBatch = 4;      // loads in flight per operand and thread
+constexpr int kCheckSlice = 2048;   // columns a CTA takes, where eight CTAs suffice
+constexpr int kCheckMaxCluster = 8;
 
-__global__ void __launch_bounds__(kCheckThreads) k_check(const uint32_t *__restrict__ Xhat, int K,
-                                                        const uint32_t *__restrict__ Yhat, int m,
-                                                        const uint32_t *__restrict__ g,
-                                                        const uint32_t *__restrict__ u, uint32_t ell,
-                                                        int32_t *__restrict__ accept) {
+__global__ void __launch_bounds__(kCheckThreads, 4) k_check(const uint32_t *__restrict__ Xhat, int K,
+                                                           const uint32_t *__restrict__ Yhat, int m,
+                                                           const uint32_t *__restrict__ g,
+                                                           const uint32_t *__restrict__ u, uint32_t ell,
+                                                           int32_t *__restrict__ accept) {
+    cg::cluster_group cluster = cg::this_cluster();
     __shared__ uint32_t s_part[4][kCheckThreads / 32];
+    __shared__ uint32_t s_sum[4];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const size_t b = blockIdx.x;
+    const uint32_t S = cluster.num_blocks(), rank = cluster.block_rank();
+    const size_t b = blockIdx.y;
     const uint32_t *xh = Xhat + b * K, *yh = Yhat + b * m;
     // the kernel after this one (the next call's encode) may start its
-    // key-only work now
+    // key-only work now; g and u come from the kernels before
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int n = K > m ? K : m;
+    const int per = (n + (int)S - 1) / (int)S;
+    const int n0 = (int)rank * per, n1 = min(n, n0 + per);
     int ok = 1;
     // two repetitions per pass: x_hat and y_hat are read once per pair
     for (uint32_t q = 0; q < ell; q += 2) {
@@ -257,37 +268,34 @@ __global__ void __launch_bounds__(kCheckThreads) k_check(const uint32_t *__restr
         const uint32_t *u0 = u + (size_t)q * K, *g0 = g + (size_t)q * m;
         const uint32_t *u1 = two ? u0 + K : u0, *g1 = two ? g0 + m : g0;
         uint64_t l0 = 0, l1 = 0, r0 = 0, r1 = 0;
-        for (int k0 = tid; k0 < n; k0 += kCheckBatch * kCheckThreads) {
+        for (int k0 = n0 + tid; k0 < n1; k0 += kCheckBatch * kCheckThreads) {
             uint32_t x[kCheckBatch], y[kCheckBatch], a0[kCheckBatch], a1[kCheckBatch], c0[kCheckBatch],
                 c1[kCheckBatch];
 #pragma unroll
             for (int v = 0; v < kCheckBatch; ++v) {
                 const int k = k0 + v * kCheckThreads;
-                const bool kx = k < K, ky = k < m;
+                const bool kx = k < n1 && k < K, ky = k < n1 && k < m;
                 x[v] = kx ? xh[k] : 0u;
-                a0[v] = kx ? __ldg(u0 + k) : 0u;
-                a1[v] = kx ? __ldg(u1 + k) : 0u;
+                a0[v] = kx ? __ldcg(u0 + k) : 0u;
+                a1[v] = kx ? __ldcg(u1 + k) : 0u;
                 y[v] = ky ? yh[k] : 0u;
-                c0[v] = ky ? __ldg(g0 + k) : 0u;
-                c1[v] = ky ? __ldg(g1 + k) : 0u;
+                c0[v] = ky ? __ldcg(g0 + k) : 0u;
+                c1[v] = ky ? __ldcg(g1 + k) : 0u;
             }
             // four products of values below q stay below 2^64 with the
-            // reduced running sum, so the sums are reduced every four
+            // reduced running sum
+            static_assert(kCheckBatch <= 4, "sums reduced after at most four products");
 #pragma unroll
-            for (int v0 = 0; v0 < kCheckBatch; v0 += 4) {
-#pragma unroll
-                for (int v = v0; v < v0 + 4; ++v) {
-                    l0 += (uint64_t)a0[v] * x[v];
-                    l1 += (uint64_t)a1[v] * x[v];
-                    r0 += (uint64_t)c0[v] * y[v];
-                    r1 += (uint64_t)c1[v] * y[v];
-                }
-                l0 = fred(l0);
-                l1 = fred(l1);
-                r0 = fred(r0);
-                r1 = fred(r1);
+            for (int v = 0; v < kCheckBatch; ++v) {
+                l0 += (uint64_t)a0[v] * x[v];
+                l1 += (uint64_t)a1[v] * x[v];
+                r0 += (uint64_t)c0[v] * y[v];
+                r1 += (uint64_t)c1[v] * y[v];
             }
-            static_assert(kCheckBatch % 4 == 0, "sums reduced every four products");
+            l0 = fred(l0);
+            l1 = fred(l1);
+            r0 = fred(r0);
+            r1 = fred(r1);
         }
         const uint32_t w0 = warp_fsum((uint32_t)l0), w1 = warp_fsum((uint32_t)l1);
         const uint32_t w2 = warp_fsum((uint32_t)r0), w3 = warp_fsum((uint32_t)r1);
@@ -298,20 +306,25 @@ __global__ void __launch_bounds__(kCheckThreads) k_check(const uint32_t *__restr
             s_part[3][warp] = w3;
         }
         __syncthreads();
-        if (tid == 0) {
-            uint32_t L0 = 0, L1 = 0, R0 = 0, R1 = 0;
-            for (int w = 0; w < kCheckThreads / 32; ++w) {
-                L0 = fadd(L0, s_part[0][w]);
-                L1 = fadd(L1, s_part[1][w]);
-                R0 = fadd(R0, s_part[2][w]);
-                R1 = fadd(R1, s_part[3][w]);
-            }
-            ok &= (L0 == R0);
-            if (two) ok &= (L1 == R1);
+        if (tid < 4) {
+            uint32_t sum = 0;
+            for (int w = 0; w < kCheckThreads / 32; ++w) sum = fadd(sum, s_part[tid][w]);
+            s_sum[tid] = sum;
         }
-        __syncthreads();
+        cluster.sync();
+        if (rank == 0 && tid == 0) {
+            uint32_t t[4] = {0u, 0u, 0u, 0u};
+            for (uint32_t c = 0; c < S; ++c) {
+                const uint32_t *ps = cluster.map_shared_rank(s_sum, c);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) t[i] = fadd(t[i], ps[i]);
+            }
+            ok &= (t[0] == t[2]);
+            if (two) ok &= (t[1] == t[3]);
+        }
+        cluster.sync();  // the sums are read before a CTA writes the next ones or exits
     }
-    if (tid == 0) accept[b] = ok;
+    if (rank == 0 && tid == 0) accept[b] = ok;
 }
 
 // out[b][col] = (P e_x,b)_col for the columns of this CTA (1024 per CTA).
@@ -451,8 +464,29 @@ cudaError_t launch_decrypt(const uint32_t *PT, int m, const uint32_t *st, uint32
 cudaError_t launch_check(const uint32_t *Xhat, int K, const uint32_t *Yhat, int m, const uint32_t *g,
                          const uint32_t *u, uint32_t ell, int B, int32_t *accept, cudaStream_t s) {
     if (B <= 0) return cudaSuccess;
-    k_check<<<(unsigned)B, kCheckThreads, 0, s>>>(Xhat, K, Yhat, m, g, u, ell, accept); note_launch();
-    return cudaGetLastError();
+    const int n = K > m ? K : m;
+    unsigned S = 1;
+    while (S < (unsigned)kCheckMaxCluster && (int64_t)S * kCheckSlice < n) S *= 2;
+    for (int b0 = 0; b0 < B; b0 += 65535) {
+        const int nb = B - b0 < 65535 ? B - b0 : 65535;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(S, (unsigned)nb, 1);
+        cfg.blockDim = dim3(kCheckThreads, 1, 1);
+        cfg.stream = s;
+        cudaLaunchAttribute attr[2];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = S;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[1].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 2;
+        const cudaError_t e = counted_launch(cudaLaunchKernelEx(&cfg, k_check, Xhat + (size_t)b0 * K, K,
+                                                                Yhat + (size_t)b0 * m, m, g, u, ell, accept + b0));
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace pv

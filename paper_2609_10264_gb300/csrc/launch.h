@@ -39,36 +39,21 @@ cudaError_t launch_syndrome_scan(const uint32_t *pi2inv, const uint32_t *v2p, co
                                  uint32_t *F, unsigned long long *status, uint32_t *err,
                                  cudaStream_t s);
 
-// Cluster spread of the fused syndrome (how far a small batch's clusters
-// grow): encodes of a few vectors, and the few shared challenges of a
-// verification, each measured best at a different setting.  The challenges
-// of a large batch run beside a large decrypt and keep their clusters
-// small; those of a small batch, and those of boost mode (no decrypt of
-// P^T rows beside them), are the decode's critical path.
-constexpr int kSpreadEncode = 4;
-constexpr int kSpreadChallenge = 16;
-constexpr int kSpreadChallengeSmallBatch = 4;
-constexpr int kChallengeLargeBatch = 32;
-
 // Fused syndrome for `count` freshly sampled sparse vectors (as
 // launch_sample_sparse, then out = addend + G e) in one launch with the
-// intermediate in cluster shared memory.  sparse_out: [count][2t];
-// out (and addend, may alias): [count][n].  cudaErrorNotSupported when N is
-// too long for one cluster (use the three-kernel path).
-bool syndrome_fused_plan(uint32_t N, uint32_t t, int *C, uint32_t *slice, size_t *smem);
-// Tables: pi2inv, v2p = v2 o pi2^-1, v1 (cluster form); pi2, v2m = v2 R,
-// v1pm = (v1 o pi1^-1) R (single-CTA form, Montgomery-scaled, R = 2^32).
-// pdl: launch with programmatic stream serialisation.  The kernel reads
-// nothing but the key and the tables before griddepcontrol.wait, so its
-// sampling and scans overlap the kernel before it; st, out and addend are
-// touched only after the wait.
+// intermediate in shared memory, where the code fits one CTA's.
+// sparse_out: [count][2t]; out (and addend, may alias): [count][n].
+// Tables: pi1inv, pi2, v2m = v2 R, v1pm = (v1 o pi1^-1) R (R = 2^32).
+// Launched with programmatic stream serialisation: the kernel reads nothing
+// but the key and the tables before griddepcontrol.wait, so its sampling and
+// scans overlap the kernel before it; st, out and addend are touched only
+// after the wait.
+bool syndrome_fused_fits(uint32_t N, uint32_t t);
 cudaError_t launch_syndrome_fused(const pvmvmd_key &key, uint32_t tag, uint64_t idx0, uint32_t N,
-                                  uint32_t t, uint32_t count, const uint32_t *pi2inv,
-                                  const uint32_t *v2p, const uint32_t *v1, const uint32_t *pi1inv,
+                                  uint32_t t, uint32_t count, const uint32_t *pi1inv,
                                   const uint32_t *pi2, const uint32_t *v2m, const uint32_t *v1pm,
                                   uint32_t n, uint32_t r, uint32_t *sparse_out,
-                                  const uint32_t *addend, uint32_t *out, cudaStream_t s,
-                                  bool pdl = false, int spread = kSpreadChallenge);
+                                  const uint32_t *addend, uint32_t *out, cudaStream_t s);
 
 // Lane-parallel syndrome for L vectors (vector b uses index idx0 + b, as
 // launch_sample_sparse): sparse_out [L][2t] as there, S lane_state_words(t,
@@ -89,7 +74,22 @@ cudaError_t launch_lane_syndrome(const pvmvmd_key &key, uint32_t tag, uint64_t i
 // (addend may be null; out may alias addend).
 cudaError_t launch_syndrome_gather(const uint32_t *pi1inv, uint32_t n, uint32_t r,
                                    const uint32_t *F, uint32_t N, const uint32_t *addend,
-                                   uint32_t *out, uint32_t count, cudaStream_t s);
+                                   uint32_t *out, uint32_t count, cudaStream_t s,
+                                   unsigned long long *status = nullptr, uint32_t nclear = 0);
+
+// Tiled syndrome (k_syndrome_tiles, then the gather) for `count` freshly
+// sampled vectors of sparsity t <= 256 and any N: sparse_out [count][2t] (may
+// be null), F [count][N] scratch, status count * scan_tiles(N) words, zero at
+// the call and zero again after it.  With u non-null also
+// u[q][k] = sum_j e_{q,j} Qm[supp_{q,j}][k] for k < K.  pdl: launched as
+// launch_syndrome_fused is (st, F, status and out are touched after the wait).
+bool syndrome_tiles_eligible(uint32_t t);
+cudaError_t launch_syndrome_tiles(const pvmvmd_key &key, uint32_t tag, uint64_t idx0, uint32_t N, uint32_t t,
+                                  uint32_t count, const uint32_t *pi2inv, const uint32_t *v2p,
+                                  const uint32_t *v1m, const uint32_t *pi1inv, uint32_t n, uint32_t r,
+                                  uint32_t *sparse_out, uint32_t *F, unsigned long long *status, uint32_t *err,
+                                  const uint32_t *addend, uint32_t *out, cudaStream_t s, bool pdl,
+                                  const uint32_t *Qm = nullptr, int K = 0, uint32_t *u = nullptr);
 
 // Every kernel launch site calls note_launch() (or wraps a cudaLaunchKernelEx
 // in counted_launch), so that pvmvmd_kernel_launches counts what the library

@@ -6,18 +6,17 @@
 //                         accumulator as a single-pass decoupled look-back scan.
 //  * k_syndrome_gather    second half: inverse permutation gather and the
 //                         block sums of R, fused with x_hat = x + x'.
+//  * k_syndrome_tiles     the syndrome's first half for a few vectors, or a few
+//                         shared challenges: every CTA samples e itself and
+//                         takes one tile of 2048 positions.
 //  * k_encode_scan        one accumulate stage of the encoding G^T w over many
 //                         lanes (preprocessing of P^T and Q, Sec. 6.3).
 //  * k_lane_*             the syndrome for a batch of vectors held as the lanes
 //                         of an N x B array (sample, step function, scan, gather).
 #include <map>
 #include <mutex>
-#include <cooperative_groups.h>
-
 #include "common.cuh"
 #include "launch.h"
-
-namespace cg = cooperative_groups;
 
 namespace pv {
 namespace {
@@ -106,6 +105,51 @@ __device__ void warp_sample_support_list(const pvmvmd_key &key, uint32_t tag, ui
                 atomicOr(&bitmap[v >> 5], 1u << (v & 31));
                 list[have + rk] = v;
             }
+            have += min((uint32_t)__popc(cmask), need);
+            __syncwarp();
+        }
+        __syncwarp();
+    }
+}
+
+// Warp: the support of e <- E_t^N in the order accepted -> list[0..t), for
+// t <= kTileMaxT without a bitmap: a draw is compared with the list itself
+// (16 bytes per shared-memory read, every lane the same address).  list is
+// 16-byte aligned and holds kTileMaxT words.
+constexpr uint32_t kTileMaxT = 256;
+__device__ void warp_sample_support_short(const pvmvmd_key &key, uint32_t tag, uint64_t sidx, uint32_t N,
+                                          uint32_t t, uint32_t *words, uint32_t *list, int lane) {
+    // unused slots hold a value no draw takes (draws are below N)
+    for (uint32_t i = lane; i < kTileMaxT; i += 32) list[i] = 0xffffffffu;
+    __syncwarp();
+    if (N <= 1) {
+        if (lane == 0) list[0] = 0u;
+        __syncwarp();
+        return;
+    }
+    const int shift = 32 - bitlen32(N - 1);
+    uint32_t have = 0;
+    for (uint64_t wpos = 0; have < t; wpos += 512) {
+        uint32_t blk[16];
+        chacha20_block_dev(key, (uint32_t)(wpos / 16 + lane), tag, (uint32_t)sidx,
+                           (uint32_t)(sidx >> 32), blk);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) words[lane * 16 + i] = blk[i];
+        __syncwarp();
+        for (int batch = 0; batch < 16 && have < t; ++batch) {
+            const uint32_t v = words[batch * 32 + lane] >> shift;
+            const bool valid = v < N;
+            bool seen = false;
+            for (uint32_t h = 0; h < have; h += 4) {
+                const uint4 a = *reinterpret_cast<const uint4 *>(list + h);
+                seen |= (a.x == v) | (a.y == v) | (a.z == v) | (a.w == v);
+            }
+            const uint32_t vmask = __ballot_sync(kFull, valid);
+            const uint32_t same = __match_any_sync(kFull, valid ? v : 0xffffffffu);
+            const bool cand = valid && !seen && (same & vmask & lanemask_lt()) == 0u;
+            const uint32_t cmask = __ballot_sync(kFull, cand);
+            const uint32_t need = t - have, rk = __popc(cmask & lanemask_lt());
+            if (cand && rk < need) list[have + rk] = v;
             have += min((uint32_t)__popc(cmask), need);
             __syncwarp();
         }
@@ -343,59 +387,287 @@ __global__ void __launch_bounds__(kScanThreads) k_syndrome_scan(
     }
 }
 
+// -----------------------------------------------------------------------------
+// Tiled syndrome, first half, for `count` freshly sampled sparse vectors:
+// every CTA of 256 threads takes one tile of kScanTile positions of one vector
+// and draws that vector's e itself (a draw costs about 2 us of latency and no
+// traffic), so one launch holds as many small CTAs as there are tiles; they
+// fit beside a decrypt's.  The tables of a tile are requested before the
+// draw.  Tile sums are chained by a look-back over the tiles after it: their
+// own sums only, 32 at a time by one warp, since all of them are published
+// at about the same time.  A tile waits only for CTAs of lower index, which
+// the GPU starts first.  status holds one 64-bit word per (vector, tile)
+// (1 << 32 | sum), zero at launch; the gather kernel that follows clears it.
+//
+// Latency-bound.  Against one cluster of 2 to 8 CTAs of 1024 threads per
+// vector (and e^T Q in a kernel after it): decode of 14336 x 4096, 64 vectors
+// 115.1 -> 101.6 us, of 4096 x 4096, 100 vectors 55.9 -> 49.4 us; round trip of
+// 4096 x 2560, 8 vectors, 16-bit weights 91.7 -> 67.8 us; a mask alone, 8
+// vectors: K = 8192 43.1 -> 20.6 us, K = 30000 77.3 -> 44.8 us.
+//
+// With ucols != 0, ucols more CTAs per vector form u = e^T Q (64 columns
+// each, the t rows over four row groups as in k_verify_u): u needs e alone,
+// so it runs beside the scan instead of after the syndrome.
+// -----------------------------------------------------------------------------
+constexpr int kTileUCols = 64, kTileUGroups = kScanThreads / kTileUCols;
+__global__ void __launch_bounds__(kScanThreads, 4) k_syndrome_tiles(
+    pvmvmd_key key, uint32_t tag, uint64_t idx0, uint32_t N, uint32_t t, uint32_t count,
+    const uint32_t *__restrict__ pi2inv, const uint32_t *__restrict__ v2p, const uint32_t *__restrict__ v1m,
+    uint32_t *__restrict__ sparse_out, uint32_t *__restrict__ F, unsigned long long *__restrict__ status,
+    uint32_t *__restrict__ err, uint32_t skip_tile, uint32_t spin_limit, const uint32_t *__restrict__ Qm, int K,
+    uint32_t ucols, uint32_t *__restrict__ u) {
+    __shared__ __align__(16) uint32_t s_list[kTileMaxT];
+    __shared__ uint32_t s_supp[kTileMaxT], s_val[kTileMaxT], s_suf[kTileMaxT + 1];
+    __shared__ uint32_t s_words[2][512];
+    __shared__ uint32_t s_wsum[kScanThreads / 32], s_agg, s_prefix;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int nw = kScanThreads / 32;
+    const uint32_t ntiles = scan_tiles(N), nscan = count * ntiles;
+    const bool scan = blockIdx.x < nscan;
+    const uint32_t vec = scan ? blockIdx.x / ntiles : (blockIdx.x - nscan) / ucols;
+    const uint32_t tile = scan ? ntiles - 1 - blockIdx.x % ntiles : 0u;  // from the end of the vector
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+    const uint32_t base = tile * kScanTile + tid * kScanItems;
+    uint32_t idx[kScanItems], scale[kScanItems];
+    if (scan) {
+        if (base + kScanItems <= N) {
+#pragma unroll
+            for (int h = 0; h < kScanItems; h += 4) {
+                const uint4 a = __ldg(reinterpret_cast<const uint4 *>(pi2inv + base + h));
+                const uint4 b = __ldg(reinterpret_cast<const uint4 *>(v2p + base + h));
+                idx[h] = a.x; idx[h + 1] = a.y; idx[h + 2] = a.z; idx[h + 3] = a.w;
+                scale[h] = b.x; scale[h + 1] = b.y; scale[h + 2] = b.z; scale[h + 3] = b.w;
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < kScanItems; ++i) {
+                const bool ok = base + i < N;
+                idx[i] = ok ? __ldg(pi2inv + base + i) : 0u;
+                scale[i] = ok ? __ldg(v2p + base + i) : 0u;
+            }
+        }
+    }
+
+    // ---- e: warp 0 the support, warp 1 the values
+    const uint64_t vidx = idx0 + vec;
+    if (warp == 0) warp_sample_support_short(key, tag, 2 * vidx, N, t, s_words[0], s_list, lane);
+    else if (warp == 1) warp_sample_values(key, tag, 2 * vidx + 1, t, s_words[1], s_val, lane);
+    __syncthreads();
+    if (warp == nw - 1) {  // s_suf[j] = sum_{j' >= j} e_{j'}; s_suf[t] = 0
+        const uint32_t per = (t + 31) / 32;
+        const uint32_t lo = min(t, lane * per), hi = min(t, lo + per);
+        uint32_t sum = 0;
+        for (uint32_t j = hi; j-- > lo;) sum = fadd(sum, s_val[j]);
+        uint32_t incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_down_sync(kFull, incl, o);
+            if (lane + o < 32) incl = fadd(incl, y);
+        }
+        uint32_t run = fsub(incl, sum);
+        for (uint32_t j = hi; j-- > lo;) {
+            run = fadd(run, s_val[j]);
+            s_suf[j] = run;
+        }
+        if (lane == 0) s_suf[t] = 0;
+    }
+    if (tid < t) {  // ascending support by rank (entries distinct; unused slots are larger than all)
+        const uint32_t v = s_list[tid];
+        uint32_t rk = 0;
+        for (uint32_t h = 0; h < t; h += 4) {
+            const uint4 a = *reinterpret_cast<const uint4 *>(s_list + h);
+            rk += (a.x < v) + (a.y < v) + (a.z < v) + (a.w < v);
+        }
+        s_supp[rk] = v;
+    }
+    __syncthreads();
+
+    if (!scan) {
+        // ---- u: 64 columns, the t rows over four groups
+        __shared__ uint32_t s_part[kTileUGroups - 1][kTileUCols];
+        const int grp = tid / kTileUCols, c = tid % kTileUCols;
+        const int k = (int)((blockIdx.x - nscan) % ucols) * kTileUCols + c;
+        const uint32_t per = (t + kTileUGroups - 1) / kTileUGroups;
+        const uint32_t j0 = min(t, (uint32_t)grp * per), j1 = min(t, j0 + per);
+        uint64_t acc = 0;
+        if (k < K) {
+            uint32_t j = j0;
+            for (; j + 8 <= j1; j += 8) {
+                uint32_t v[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) v[i] = __ldg(Qm + (size_t)s_supp[j + i] * K + k);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    acc += (uint64_t)s_val[j + i] * v[i];
+                    if (i & 1) acc = fred(acc);
+                }
+            }
+            uint32_t v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] = j + i < j1 ? __ldg(Qm + (size_t)s_supp[j + i] * K + k) : 0u;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                if (j + i < j1) acc += (uint64_t)s_val[j + i] * v[i];
+                if (i & 1) acc = fred(acc);
+            }
+        }
+        if (grp > 0) s_part[grp - 1][c] = (uint32_t)acc;
+        __syncthreads();
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (grp == 0 && k < K) {
+            uint32_t sum = (uint32_t)acc;
+#pragma unroll
+            for (int g = 0; g < kTileUGroups - 1; ++g) sum = fadd(sum, s_part[g][c]);
+            u[(size_t)vec * K + k] = sum;
+        }
+        return;
+    }
+
+    // ---- c over the tile, suffix sums inside it
+    uint32_t c[kScanItems];
+#pragma unroll
+    for (int i = 0; i < kScanItems; ++i) {
+        uint32_t lo = 0, hi = t;  // first support index >= idx[i]
+        while (lo < hi) {
+            const uint32_t mid = (lo + hi) >> 1;
+            if (s_supp[mid] < idx[i]) lo = mid + 1; else hi = mid;
+        }
+        c[i] = fmul(scale[i], s_suf[lo]);  // 0 past N (scale 0)
+    }
+    uint32_t run = 0;
+#pragma unroll
+    for (int i = kScanItems - 1; i >= 0; --i) {
+        run = fadd(run, c[i]);
+        c[i] = run;
+    }
+    uint32_t w1[kScanItems];  // requested here, used after the look-back
+#pragma unroll
+    for (int i = 0; i < kScanItems; ++i) w1[i] = base + i < N ? __ldg(v1m + base + i) : 0u;
+    uint32_t incl = run;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_down_sync(kFull, incl, o);
+        if (lane + o < 32) incl = fadd(incl, y);
+    }
+    if (lane == 0) s_wsum[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+        const uint32_t wv = lane < nw ? s_wsum[lane] : 0u;
+        uint32_t winc = wv;
+#pragma unroll
+        for (int o = 1; o < nw; o <<= 1) {
+            const uint32_t y = __shfl_down_sync(kFull, winc, o);
+            if (lane + o < 32) winc = fadd(winc, y);
+        }
+        __syncwarp();
+        if (lane < nw) s_wsum[lane] = fsub(winc, wv);
+        if (lane == 0) s_agg = winc;
+    }
+    // everything so far came from the key and the tables; what the kernels
+    // before this one may still use is written from here on
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    __syncthreads();
+    unsigned long long *st = status + (size_t)vec * ntiles;
+    if (warp == 0) {
+        // a failure-path test withholds one tile's word, so that the waits of
+        // the tiles before it run out (off: skip_tile >= ntiles)
+        if (lane == 0 && tile != skip_tile) st_relaxed_u64(st + tile, (1ull << 32) | s_agg);
+        uint32_t sum = 0;
+        for (uint32_t p = tile + 1 + lane; p < ntiles; p += 32) {
+            uint32_t spins = 0;
+            for (;;) {
+                const unsigned long long w = ld_relaxed_u64(st + p);
+                if (w >> 32) {
+                    sum = fadd(sum, (uint32_t)w);
+                    break;
+                }
+                if (++spins > spin_limit) {
+                    record_error(err, kErrScanTimeout);
+                    break;
+                }
+            }
+        }
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) sum = fadd(sum, __shfl_xor_sync(kFull, sum, o));
+        if (lane == 0) s_prefix = sum;
+    }
+    if (sparse_out && tile == 0) {
+        uint32_t *so = sparse_out + (size_t)vec * 2 * t;
+        for (uint32_t j = tid; j < t; j += kScanThreads) {
+            so[j] = s_supp[j];
+            so[t + j] = s_val[j];
+        }
+    }
+    __syncthreads();
+    const uint32_t add = fadd(fadd(fsub(incl, run), s_wsum[warp]), s_prefix);
+    uint32_t *Fv = F + (size_t)vec * N;
+    uint32_t f[kScanItems];
+#pragma unroll
+    for (int i = 0; i < kScanItems; ++i) f[i] = fmul_mont(fadd(c[i], add), w1[i]);
+    if (base + kScanItems <= N && N % 4 == 0) {
+#pragma unroll
+        for (int h = 0; h < kScanItems; h += 4)
+            *reinterpret_cast<uint4 *>(Fv + base + h) = make_uint4(f[h], f[h + 1], f[h + 2], f[h + 3]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < kScanItems; ++i)
+            if (base + i < N) Fv[base + i] = f[i];
+    }
+}
+
 // out_j = addend_j + sum_{c<r} F[pi1^-1(r j + c)]  ((R Pi1 F)_j, plus x_j).
+// The table is read before griddepcontrol.wait.  status[0 .. nclear) is set to
+// zero (the words k_syndrome_tiles used).
 __global__ void __launch_bounds__(256) k_syndrome_gather(const uint32_t *__restrict__ pi1inv,
                                                         uint32_t n, uint32_t r,
-                                                        const uint32_t *__restrict__ F, uint32_t N,
-                                                        const uint32_t *addend, uint32_t *out) {
+                                                        const uint32_t *F, uint32_t N,
+                                                        const uint32_t *addend, uint32_t *out,
+                                                        unsigned long long *status, uint32_t nclear) {
     const uint32_t vec = blockIdx.y;
     const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const uint32_t *p = pi1inv + (size_t)j * r;
+    uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
+    if (r == 8 && j < n) {
+        a = __ldg(reinterpret_cast<const uint4 *>(p));
+        b = __ldg(reinterpret_cast<const uint4 *>(p + 4));
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const uint32_t gid = (blockIdx.y * gridDim.x + blockIdx.x) * 256u + threadIdx.x;
+    for (uint32_t i = gid; i < nclear; i += gridDim.x * gridDim.y * 256u) status[i] = 0ull;
     if (j >= n) return;
     const uint32_t *Fv = F + (size_t)vec * N;
-    const uint32_t *p = pi1inv + (size_t)j * r;
-    uint32_t s = 0;
+    const size_t o = (size_t)vec * n + j;
+    uint32_t s = addend ? addend[o] : 0u;
     if (r == 8) {
-        const uint4 a = __ldg(reinterpret_cast<const uint4 *>(p));
-        const uint4 b = __ldg(reinterpret_cast<const uint4 *>(p + 4));
-        s = fadd(fadd(fadd(Fv[a.x], Fv[a.y]), fadd(Fv[a.z], Fv[a.w])),
-                 fadd(fadd(Fv[b.x], Fv[b.y]), fadd(Fv[b.z], Fv[b.w])));
+        s = fadd(s, fadd(fadd(fadd(Fv[a.x], Fv[a.y]), fadd(Fv[a.z], Fv[a.w])),
+                         fadd(fadd(Fv[b.x], Fv[b.y]), fadd(Fv[b.z], Fv[b.w]))));
     } else {
         for (uint32_t c = 0; c < r; ++c) s = fadd(s, Fv[p[c]]);
     }
-    const size_t o = (size_t)vec * n + j;
-    out[o] = addend ? fadd(addend[o], s) : s;
+    out[o] = s;
 }
 
 // -----------------------------------------------------------------------------
-// Fused syndrome: x' = G e for a freshly sampled sparse e, in one kernel per
-// vector, with the length-N intermediate held in shared memory: one CTA of
-// 1024 threads when it fits, else a thread-block cluster whose CTAs each hold
-// a slice (CTA `rank` owns positions [rank*slice, (rank+1)*slice)) and read
-// each other's through DSMEM.  Steps (App. B, syndrome direction):
-//   sample e (warp 0: support; warp 1: values; every CTA of a cluster draws
-//     the same keystream, rank 0 writes the state), the ascending support
-//     read off the sampling bitmap by a block-wide scan;
-//   c_i = v2[pi2^-1(i)] * (A e)_{pi2^-1(i)}, the step function (A e)_k found
-//     through a bucket index over the sorted support;
-//   d = A c: a block suffix scan plus the aggregates of later CTAs;
-//   F_i = v1_i * d_i;  out_j = addend_j + sum_{c<r} F[pi1^-1(r j + c)].
-// No global scratch and no look-back.
+// Fused syndrome: x' = G e for a freshly sampled sparse e, one CTA of 1024
+// threads per vector with the length-N intermediate in its shared memory
+// (codes of up to about 45 K positions).  Steps (App. B, syndrome direction):
+//   sample e (warp 0: support; warp 1: values), the ascending support read
+//     off the sampling bitmap by a block-wide scan;
+//   c_{pi2(k)} = v2_k (A e)_k, the step function (A e)_k found through a
+//     bucket index over the sorted support;
+//   d = A c: a block suffix scan;
+//   out_j = addend_j + sum_{c<r} v1 d at pi1^-1(r j + c).
+// No global scratch and no look-back.  (Spreading a vector over a cluster of
+// 2 to 8 CTAs, for longer codes and for small batches, took 21 to 77 us where
+// k_syndrome_tiles takes 7 to 11.)
 // -----------------------------------------------------------------------------
 constexpr int kFusedThreads = 1024;
 constexpr int kFusedBuckets = 512;   // index over the sorted support
-constexpr int kFusedBatch = 16;      // loads in flight per thread
-constexpr int kFusedBatch1 = 8;      // the same in the single-CTA scatter
+constexpr int kFusedBatch1 = 8;      // loads in flight per thread
 
 __device__ __forceinline__ uint32_t fpad(uint32_t i) { return i + (i >> 5); }  // bank padding
-
-// floor(x / d) as (x * ceil(2^40 / d)) >> 40 (division by an invariant
-// integer through a rounded-up reciprocal, Granlund and Montgomery 1994).
-// Exact when x * d < 2^40: the product is x / d + x * eps / 2^40 with
-// 0 <= eps < 1, and x / 2^40 < 1 / d never reaches the next integer.
-__host__ __device__ __forceinline__ uint64_t div_magic(uint32_t d) { return ((1ull << 40) + d - 1) / d; }
-__device__ __forceinline__ uint32_t div_by(uint32_t x, uint64_t magic) {
-    return (uint32_t)(((uint64_t)x * magic) >> 40);
-}
 
 // Everything before this point reads only the key and the code tables; the
 // state st and the output are written after griddepcontrol.wait, so a launch
@@ -413,20 +685,15 @@ __device__ __forceinline__ void fused_publish(uint32_t *st, const uint32_t *supp
 
 __global__ void __launch_bounds__(kFusedThreads) k_syndrome_fused(
     pvmvmd_key key, uint32_t tag, uint64_t idx0, uint32_t N, uint32_t t, uint32_t slice,
-    const uint32_t *__restrict__ pi2inv, const uint32_t *__restrict__ v2p,
-    const uint32_t *__restrict__ v1, const uint32_t *__restrict__ pi1inv, uint32_t n, uint32_t r,
+    const uint32_t *__restrict__ pi1inv, uint32_t n, uint32_t r,
     uint32_t *__restrict__ sparse_out, const uint32_t *addend, uint32_t *out,
     const uint32_t *__restrict__ pi2, const uint32_t *__restrict__ v2m,
     const uint32_t *__restrict__ v1pm) {
-    cg::cluster_group cluster = cg::this_cluster();
     extern __shared__ uint32_t sm[];
     __shared__ uint32_t s_wsum[kFusedThreads / 32];
-    __shared__ uint32_t s_texcl[kFusedThreads];
     __shared__ uint32_t s_first[kFusedBuckets];
-    __shared__ uint32_t s_agg;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint32_t C = cluster.num_blocks(), rank = cluster.block_rank();
-    const uint32_t vec = blockIdx.y;
+    const uint32_t vec = blockIdx.x;
     const uint64_t idx = idx0 + vec;
     const uint32_t fwords = fpad(slice);
     uint32_t *F = sm;                 // padded slice (bitmap while sampling)
@@ -504,107 +771,11 @@ __global__ void __launch_bounds__(kFusedThreads) k_syndrome_fused(
         }
         if (lane == 0) suf[t] = 0;
     }
-    if (C == 1) {
-        // ---- the whole vector in this CTA: c_{pi2(k)} = v2_k (A e)_k,
-        // scattered into the slice.  Positions are interleaved over the
-        // threads (k = u * 1024 + tid), so the table loads are coalesced and
-        // kFusedBatch1 of them are in flight per thread; (A e)_k is found
-        // from a bucket index into the sorted support.
-        int bshift = 0;
-        while ((N >> bshift) > (uint32_t)kFusedBuckets - 1) ++bshift;
-        const uint32_t nbk = (N >> bshift) + 1;
-        for (uint32_t b = tid; b < nbk; b += kFusedThreads) {
-            const uint32_t start = b << bshift;
-            uint32_t lo = 0, hi = t;
-            while (lo < hi) {
-                const uint32_t mid = (lo + hi) >> 1;
-                if (supp[mid] < start) lo = mid + 1; else hi = mid;
-            }
-            s_first[b] = lo;
-        }
-        __syncthreads();
-        const uint32_t items = slice / kFusedThreads;
-        for (uint32_t i = N + tid; i < slice; i += kFusedThreads) F[fpad(i)] = 0u;  // padding
-        for (uint32_t u0 = 0; u0 < items; u0 += kFusedBatch1) {
-            uint32_t pk[kFusedBatch1], vk[kFusedBatch1];
-#pragma unroll
-            for (int u = 0; u < kFusedBatch1; ++u) {
-                const uint32_t k = (u0 + u) * kFusedThreads + tid;
-                const bool ok = u0 + u < items && k < N;
-                pk[u] = ok ? __ldg(pi2 + k) : 0u;
-                vk[u] = ok ? __ldg(v2m + k) : 0u;
-            }
-#pragma unroll
-            for (int u = 0; u < kFusedBatch1; ++u) {
-                const uint32_t k = (u0 + u) * kFusedThreads + tid;
-                if (u0 + u < items && k < N) {
-                    uint32_t j = s_first[k >> bshift];
-                    while (j < t && supp[j] < k) ++j;
-                    F[fpad(pk[u])] = fmul_mont(suf[j], vk[u]);
-                }
-            }
-        }
-        __syncthreads();
-        // d = A c: thread tid owns positions [tid*items, (tid+1)*items)
-        uint32_t run = 0;
-        for (uint32_t u = items; u-- > 0;) {
-            const uint32_t li = tid * items + u;
-            run = fadd(run, F[fpad(li)]);
-            F[fpad(li)] = run;
-        }
-        uint32_t incl = run;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_down_sync(kFull, incl, o);
-            if (lane + o < 32) incl = fadd(incl, y);
-        }
-        if (lane == 0) s_wsum[warp] = incl;
-        __syncthreads();
-        if (warp == 0) {
-            constexpr int nw = kFusedThreads / 32;
-            const uint32_t wv = lane < nw ? s_wsum[lane] : 0u;
-            uint32_t winc = wv;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_down_sync(kFull, winc, o);
-                if (lane + o < 32) winc = fadd(winc, y);
-            }
-            __syncwarp();
-            if (lane < nw) s_wsum[lane] = fsub(winc, wv);
-        }
-        __syncthreads();
-        const uint32_t add = fadd(fsub(incl, run), s_wsum[warp]);
-        for (uint32_t u = 0; u < items; ++u) {
-            const uint32_t li = tid * items + u;
-            F[fpad(li)] = fadd(F[fpad(li)], add);
-        }
-        __syncthreads();
-        fused_publish(sparse_out + (size_t)vec * 2 * t, supp, suf, t, tid);
-        // out_j = addend_j + sum_c v1[pi1^-1(r j + c)] d[pi1^-1(r j + c)]
-        for (uint32_t jo = tid; jo < n; jo += kFusedThreads) {
-            const uint32_t *p = pi1inv + (size_t)jo * r;
-            const uint32_t *w = v1pm + (size_t)jo * r;
-            uint32_t acc = 0;
-            if (r == 8) {
-                const uint4 a = __ldg(reinterpret_cast<const uint4 *>(p));
-                const uint4 b = __ldg(reinterpret_cast<const uint4 *>(p + 4));
-                const uint4 c = __ldg(reinterpret_cast<const uint4 *>(w));
-                const uint4 d = __ldg(reinterpret_cast<const uint4 *>(w + 4));
-                acc = fadd(fadd(fadd(fmul_mont(F[fpad(a.x)], c.x), fmul_mont(F[fpad(a.y)], c.y)),
-                                fadd(fmul_mont(F[fpad(a.z)], c.z), fmul_mont(F[fpad(a.w)], c.w))),
-                           fadd(fadd(fmul_mont(F[fpad(b.x)], d.x), fmul_mont(F[fpad(b.y)], d.y)),
-                                fadd(fmul_mont(F[fpad(b.z)], d.z), fmul_mont(F[fpad(b.w)], d.w))));
-            } else {
-                for (uint32_t cc = 0; cc < r; ++cc) acc = fadd(acc, fmul_mont(F[fpad(__ldg(p + cc))], __ldg(w + cc)));
-            }
-            const size_t o = (size_t)vec * n + jo;
-            out[o] = addend ? fadd(addend[o], acc) : acc;
-        }
-        return;
-    }
-
-    // bucket index: position k lies in bucket k >> bshift; s_first[b] is the
-    // first support index >= b << bshift
+    // ---- the whole vector in this CTA: c_{pi2(k)} = v2_k (A e)_k,
+    // scattered into the slice.  Positions are interleaved over the
+    // threads (k = u * 1024 + tid), so the table loads are coalesced and
+    // kFusedBatch1 of them are in flight per thread; (A e)_k is found
+    // from a bucket index into the sorted support.
     int bshift = 0;
     while ((N >> bshift) > (uint32_t)kFusedBuckets - 1) ++bshift;
     const uint32_t nbk = (N >> bshift) + 1;
@@ -618,31 +789,29 @@ __global__ void __launch_bounds__(kFusedThreads) k_syndrome_fused(
         s_first[b] = lo;
     }
     __syncthreads();
-
-    // ---- c over this CTA's slice (coalesced positions, loads batched)
-    const uint32_t base = rank * slice;
     const uint32_t items = slice / kFusedThreads;
-    const uint64_t items_magic = div_magic(items), slice_magic = div_magic(slice);
-    for (uint32_t u0 = 0; u0 < items; u0 += kFusedBatch) {
-        uint32_t kk[kFusedBatch], sc[kFusedBatch];
+    for (uint32_t i = N + tid; i < slice; i += kFusedThreads) F[fpad(i)] = 0u;  // padding
+    for (uint32_t u0 = 0; u0 < items; u0 += kFusedBatch1) {
+        uint32_t pk[kFusedBatch1], vk[kFusedBatch1];
 #pragma unroll
-        for (int u = 0; u < kFusedBatch; ++u) {
-            const uint32_t i = base + (u0 + u) * kFusedThreads + tid;
-            const bool ok = u0 + u < items && i < N;
-            kk[u] = ok ? __ldg(pi2inv + i) : 0u;
-            sc[u] = ok ? __ldg(v2p + i) : 0u;
+        for (int u = 0; u < kFusedBatch1; ++u) {
+            const uint32_t k = (u0 + u) * kFusedThreads + tid;
+            const bool ok = u0 + u < items && k < N;
+            pk[u] = ok ? __ldg(pi2 + k) : 0u;
+            vk[u] = ok ? __ldg(v2m + k) : 0u;
         }
 #pragma unroll
-        for (int u = 0; u < kFusedBatch; ++u) {
-            if (u0 + u < items) {
-                uint32_t j = s_first[kk[u] >> bshift];  // first support index >= kk[u]
-                while (j < t && supp[j] < kk[u]) ++j;
-                F[fpad((u0 + u) * kFusedThreads + tid)] = fmul(sc[u], suf[j]);
+        for (int u = 0; u < kFusedBatch1; ++u) {
+            const uint32_t k = (u0 + u) * kFusedThreads + tid;
+            if (u0 + u < items && k < N) {
+                uint32_t j = s_first[k >> bshift];
+                while (j < t && supp[j] < k) ++j;
+                F[fpad(pk[u])] = fmul_mont(suf[j], vk[u]);
             }
         }
     }
     __syncthreads();
-    // ---- suffix sums: thread tid owns [tid*items, (tid+1)*items)
+    // d = A c: thread tid owns positions [tid*items, (tid+1)*items)
     uint32_t run = 0;
     for (uint32_t u = items; u-- > 0;) {
         const uint32_t li = tid * items + u;
@@ -668,76 +837,35 @@ __global__ void __launch_bounds__(kFusedThreads) k_syndrome_fused(
         }
         __syncwarp();
         if (lane < nw) s_wsum[lane] = fsub(winc, wv);
-        if (lane == 0) s_agg = winc;
     }
     __syncthreads();
-    s_texcl[tid] = fadd(fsub(incl, run), s_wsum[warp]);
-    uint32_t after = 0;  // sum over the positions owned by later CTAs
-    if (C > 1) {
-        cluster.sync();
-        // every warp reads the later ranks' totals at once (one DSMEM load
-        // per lane) and sums them with shuffles
-        const uint32_t rr = rank + 1 + (uint32_t)lane;
-        after = rr < C ? *cluster.map_shared_rank(&s_agg, rr) : 0u;
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) after = fadd(after, __shfl_xor_sync(kFull, after, o));
-    } else {
-        __syncthreads();
+    const uint32_t add = fadd(fsub(incl, run), s_wsum[warp]);
+    for (uint32_t u = 0; u < items; ++u) {
+        const uint32_t li = tid * items + u;
+        F[fpad(li)] = fadd(F[fpad(li)], add);
     }
-    for (uint32_t u0 = 0; u0 < items; u0 += kFusedBatch) {
-        uint32_t sc[kFusedBatch];
-#pragma unroll
-        for (int u = 0; u < kFusedBatch; ++u) {
-            const uint32_t i = base + (u0 + u) * kFusedThreads + tid;
-            sc[u] = (u0 + u < items && i < N) ? __ldg(v1 + i) : 0u;
-        }
-#pragma unroll
-        for (int u = 0; u < kFusedBatch; ++u) {
-            if (u0 + u < items) {
-                const uint32_t li = (u0 + u) * kFusedThreads + tid;
-                const uint32_t d = fadd(F[fpad(li)], fadd(s_texcl[div_by(li, items_magic)], after));
-                F[fpad(li)] = fmul(sc[u], d);
-            }
-        }
-    }
-    if (C > 1) cluster.sync(); else __syncthreads();
-    if (rank == 0) fused_publish(sparse_out + (size_t)vec * 2 * t, supp, suf, t, tid);
-    else asm volatile("griddepcontrol.wait;" ::: "memory");
-
-    // ---- gather: out_j = addend_j + sum_c F[pi1^-1(r j + c)]
-    const uint32_t nsl = (n + C - 1) / C;
-    const uint32_t j0 = rank * nsl, j1 = min(n, j0 + nsl);
-    for (uint32_t j = j0 + tid; j < j1; j += kFusedThreads) {
-        const uint32_t *p = pi1inv + (size_t)j * r;
+    __syncthreads();
+    fused_publish(sparse_out + (size_t)vec * 2 * t, supp, suf, t, tid);
+    // out_j = addend_j + sum_c v1[pi1^-1(r j + c)] d[pi1^-1(r j + c)]
+    for (uint32_t jo = tid; jo < n; jo += kFusedThreads) {
+        const uint32_t *p = pi1inv + (size_t)jo * r;
+        const uint32_t *w = v1pm + (size_t)jo * r;
         uint32_t acc = 0;
         if (r == 8) {
             const uint4 a = __ldg(reinterpret_cast<const uint4 *>(p));
             const uint4 b = __ldg(reinterpret_cast<const uint4 *>(p + 4));
-            const uint32_t gi[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-            uint32_t v[8];
-            if (C == 1) {
-#pragma unroll
-                for (int c = 0; c < 8; ++c) v[c] = F[fpad(gi[c])];
-            } else {
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const uint32_t owner = div_by(gi[c], slice_magic);
-                    v[c] = cluster.map_shared_rank(F, owner)[fpad(gi[c] - owner * slice)];
-                }
-            }
-#pragma unroll
-            for (int c = 0; c < 8; ++c) acc = fadd(acc, v[c]);
+            const uint4 c = __ldg(reinterpret_cast<const uint4 *>(w));
+            const uint4 d = __ldg(reinterpret_cast<const uint4 *>(w + 4));
+            acc = fadd(fadd(fadd(fmul_mont(F[fpad(a.x)], c.x), fmul_mont(F[fpad(a.y)], c.y)),
+                            fadd(fmul_mont(F[fpad(a.z)], c.z), fmul_mont(F[fpad(a.w)], c.w))),
+                       fadd(fadd(fmul_mont(F[fpad(b.x)], d.x), fmul_mont(F[fpad(b.y)], d.y)),
+                            fadd(fmul_mont(F[fpad(b.z)], d.z), fmul_mont(F[fpad(b.w)], d.w))));
         } else {
-            for (uint32_t c = 0; c < r; ++c) {
-                const uint32_t gi = __ldg(p + c);
-                const uint32_t owner = div_by(gi, slice_magic), off = gi - owner * slice;
-                acc = fadd(acc, C == 1 ? F[fpad(off)] : cluster.map_shared_rank(F, owner)[fpad(off)]);
-            }
+            for (uint32_t cc = 0; cc < r; ++cc) acc = fadd(acc, fmul_mont(F[fpad(__ldg(p + cc))], __ldg(w + cc)));
         }
-        const size_t o = (size_t)vec * n + j;
+        const size_t o = (size_t)vec * n + jo;
         out[o] = addend ? fadd(addend[o], acc) : acc;
     }
-    if (C > 1) cluster.sync();  // peers may still read this CTA's F
 }
 
 // -----------------------------------------------------------------------------
@@ -1234,6 +1362,22 @@ __global__ void __launch_bounds__(kLaneCta, 4) k_lane_gather(const uint4 *__rest
 
 }  // namespace
 
+namespace {
+cudaError_t launch_pdl(const void *fn, dim3 grid, dim3 block, size_t smem, cudaStream_t s, void **args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute a[1];
+    a[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = a;
+    cfg.numAttrs = 1;
+    return counted_launch(cudaLaunchKernelExC(&cfg, fn, args));
+}
+}  // namespace
+
 // Bitmap of N bits plus 512 keystream words; covers N up to 8 * PVMVMD_MAX_K.
 constexpr size_t kSampleMaxSmem = 200 * 1024;
 
@@ -1267,11 +1411,56 @@ cudaError_t launch_syndrome_scan(const uint32_t *pi2inv, const uint32_t *v2p, co
 
 cudaError_t launch_syndrome_gather(const uint32_t *pi1inv, uint32_t n, uint32_t r,
                                    const uint32_t *F, uint32_t N, const uint32_t *addend,
-                                   uint32_t *out, uint32_t count, cudaStream_t s) {
+                                   uint32_t *out, uint32_t count, cudaStream_t s,
+                                   unsigned long long *status, uint32_t nclear) {
     if (count == 0 || n == 0) return cudaSuccess;
-    dim3 grid((n + 255) / 256, count);
-    k_syndrome_gather<<<grid, 256, 0, s>>>(pi1inv, n, r, F, N, addend, out); note_launch();
-    return cudaGetLastError();
+    void *args[] = {&pi1inv, &n, &r, &F, &N, &addend, &out, &status, &nclear};
+    return launch_pdl((const void *)k_syndrome_gather, dim3((n + 255) / 256, count), dim3(256), 0, s, args);
+}
+
+bool syndrome_tiles_eligible(uint32_t t) { return t <= kTileMaxT; }
+
+cudaError_t launch_syndrome_tiles(const pvmvmd_key &key, uint32_t tag, uint64_t idx0, uint32_t N, uint32_t t,
+                                  uint32_t count, const uint32_t *pi2inv, const uint32_t *v2p,
+                                  const uint32_t *v1m, const uint32_t *pi1inv, uint32_t n, uint32_t r,
+                                  uint32_t *sparse_out, uint32_t *F, unsigned long long *status, uint32_t *err,
+                                  const uint32_t *addend, uint32_t *out, cudaStream_t s, bool pdl,
+                                  const uint32_t *Qm, int K, uint32_t *u) {
+    if (count == 0) return cudaSuccess;
+    constexpr uint32_t kMost = 65535;  // the gather's grid
+    if (count > kMost) {
+        const cudaError_t e =
+            launch_syndrome_tiles(key, tag, idx0, N, t, kMost, pi2inv, v2p, v1m, pi1inv, n, r, sparse_out, F, status,
+                                  err, addend, out, s, pdl, Qm, K, u);
+        if (e != cudaSuccess) return e;
+        return launch_syndrome_tiles(key, tag, idx0 + kMost, N, t, count - kMost, pi2inv, v2p, v1m, pi1inv, n, r,
+                                     sparse_out ? sparse_out + (size_t)kMost * 2 * t : nullptr, F, status, err,
+                                     addend ? addend + (size_t)kMost * n : nullptr, out + (size_t)kMost * n, s, pdl,
+                                     Qm, K, u ? u + (size_t)kMost * K : nullptr);
+    }
+    const uint32_t ntiles = scan_tiles(N);
+    const uint32_t ucols = u ? (uint32_t)(K + kTileUCols - 1) / kTileUCols : 0u;
+    const uint64_t ctas = (uint64_t)count * (ntiles + ucols);
+    if (!syndrome_tiles_eligible(t) || ctas > 0x7fffffffu) return cudaErrorInvalidValue;
+    const DebugWait dbg = debug_wait();
+    const bool inject = dbg.site == PVMVMD_DEBUG_WAIT_SCAN;
+    uint32_t skip = inject ? dbg.index : 0xFFFFFFFFu, limit = inject ? (uint32_t)dbg.limit : kSpinLimit;
+    const uint32_t grid = (uint32_t)ctas;
+    cudaError_t e;
+    if (pdl) {
+        void *args[] = {(void *)&key, &tag, &idx0, &N, &t, &count, &pi2inv, &v2p, &v1m, &sparse_out, &F, &status,
+                        &err, &skip, &limit, &Qm, &K, (void *)&ucols, &u};
+        e = launch_pdl((const void *)k_syndrome_tiles, dim3(grid), dim3(kScanThreads), 0, s, args);
+    } else {
+        k_syndrome_tiles<<<grid, kScanThreads, 0, s>>>(key, tag, idx0, N, t, count, pi2inv, v2p, v1m, sparse_out, F,
+                                                       status, err, skip, limit, Qm, K, ucols, u);
+        e = counted_launch(cudaGetLastError());
+    }
+    if (e != cudaSuccess) return e;
+    e = launch_syndrome_gather(pi1inv, n, r, F, N, addend, out, count, s, status, count * ntiles);
+    // the words must be zero for the next call also where the gather did not start
+    if (e != cudaSuccess) (void)cudaMemsetAsync(status, 0, (size_t)count * ntiles * sizeof(unsigned long long), s);
+    return e;
 }
 
 size_t encode_scan_status_words(uint32_t N, uint32_t L) {
@@ -1312,126 +1501,32 @@ cudaError_t launch_transpose_i8(const int8_t *in, int R, int C, int8_t *out, cud
 
 
 namespace {
-uint32_t fused_slice(uint32_t N, int C) {
-    return (uint32_t)(((N + C - 1) / C + kFusedThreads - 1) / kFusedThreads) * kFusedThreads;
-}
+uint32_t fused_slice(uint32_t N) { return (N + kFusedThreads - 1) / kFusedThreads * kFusedThreads; }
 size_t fused_smem(uint32_t slice, uint32_t t) {
     return ((size_t)slice + slice / 32 + 3 * (size_t)t + 1 + 1024) * sizeof(uint32_t);
 }
 constexpr size_t kFusedMaxSmem = 180 * 1024;
-
 }  // namespace
 
-// Cluster size and slice for the fused syndrome; false if N is too long for
-// one cluster of at most 8 CTAs.
-bool syndrome_fused_plan(uint32_t N, uint32_t t, int *C_out, uint32_t *slice_out, size_t *smem_out) {
-    // one CTA when the padded intermediate fits, else the smallest cluster
-    for (int C = 1; C <= 8; C *= 2) {
-        const uint32_t slice = fused_slice(N, C);
-        const size_t smem = fused_smem(slice, t);
-        if (smem <= kFusedMaxSmem) {
-            *C_out = C;
-            *slice_out = slice;
-            *smem_out = smem;
-            return true;
-        }
-    }
-    return false;
-}
-
-// The cluster size one launch of `count` vectors uses: the smallest that
-// holds the intermediate, and for a batch that leaves most SMs idle (at most
-// a quarter busy) doubled while count * C * spread CTAs still fit the SMs
-// and every CTA keeps at least one position per thread, up to 8 CTAs.  A
-// small batch then spreads each vector's serial work over a few SMs instead
-// of one; larger batches keep the cheaper per-position work of the smallest
-// cluster.  The callers' spread (launch_syndrome_fused) was measured: 4 for
-// encodes (8 vectors per call: Qwen3-4B block 0.265 -> 0.227 ms per step
-// against spread 1; 2 gave 0.275, 8 gave 0.255); for the ell = 2 shared
-// challenges 16 when the batch is large (a cluster of at most 2 CTAs at
-// N_y = 32768, taking few SMs from the decrypt beside it: batch-1 workload of
-// 100 vectors 0.3256 -> 0.3220 ms per step against spread 4), else 4 (the
-// challenges are then the decode's critical path: Qwen3-4B block, 8
-// vectors, 0.227 against 0.235 ms; one token with its 448 single-vector
-// encodes and decodes, client part 9.7 against 10.2 ms).  (Up to 16 CTAs, a
-// non-portable size, made one decode call alone slightly faster, 0.3228
-// against 0.3242 ms per batch-1 step, but a layer's decodes side by side
-// fit only seven 16-CTA clusters at once: 8B layer, 64 vectors, 0.528
-// against 0.506 ms per step; Qwen3-4B block, 8 vectors, 0.324 against
-// 0.266 ms.)
-constexpr int kFusedClusterMax = 8;
-static void syndrome_fused_launch_plan(uint32_t N, uint32_t t, uint32_t count, int *C, uint32_t *slice,
-                                       size_t *smem, int spread) {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if ((uint64_t)count * (uint64_t)*C * 4 > (uint64_t)sms) return;
-    const int cmax = kFusedClusterMax;
-    while (*C < cmax && (uint64_t)count * (uint64_t)(2 * *C) * (uint64_t)spread <= (uint64_t)sms &&
-           (uint64_t)(2 * *C) * kFusedThreads <= (uint64_t)N) {
-        *C *= 2;
-        *slice = fused_slice(N, *C);
-        *smem = fused_smem(*slice, t);
-    }
+bool syndrome_fused_fits(uint32_t N, uint32_t t) {
+    return N <= (1u << 20) && fused_smem(fused_slice(N), t) <= kFusedMaxSmem;
 }
 
 cudaError_t launch_syndrome_fused(const pvmvmd_key &key, uint32_t tag, uint64_t idx0, uint32_t N,
-                                  uint32_t t, uint32_t count, const uint32_t *pi2inv,
-                                  const uint32_t *v2p, const uint32_t *v1, const uint32_t *pi1inv,
+                                  uint32_t t, uint32_t count, const uint32_t *pi1inv,
                                   const uint32_t *pi2, const uint32_t *v2m, const uint32_t *v1pm,
                                   uint32_t n, uint32_t r, uint32_t *sparse_out,
-                                  const uint32_t *addend, uint32_t *out, cudaStream_t s, bool pdl,
-                                  int spread) {
+                                  const uint32_t *addend, uint32_t *out, cudaStream_t s) {
     if (count == 0) return cudaSuccess;
-    int C = 0;
-    uint32_t slice = 0;
-    size_t smem = 0;
-    if (!syndrome_fused_plan(N, t, &C, &slice, &smem)) return cudaErrorNotSupported;
+    if (!syndrome_fused_fits(N, t)) return cudaErrorNotSupported;
     const cudaError_t attr = func_attr((const void *)k_syndrome_fused, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)kFusedMaxSmem);
     if (attr != cudaSuccess) return attr;
-    syndrome_fused_launch_plan(N, t, count < 65535 ? count : 65535, &C, &slice, &smem, spread < 1 ? 1 : spread);
-    for (uint32_t c0 = 0; c0 < count; c0 += 65535) {
-        const uint32_t nb = count - c0 < 65535 ? count - c0 : 65535;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(C, nb, 1);
-        cfg.blockDim = dim3(kFusedThreads, 1, 1);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = s;
-        cudaLaunchAttribute attr1[2];
-        attr1[0].id = cudaLaunchAttributeClusterDimension;
-        attr1[0].val.clusterDim.x = C;
-        attr1[0].val.clusterDim.y = 1;
-        attr1[0].val.clusterDim.z = 1;
-        attr1[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr1[1].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr1;
-        cfg.numAttrs = pdl ? 2 : 1;
-        cudaError_t e = counted_launch(cudaLaunchKernelEx(&cfg, k_syndrome_fused, key, tag, idx0 + c0, N, t, slice,
-                                           pi2inv, v2p, v1, pi1inv, n, r,
-                                           sparse_out + (size_t)c0 * 2 * t,
-                                           addend ? addend + (size_t)c0 * n : nullptr,
-                                           out + (size_t)c0 * n, pi2, v2m, v1pm));
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    uint32_t slice = fused_slice(N);
+    void *args[] = {(void *)&key, &tag, &idx0, &N, &t, &slice, &pi1inv, &n, &r, &sparse_out, &addend, &out,
+                    &pi2, &v2m, &v1pm};
+    return launch_pdl((const void *)k_syndrome_fused, dim3(count), dim3(kFusedThreads), fused_smem(slice, t), s, args);
 }
-
-namespace {
-cudaError_t launch_pdl(const void *fn, dim3 grid, dim3 block, size_t smem, cudaStream_t s, void **args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute a[1];
-    a[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    a[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = a;
-    cfg.numAttrs = 1;
-    return counted_launch(cudaLaunchKernelExC(&cfg, fn, args));
-}
-}  // namespace
 
 size_t lane_state_words(uint32_t t, uint32_t L) {
     return (size_t)L * (t + 1) + (size_t)L * kLaneBuckets / 2;

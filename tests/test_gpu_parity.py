@@ -120,6 +120,24 @@ def test_small_parameters_round_trip(pv, wl):
                      oracle_kw=dict(t_x=5, t_y=3, ell=3, rate=3))
 
 
+@pytest.mark.parametrize("m,K,B,kw", [
+    (300, 1025, 3, {}),                             # N_x = 8200: a last tile of 8 positions
+    (683, 4101, 2, dict(rate=3)),                   # N_x = 12303, N_y = 2049: unaligned rows, a tile of 1
+    (16, 1100, 30, {}), (16, 1100, 31, {}),         # 150 and 155 tiles, on both sides of one per SM
+    (40, 1030, 2, dict(t_x=256, t_y=256)),          # the longest support the tiles sort
+    (40, 1030, 2, dict(t_x=257, t_y=257)),          # one more: the paths without tiles
+    (40, 1030, 2, dict(t_x=1, t_y=1, ell=3)),       # one support; an odd number of challenges
+])
+def test_tiled_syndrome_round_trip(pv, wl, m, K, B, kw):
+    """The tiled syndrome (masks of a few vectors, and every challenge) at the
+    edges of its tiles and of the rule that picks it."""
+    W = wl.weights_uniform(m, K, m + 3 * K)
+    x = wl.int8_vectors(B, K, m + B)
+    okw = dict(rate=kw.get("rate", 8), ell=kw.get("ell", 2))
+    okw.update({k: kw[k] for k in ("t_x", "t_y") if k in kw})
+    _full_round_trip(pv, W, x, seeds=(m + B, K, B), params=_params(pv, **kw), oracle_kw=okw)
+
+
 def test_encode_chunking_matches(pv, wl):
     """Encoding in chunks of 3 vectors (scratch_batch) gives the same result."""
     W = wl.weights_uniform(64, 96, 1)
