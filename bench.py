@@ -690,7 +690,7 @@ def run_ours(args):
             "data": "synthetic", "config": arm_config(args),
             "hbm_gbs_gemv": achieved,
             "phases_ms": {"encode": enc_ms, "server_100_gemv": srv_ms, "decode_verify": dec_ms},
-            "roofline": {"bound": "hbm", "kernel": "k_gemv_multi (batch-1 field GEMV, 100 requests per launch)",
+            "roofline": {"bound": "hbm", "kernel": "k_gemv_ring (batch-1 field GEMV, 100 requests per launch)",
                          "achieved": achieved,
                          "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": achieved / peaks["hbm_gbs"],
                          "peak_kind": f"{peak_kind} hbm_gbs", "traffic": traffic,
@@ -1348,7 +1348,7 @@ def measure_token(args, device, rank=0):
                                            "down's dependence on q/k/v and gate/up"},
             "one_call_per_token": {"ms": relaxed["one"], "hbm_gbs": nbytes / (relaxed["one"] / 1e3) / 1e9,
                                    "note": "all 224 products in one call (a replay of a finished token)"}},
-        "roofline": {"bound": "hbm", "kernel": "k_gemv_multi (1-3 requests per launch, 128 dependent launches)",
+        "roofline": {"bound": "hbm", "kernel": "k_gemv_ring (1-3 requests per launch, 128 dependent launches)",
                      "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                      "frac": achieved / peaks["hbm_gbs"], "peak_kind": f"{kind} hbm_gbs", "traffic": None,
                      "algorithmic_bytes_per_token": nbytes},

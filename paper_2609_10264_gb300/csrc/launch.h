@@ -128,7 +128,7 @@ struct MvmJob {
     int accumulate;  // y += M x_hat instead of y = M x_hat
 };
 constexpr int kMultiMaxJobs = 256;  // jobs per grouped launch
-constexpr int kMultiMaxK = 16384;   // K per grouped launch (longer K is segmented)
+constexpr int kMultiMaxK = 16384;   // K per grouped launch (two chunks per thread; longer K is segmented)
 
 // Y_hat = M X_hat for a few vectors (2 <= B <= 16): one pass over M per group
 // of four vectors.  Needs K % 16 == 0 and 16-byte aligned W and X_hat.

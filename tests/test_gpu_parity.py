@@ -576,6 +576,31 @@ def test_qwen3_4b_block_8_tokens(pv, wl, name):
     _batched_pipeline(pv, W, 8, seed=600 + len(name))
 
 
+@pytest.mark.parametrize("shapes", [
+    [(1, 16)], [(3, 512)], [(700, 528)],             # one warp per row; just past it
+    [(33, 8192)], [(40, 8208)], [(65, 16384)],       # one chunk per thread, two, the longest
+    [(5, 16400)],                                    # a second segment of one chunk
+    [(5000, 32), (300, 4096), (2, 8192)],            # jobs that share CTAs
+    [(2048, 4096), (2048, 4096), (2048, 4096)],      # jobs with CTAs of their own
+    [(1000 + i, 16 * (1 + i)) for i in range(9)],    # more jobs than the small parameter block holds
+])
+def test_gemv_ring_edges(pv, shapes):
+    """The grouped batch-1 kernel where its split of a row over threads, of the
+    rows over CTAs and of K over launches changes, with extreme digits."""
+    rng = np.random.default_rng(len(shapes) + shapes[0][0])
+    jobs, exp = [], []
+    for m, K in shapes:
+        W = rng.integers(-128, 128, size=(m, K), dtype=np.int8)
+        x = rng.integers(0, Q, size=K).astype(np.uint32)
+        W[0] = -128
+        x[: K // 2] = (Q + int(-128 * (1 + 2**8 + 2**16))) % Q
+        exp.append(oracle.server_mvm(W, x))
+        jobs.append((to_dev(W), to_dev(x), to_dev(np.zeros(m, np.uint32))))
+    pv.pvmvmd_server_mvm_multi(jobs)
+    for (m, K), (_, _, y), e in zip(shapes, jobs, exp):
+        assert_equal_report(pv.as_u32(y), e, f"{m}x{K}")
+
+
 def test_server_mvm_multi_mixed_jobs(pv, wl):
     """Grouped batch-1 products over mixed shapes, including K beyond one
     segment (20000), a K that is not a multiple of 16 (1001) and tiny matrices; equal to the
