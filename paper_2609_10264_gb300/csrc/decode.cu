@@ -157,10 +157,10 @@ __device__ __forceinline__ void pe_cols(const uint32_t *__restrict__ PT, int m, 
 // segments) and splits the t_x rows over kDecGroups = 2 row groups, so each
 // thread streams about t_x / 2 row segments (rounds of 8 loads in flight)
 // and the grid holds many short CTAs whatever m and B are; or 256 columns
-// over 4 row groups when that fills the last wave of resident CTAs better.
-// The groups' partial sums meet in shared memory.  (256 columns everywhere,
-// or 1024 columns and 1 group, were 6 and 13 % slower at m = K = 8192,
-// B = 256.)
+// over 4 row groups when that fills the last wave of resident CTAs better;
+// or 64 columns over 16 when the whole grid is resident at once.  The groups'
+// partial sums meet in shared memory.  (256 columns everywhere, or 1024
+// columns and 1 group, were 6 and 13 % slower at m = K = 8192, B = 256.)
 // In boost mode (Sec. 7.2) P e_x,b was prepared ahead: Y_b = y_hat_b - mask_b.
 // The grid runs vectors fastest (blockIdx.x = b, blockIdx.y = column block),
 // so the CTAs in flight share a few column blocks and a row of P^T drawn by
@@ -444,16 +444,21 @@ cudaError_t launch_decrypt(const uint32_t *PT, int m, const uint32_t *st, uint32
     // 2.63; decrypt 47 -> 41 us, step 0.3221 -> 0.3202 ms).  Where both
     // fill alike the wider CTAs stay (70B-class shapes, 256 vectors: 256
     // columns everywhere took 2.221 -> 2.272 ms per step).
+    // Where 64-column CTAs, with the rows over 16 groups, fit the GPU at once
+    // they are used: a thread then waits for about t_x / 128 rounds of eight
+    // rows instead of t_x / 16 (256 x 256, one vector: 15.7 -> 5 us cold).
     const int slots = decrypt_slots();
     auto fill = [&](int cols) {
         const double waves = (double)B * (double)((m + cols - 1) / cols) / slots;
         return waves / std::ceil(waves);
     };
-    const bool narrow = slots > 0 && fill(256) > fill(512) + 0.1;
-    const int cols = narrow ? 256 : 512;
+    const bool once = slots > 0 && (double)B * (double)((m + 63) / 64) <= slots;
+    const int cols = once ? 64 : slots > 0 && fill(256) > fill(512) + 0.1 ? 256 : 512;
     if ((m + cols - 1) / cols > 65535) return cudaErrorInvalidValue;
     const dim3 grid((unsigned)B, (m + cols - 1) / cols);
-    if (narrow)
+    if (cols == 64)
+        k_decrypt<false, 16><<<grid, kDecThreads, smem, s>>>(PT, m, st, t_x, Nx, Yhat, Y, nullptr, vec);
+    else if (cols == 256)
         k_decrypt<false, 4><<<grid, kDecThreads, smem, s>>>(PT, m, st, t_x, Nx, Yhat, Y, nullptr, vec);
     else
         k_decrypt<false, 2><<<grid, kDecThreads, smem, s>>>(PT, m, st, t_x, Nx, Yhat, Y, nullptr, vec);
