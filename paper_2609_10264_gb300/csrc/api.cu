@@ -543,15 +543,45 @@ int pvmvmd_weights_split_i16(const int16_t *W_dev, int m, int K, int8_t *Whi_dev
     return PVMVMD_OK;
 }
 
+namespace pv {
+namespace {
+// The path of a product of 2 <= B <= 16 vectors: one pass over M per four
+// vectors with dp4a, unless the problem is large enough for the tensor-core
+// product with 16-vector tiles to win (measured: 14336 x 4096 with 8 vectors
+// 41.0 against 27.1 us, with 4 vectors 23.8 against 26.0 us; 4096 x 2560 with
+// 8 vectors 12.1 against 12.9 us).
+bool small_batch_wins(const void *W, int m, int K, const uint32_t *Xhat, int B) {
+    const bool tensor_small = B >= 8 && (double)m * K * B >= 128.0 * 1024 * 1024;
+    return B > 1 && B <= kSmallBatchMax && !tensor_small && K % 16 == 0 &&
+           ((reinterpret_cast<uintptr_t>(W) | reinterpret_cast<uintptr_t>(Xhat)) & 15u) == 0;
+}
+}  // namespace
+}  // namespace pv
+
+// Both planes in one launch where that needs no more scratch than a product:
+// of the small-batch kernel, which combines them itself (4096 x 2560, 8
+// vectors: 28.8 -> 19.8 us a call), or as two jobs of the batch-1 kernel (one
+// vector: 28.6 -> 17.5 us).
 int pvmvmd_server_mvm_i16(const int8_t *Whi_dev, const int8_t *Wlo_dev, int m, int K, const uint32_t *Xhat_dev,
                           int B, uint32_t *Yhat_dev, uint32_t *Ytmp_dev, void *stream) {
     using namespace pv;
-    if (!Whi_dev || !Wlo_dev || !Ytmp_dev) return PVMVMD_E_ARG;
-    int st = pvmvmd_server_mvm(Whi_dev, m, K, Xhat_dev, B, Yhat_dev, stream);
-    if (st) return st;
-    st = pvmvmd_server_mvm(Wlo_dev, m, K, Xhat_dev, B, Ytmp_dev, stream);
-    if (st) return st;
-    PV_CUDA(launch_combine_256(Yhat_dev, Ytmp_dev, (size_t)B * m, static_cast<cudaStream_t>(stream)));
+    if (!Whi_dev || !Wlo_dev || !Ytmp_dev || !Xhat_dev || !Yhat_dev) return PVMVMD_E_ARG;
+    if (m < 1 || K < 1 || K > PVMVMD_MAX_K || B < 1) return PVMVMD_E_SHAPE;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    if (small_batch_wins(Whi_dev, m, K, Xhat_dev, B) && small_batch_wins(Wlo_dev, m, K, Xhat_dev, B)) {
+        PV_CUDA(launch_gemv_small_batch(Wlo_dev, m, K, Xhat_dev, B, Yhat_dev, s, Whi_dev));
+        return PVMVMD_OK;
+    }
+    if (B == 1) {
+        const pvmvmd_mvm_job jobs[2] = {{Whi_dev, Xhat_dev, Yhat_dev, m, K}, {Wlo_dev, Xhat_dev, Ytmp_dev, m, K}};
+        const int st = pvmvmd_server_mvm_multi(jobs, 2, stream);
+        if (st) return st;
+    } else {
+        int st = pvmvmd_server_mvm(Whi_dev, m, K, Xhat_dev, B, Yhat_dev, stream);
+        if (!st) st = pvmvmd_server_mvm(Wlo_dev, m, K, Xhat_dev, B, Ytmp_dev, stream);
+        if (st) return st;
+    }
+    PV_CUDA(launch_combine_256(Yhat_dev, Ytmp_dev, (size_t)B * m, s));
     return PVMVMD_OK;
 }
 
@@ -674,14 +704,7 @@ int pvmvmd_server_mvm(const int8_t *W_dev, int m, int K, const uint32_t *Xhat_de
         PV_CUDA(launch_gemv(W_dev, m, K, Xhat_dev, Yhat_dev, err, s));
         return PVMVMD_OK;
     }
-    // a few vectors: one pass over M per four vectors with dp4a, unless the
-    // problem is large enough for the tensor-core product with 16-vector
-    // tiles to win (measured: 14336 x 4096 with 8 vectors 41.0 against
-    // 27.1 us, with 4 vectors 23.8 against 26.0 us; 4096 x 2560 with 8
-    // vectors 12.1 against 12.9 us)
-    const bool tensor_small = B >= 8 && (double)m * K * B >= 128.0 * 1024 * 1024;
-    if (B <= kSmallBatchMax && !tensor_small && K % 16 == 0 &&
-        ((reinterpret_cast<uintptr_t>(W_dev) | reinterpret_cast<uintptr_t>(Xhat_dev)) & 15u) == 0) {
+    if (small_batch_wins(W_dev, m, K, Xhat_dev, B)) {
         PV_CUDA(launch_gemv_small_batch(W_dev, m, K, Xhat_dev, B, Yhat_dev, s));
         return PVMVMD_OK;
     }
@@ -729,7 +752,7 @@ int pvmvmd_server_mvm_grouped(const pvmvmd_mvm_batch_job *jobs, int count, void 
     std::vector<MvmJob> single;
     for (int i = 0; i < count; ++i) {
         const pvmvmd_mvm_batch_job &j = jobs[i];
-        if (j.B > 1 && batched_grouped_eligible(j.W_dev, j.m, j.K, j.B)) {
+        if (j.B > 1 && batched_grouped_eligible(j.W_dev, j.Xhat_dev, j.m, j.K, j.B)) {
             grouped.push_back(BatchJob{j.W_dev, j.Xhat_dev, j.Yhat_dev, j.m, j.K, j.B});
             continue;
         }

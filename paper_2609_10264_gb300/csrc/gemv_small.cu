@@ -62,7 +62,7 @@ constexpr int kNbStride = kNbMaxK / 16;  // 16-byte chunks per plane row
 constexpr int kNbSmem = 4 * kNbVec * kNbMaxK;
 
 struct NbJob {
-    const int8_t *W;
+    const int8_t *W, *Whi;   // Whi: the high plane of a pair launch, M = 256 Whi + W
     const uint32_t *planes;  // row (p, v) of the segment at planes + (p * kNbVec + v) * ldp
     uint32_t *y;             // vector v at y + v * ldy
     int m, K, nb, accumulate;
@@ -105,12 +105,15 @@ __global__ void __launch_bounds__(256) k_nb_planes(const uint32_t *__restrict__ 
     for (int d = 0; d < 4; ++d) dst[((size_t)d * kNbVec + v) * per_vec + q4] = p[d];
 }
 
-template <int ROWS, int UNROLL>
+// kPair: the two register rows of a warp are one row of the two int8 planes of
+// a 16-bit matrix (M = 256 Whi + W), combined before the store.
+template <int ROWS, int UNROLL, bool kPair>
 __global__ void __launch_bounds__(kMultiThreads, 2) k_gemv_nb(const __grid_constant__ NbArgs args) {
     extern __shared__ uint4 s_planes[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int V = ROWS * 4 * kNbVec;
     static_assert(V == 32, "ROWS * 4 planes * 4 vectors must be one entry per lane");
+    constexpr int kStep = kPair ? 1 : ROWS;  // matrix rows per warp and turn
     const long long total = args.base[args.count];
     const long long lo = total * blockIdx.x / gridDim.x;
     const long long hi = total * (blockIdx.x + 1) / gridDim.x;
@@ -129,7 +132,7 @@ __global__ void __launch_bounds__(kMultiThreads, 2) k_gemv_nb(const __grid_const
         const int row_a = lo > b0 ? (int)((lo - b0 + K - 1) / K) : 0;
         const int row_b = (int)min((long long)m, (hi - b0 + K - 1) / K);
         if (row_a >= row_b) continue;
-        const int ngroups = (row_b - row_a + ROWS - 1) / ROWS;
+        const int ngroups = (row_b - row_a + kStep - 1) / kStep;
 
         uint4 wbuf[UNROLL][ROWS];
         auto issue = [&](int grp, int c) {
@@ -137,9 +140,10 @@ __global__ void __launch_bounds__(kMultiThreads, 2) k_gemv_nb(const __grid_const
             for (int u = 0; u < UNROLL; ++u)
 #pragma unroll
                 for (int r = 0; r < ROWS; ++r) {
-                    const int cc = c + 32 * u, row = row_a + grp * ROWS + r;
+                    const int cc = c + 32 * u, row = row_a + grp * kStep + (kPair ? 0 : r);
+                    const int8_t *M = kPair && r == 1 ? job.Whi : job.W;
                     wbuf[u][r] = (cc < nchunks && row < row_b)
-                                     ? ldg_stream(job.W + (size_t)row * job.ldw + (size_t)cc * 16)
+                                     ? ldg_stream(M + (size_t)row * job.ldw + (size_t)cc * 16)
                                      : make_uint4(0u, 0u, 0u, 0u);
                 }
         };
@@ -217,16 +221,14 @@ __global__ void __launch_bounds__(kMultiThreads, 2) k_gemv_nb(const __grid_const
             const int a1 = __shfl_down_sync(kFull, tot, 1);
             const int a2 = __shfl_down_sync(kFull, tot, 2);
             const int a3 = __shfl_down_sync(kFull, tot, 3);
-            if ((lane & 3) == 0) {
-                const int v = (lane >> 2) % kNbVec, r = (lane >> 2) / kNbVec;
-                const int row = row_a + g * ROWS + r;
-                if (row < row_b && v < job.nb) {
-                    const int64_t sum = (int64_t)tot + ((int64_t)a1 << 8) + ((int64_t)a2 << 16) +
-                                        ((int64_t)a3 << 24);
-                    const uint32_t part = fred_signed(sum);
-                    uint32_t *yp = job.y + (size_t)v * job.ldy + row;
-                    *yp = job.accumulate ? fadd(*yp, part) : part;
-                }
+            const int v = (lane >> 2) % kNbVec, r = (lane >> 2) / kNbVec;
+            const int64_t sum = (int64_t)tot + ((int64_t)a1 << 8) + ((int64_t)a2 << 16) + ((int64_t)a3 << 24);
+            uint32_t part = fred_signed(sum);  // of the lanes that hold digit 0
+            if (kPair) part = fadd(part, fmul(__shfl_down_sync(kFull, part, 16), 256u));
+            const int row = row_a + g * kStep + (kPair ? 0 : r);
+            if ((lane & 3) == 0 && (!kPair || r == 0) && row < row_b && v < job.nb) {
+                uint32_t *yp = job.y + (size_t)v * job.ldy + row;
+                *yp = job.accumulate ? fadd(*yp, part) : part;
             }
         }
     }
@@ -235,6 +237,7 @@ __global__ void __launch_bounds__(kMultiThreads, 2) k_gemv_nb(const __grid_const
     if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+template <bool kPair>
 cudaError_t run_gemv_nb(const NbJob *jobs, int count, cudaStream_t s) {
     static NbArgs args;  // host staging of the kernel parameters (copied at launch)
     static std::mutex mu;
@@ -249,7 +252,7 @@ cudaError_t run_gemv_nb(const NbJob *jobs, int count, cudaStream_t s) {
     }
     if (rows == 0) return cudaSuccess;
     const cudaError_t attr =
-        func_attr((const void *)k_gemv_nb<2, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNbSmem);
+        func_attr((const void *)k_gemv_nb<2, 2, kPair>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNbSmem);
     if (attr != cudaSuccess) return attr;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
@@ -266,13 +269,13 @@ cudaError_t run_gemv_nb(const NbJob *jobs, int count, cudaStream_t s) {
     attrs[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attrs;
     cfg.numAttrs = 1;
-    return counted_launch(cudaLaunchKernelEx(&cfg, k_gemv_nb<2, 2>, args));
+    return counted_launch(cudaLaunchKernelEx(&cfg, k_gemv_nb<2, 2, kPair>, args));
 }
 
 }  // namespace
 
 cudaError_t launch_gemv_small_batch(const int8_t *W, int m, int K, const uint32_t *Xhat, int B,
-                                    uint32_t *Yhat, cudaStream_t s) {
+                                    uint32_t *Yhat, cudaStream_t s, const int8_t *Whi) {
     if (m <= 0 || K <= 0 || B <= 0) return cudaSuccess;
     // digit planes of all vectors once: [job][plane][vector][K] bytes
     const int Bp = (B + kNbVec - 1) / kNbVec * kNbVec;
@@ -303,6 +306,7 @@ cudaError_t launch_gemv_small_batch(const int8_t *W, int m, int K, const uint32_
         for (int b0 = 0; b0 < B; b0 += kNbVec) {
             NbJob j;
             j.W = W + k0;
+            j.Whi = Whi ? Whi + k0 : nullptr;
             j.planes = planes + (size_t)(b0 / kNbVec) * job_words + (size_t)k0 / 4;
             j.y = Yhat + (size_t)b0 * m;
             j.m = m;
@@ -316,7 +320,7 @@ cudaError_t launch_gemv_small_batch(const int8_t *W, int m, int K, const uint32_
         }
         for (size_t a = 0; a < jobs.size(); a += kNbMaxJobs) {
             const int n = (int)std::min(jobs.size() - a, (size_t)kNbMaxJobs);
-            e = run_gemv_nb(jobs.data() + a, n, s);
+            e = Whi ? run_gemv_nb<true>(jobs.data() + a, n, s) : run_gemv_nb<false>(jobs.data() + a, n, s);
             if (e != cudaSuccess) return e;
         }
     }

@@ -131,9 +131,10 @@ constexpr int kMultiMaxJobs = 256;  // jobs per grouped launch
 constexpr int kMultiMaxK = 16384;   // K per grouped launch (two chunks per thread; longer K is segmented)
 
 // Y_hat = M X_hat for a few vectors (2 <= B <= 16): one pass over M per group
-// of four vectors.  Needs K % 16 == 0 and 16-byte aligned W and X_hat.
+// of four vectors.  Needs K % 16 == 0 and 16-byte aligned W and X_hat.  With
+// Whi (aligned as W) M is the 16-bit matrix 256 Whi + W.
 cudaError_t launch_gemv_small_batch(const int8_t *W, int m, int K, const uint32_t *Xhat, int B,
-                                    uint32_t *Yhat, cudaStream_t s);
+                                    uint32_t *Yhat, cudaStream_t s, const int8_t *Whi = nullptr);
 
 // Eligible for the grouped kernel: K % 16 == 0 and 16-byte aligned rows.
 bool multi_eligible(const MvmJob &j);
@@ -149,14 +150,14 @@ cudaError_t launch_batched(const int8_t *W, int m, int K, const uint32_t *Xhat, 
                            uint32_t *Yhat, uint32_t *err, cudaStream_t s);
 
 // Several independent batched products in one persistent tensor-core launch
-// (jobs with K % 16 == 0 and 16-byte aligned W; outputs must not overlap).
+// (jobs with K % 16 == 0 and 16-byte aligned W and X_hat; outputs must not overlap).
 struct BatchJob {
     const int8_t *W;
     const uint32_t *Xhat;
     uint32_t *Yhat;
     int m, K, B;
 };
-bool batched_grouped_eligible(const int8_t *W, int m, int K, int B);
+bool batched_grouped_eligible(const int8_t *W, const uint32_t *Xhat, int m, int K, int B);
 cudaError_t launch_batched_grouped(const BatchJob *jobs, int count, uint32_t *err, cudaStream_t s);
 
 // Grow-only scratch of at least `need` bytes for `purpose` on the current

@@ -1219,8 +1219,9 @@ double plan_makespan(const std::vector<PlanJob> &jobs, int C) {
 
 }  // namespace
 
-bool batched_grouped_eligible(const int8_t *W, int m, int K, int B) {
-    return m >= 1 && B >= 1 && K >= 1 && K % 16 == 0 && (reinterpret_cast<uintptr_t>(W) & 15u) == 0;
+bool batched_grouped_eligible(const int8_t *W, const uint32_t *Xhat, int m, int K, int B) {
+    return m >= 1 && B >= 1 && K >= 1 && K % 16 == 0 &&
+           ((reinterpret_cast<uintptr_t>(W) | reinterpret_cast<uintptr_t>(Xhat)) & 15u) == 0;
 }
 
 template <int V>
@@ -1373,7 +1374,7 @@ cudaError_t launch_batched_grouped(const BatchJob *jobs, int count, uint32_t *er
 cudaError_t launch_batched(const int8_t *W, int m, int K, const uint32_t *Xhat, int B,
                            uint32_t *Yhat, uint32_t *err, cudaStream_t s) {
     if (m <= 0 || K <= 0 || B <= 0) return cudaSuccess;
-    if (batched_grouped_eligible(W, m, K, B)) {
+    if (batched_grouped_eligible(W, Xhat, m, K, B)) {
         const BatchJob job{W, Xhat, Yhat, m, K, B};
         return launch_batched_grouped(&job, 1, err, s);
     }

@@ -306,6 +306,38 @@ def test_sixteen_bit_weights_round_trip(pv, wl, B):
     ctx.destroy()
 
 
+@pytest.mark.parametrize("m,K,B", [(33, 16, 2), (300, 6144 + 96, 5), (1025, 528, 16), (1, 512, 1), (40, 16400, 1)])
+def test_sixteen_bit_product_one_launch(pv, m, K, B):
+    """The 16-bit product where one launch takes both planes: few vectors (one
+    chunk of columns, two segments of K, the largest batch, an odd row) and
+    one vector (one launch, and two segments)."""
+    rng = np.random.default_rng(m + K + B)
+    W = rng.integers(-32768, 32640, size=(m, K)).astype(np.int16)
+    W[0] = -32768
+    hi, lo = pv.pvmvmd_weights_split_i16(to_dev(W))
+    X = rng.integers(0, Q, size=(B, K)).astype(np.uint32)
+    X[0] = (Q + int(-128 * (1 + 2**8 + 2**16))) % Q
+    got = pv.as_u32(pv.pvmvmd_server_mvm_i16(hi, lo, to_dev(X)))
+    exp = (oracle.server_mvm_batch(hi.cpu().numpy(), X).astype(np.uint64) * 256
+           + oracle.server_mvm_batch(lo.cpu().numpy(), X)) % Q
+    assert_equal_report(got, exp.astype(np.uint32), "y_hat")
+
+
+@pytest.mark.parametrize("B", [1, 5, 40])
+def test_server_mvm_unaligned_vectors(pv, B):
+    """Vectors off a 16-byte boundary with rows on one take the general path."""
+    rng = np.random.default_rng(B)
+    m, K = 300, 1024
+    W = rng.integers(-128, 128, size=(m, K), dtype=np.int8)
+    X = rng.integers(0, Q, size=(B, K)).astype(np.uint32)
+    Xd = to_dev(np.concatenate([np.zeros(1, np.uint32), X.reshape(-1)]))[1:].view(B, K)
+    exp = oracle.server_mvm_batch(W, X)
+    assert_equal_report(pv.as_u32(pv.pvmvmd_server_mvm(to_dev(W), Xd)), exp, "single call")
+    Y = to_dev(np.zeros((B, m), np.uint32))
+    pv.pvmvmd_server_mvm_grouped([(to_dev(W), Xd, Y)])
+    assert_equal_report(pv.as_u32(Y), exp, "grouped call")
+
+
 def test_server_mvm_extremes(pv):
     """Extreme weights and field values: -128, 127, x = 0, 1, (q-1)/2, (q+1)/2, q-1."""
     rng = np.random.default_rng(1)
