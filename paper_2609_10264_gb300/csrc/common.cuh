@@ -100,6 +100,25 @@ __device__ __forceinline__ void limb_split(uint32_t x, int &d0, int &d1, int &d2
     d3 = (c - d2) >> 8;
 }
 
+// 16 bytes at p, of any alignment, from the aligned words that hold them: five
+// 4-byte loads and four funnel shifts.  A word is read only if it holds a byte
+// of [lo, hi) (the matrix); other bytes of the result are zero or those of
+// neighbours, which the caller multiplies by zero digits.
+__device__ __forceinline__ uint4 load16_any(const int8_t *p, const int8_t *lo, const int8_t *hi) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(p) & ~(uintptr_t)3;
+    const uint32_t sh = 8u * (uint32_t)(reinterpret_cast<uintptr_t>(p) & 3);
+    uint32_t w[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        const uintptr_t q = a + 4 * i;
+        // the fifth word is needed only when p is not aligned
+        const bool in = q < reinterpret_cast<uintptr_t>(hi) && q + 4 > reinterpret_cast<uintptr_t>(lo) && (i < 4 || sh);
+        w[i] = in ? __ldg(reinterpret_cast<const uint32_t *>(q)) : 0u;
+    }
+    return make_uint4(__funnelshift_r(w[0], w[1], sh), __funnelshift_r(w[1], w[2], sh),
+                      __funnelshift_r(w[2], w[3], sh), __funnelshift_r(w[3], w[4], sh));
+}
+
 // ---------------------------------------------------------------- ChaCha20
 // RFC 8439 Sec. 2.3 block function; state words 4..11 key, 12 counter,
 // 13..15 nonce.

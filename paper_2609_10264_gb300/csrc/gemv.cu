@@ -8,7 +8,7 @@
 // int64 and reduced mod q once per row.
 //  * k_gemv_ring   K a multiple of 16 and 16-byte aligned rows: a list of
 //                  independent products in one launch.
-//  * k_gemv        any K and alignment, byte loads, one product.
+//  * k_gemv        any K and alignment, words and funnel shifts, one product.
 #include <algorithm>
 #include <vector>
 
@@ -22,18 +22,6 @@ constexpr int kGemvThreads = 512;
 // Digit planes of a K segment live in shared memory (4 bytes per column); a
 // longer K is done in segments whose mod-q partial results are added.
 constexpr int kGemvMaxK = 48 * 1024;
-
-// 16 bytes of row `row` starting at column 16*chunk, zero-filled past K.
-__device__ __forceinline__ uint4 load_chunk(const int8_t *__restrict__ W, size_t ldw, size_t row,
-                                            int K, int chunk) {
-    const int8_t *p = W + row * ldw + (size_t)chunk * 16;
-    uint32_t w[4] = {0u, 0u, 0u, 0u};
-    const int c0 = chunk * 16;
-#pragma unroll
-    for (int b = 0; b < 16; ++b)
-        if (c0 + b < K) w[b >> 2] |= (uint32_t)(uint8_t)__ldg(p + b) << (8 * (b & 3));
-    return make_uint4(w[0], w[1], w[2], w[3]);
-}
 
 // Sum of v[index] over the 32 lanes, where index = lane / (32 / V): after the
 // call every lane holds the total of the entry its lane number selects.
@@ -70,7 +58,9 @@ __global__ void __launch_bounds__(kGemvThreads, 1)
     const int gstride = gridDim.x * nwarps;
     int g = warp * gridDim.x + blockIdx.x;
 
-    // Issue the first batch of M loads before building the digit planes.
+    // Issue the first batch of M loads before building the digit planes (bytes
+    // past K meet zero digits).
+    const int8_t *W_end = W + (size_t)(m - 1) * ldw + K;
     uint4 wbuf[UNROLL][ROWS];
     auto issue = [&](int grp, int c) {
 #pragma unroll
@@ -78,8 +68,9 @@ __global__ void __launch_bounds__(kGemvThreads, 1)
 #pragma unroll
             for (int r = 0; r < ROWS; ++r) {
                 const int cc = c + 32 * u, row = grp * ROWS + r;
-                wbuf[u][r] = (cc < nchunks && row < m) ? load_chunk(W, ldw, (size_t)row, K, cc)
-                                                       : make_uint4(0u, 0u, 0u, 0u);
+                wbuf[u][r] = (cc < nchunks && row < m)
+                                 ? load16_any(W + (size_t)row * ldw + (size_t)cc * 16, W, W_end)
+                                 : make_uint4(0u, 0u, 0u, 0u);
             }
     };
     if (g < ngroups) issue(g, lane);

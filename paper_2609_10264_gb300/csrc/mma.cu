@@ -422,21 +422,27 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
             }
         } else {
-            // rows of any length and alignment: plain byte loads
-            for (int i = grp; i < nblk; i += 2) {
-                const int s = i % kStages;
-                const uint32_t ph = (uint32_t)(i / kStages) & 1u;
+            // rows of any length and alignment, from the words that hold them,
+            // a block ahead (bytes past K meet zero digits)
+            const int8_t *W_end = W + (size_t)m * K;
+            auto fetch = [&](int i, uint4 (&v)[4]) {
                 const int k0 = (kb0 + i) * kBK + 16 * qk;
-                uint4 v[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int grow = m0 + r0 + 32 * j;
-                    uint32_t w[4] = {0u, 0u, 0u, 0u};
-                    if (grow < m)
-                        for (int e = 0; e < 16 && k0 + e < K; ++e)
-                            w[e >> 2] |= (uint32_t)(uint8_t)W[(size_t)grow * K + k0 + e] << (8 * (e & 3));
-                    v[j] = make_uint4(w[0], w[1], w[2], w[3]);
+                    v[j] = i < nblk && grow < m && k0 < K ? load16_any(W + (size_t)grow * K + k0, W, W_end)
+                                                          : make_uint4(0u, 0u, 0u, 0u);
                 }
+            };
+            uint4 next[4];
+            fetch(grp, next);
+            for (int i = grp; i < nblk; i += 2) {
+                const int s = i % kStages;
+                const uint32_t ph = (uint32_t)(i / kStages) & 1u;
+                uint4 v[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) v[j] = next[j];
+                fetch(i + 2, next);
                 if (!mbar_wait_warp(&empty_bar[s], ph ^ 1u, err, wait_ns)) break;
                 convert_store(smem + s * kStageBytes, v);
                 fence_async_smem();

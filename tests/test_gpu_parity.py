@@ -323,6 +323,23 @@ def test_sixteen_bit_product_one_launch(pv, m, K, B):
     assert_equal_report(got, exp.astype(np.uint32), "y_hat")
 
 
+@pytest.mark.parametrize("B", [1, 3, 40])
+@pytest.mark.parametrize("K", [1, 15, 63, 65, 514, 1001])
+def test_server_mvm_unaligned_rows(pv, K, B):
+    """Rows of every alignment: K that is not a multiple of 16 (rows start at
+    any byte), and a matrix and vectors that start off a 16-byte boundary."""
+    rng = np.random.default_rng(K + B)
+    m = 131
+    W = rng.integers(-128, 128, size=(m, K), dtype=np.int8)
+    X = rng.integers(0, Q, size=(B, K)).astype(np.uint32)
+    exp = oracle.server_mvm_batch(W, X)
+    assert_equal_report(pv.as_u32(pv.pvmvmd_server_mvm(to_dev(W), to_dev(X))), exp, "aligned start")
+    for off in (1, 2, 7):
+        Wd = to_dev(np.concatenate([np.zeros(off, np.int8), W.reshape(-1)]))[off:].view(m, K)
+        Xd = to_dev(np.concatenate([np.zeros(off, np.uint32), X.reshape(-1)]))[off:].view(B, K)
+        assert_equal_report(pv.as_u32(pv.pvmvmd_server_mvm(Wd, Xd)), exp, f"offset {off}")
+
+
 @pytest.mark.parametrize("B", [1, 5, 40])
 def test_server_mvm_unaligned_vectors(pv, B):
     """Vectors off a 16-byte boundary with rows on one take the general path."""
