@@ -6,8 +6,10 @@
 #include <cstdlib>
 #include <cstring>
 #include <atomic>
+#include <initializer_list>
 #include <mutex>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "common.cuh"
@@ -235,28 +237,36 @@ cudaError_t ctx_alloc(Ctx *c, T **p, size_t count) {
     return e;
 }
 
+// Samples the context's two codes (numbers which[k], lengths N[k]) on the device,
+// their tables in one allocation.  Enqueued on s: the scratch is freed by the
+// caller once the stream has drained.
 template <typename Ctx>
-int upload_code(Ctx *c, CodeDev &d, const pvmvmd_key &key, int which, uint32_t N, cudaStream_t s) {
-    std::vector<uint32_t> pi1(N), pi2(N), v1(N), v2(N), pi1inv(N), pi2inv(N), v2p(N), v2m(N), v1pm(N), v1m(N);
-    sample_code_host(key, which, N, pi1.data(), pi2.data(), v1.data(), v2.data());
-    for (uint32_t j = 0; j < N; ++j) {
-        pi1inv[pi1[j]] = j;
-        pi2inv[pi2[j]] = j;
+int sample_codes(Ctx *c, const pvmvmd_key &key, CodeDev *const code[2], const int which[2], const uint32_t N[2],
+                 uint32_t **scratch, cudaStream_t s) {
+    size_t words = 0, swords = 0;
+    auto up = [](size_t n) { return (n + 63) & ~(size_t)63; };  // tables start on 256-byte boundaries
+    for (int k = 0; k < 2; ++k) {
+        words += 10 * up(N[k]);
+        swords += up(code_draw_scratch_words(N[k]));
     }
-    for (uint32_t i = 0; i < N; ++i) {
-        v2p[i] = v2[pi2inv[i]];
-        v2m[i] = to_mont(v2[i]);
-        v1pm[i] = to_mont(v1[pi1inv[i]]);
-        v1m[i] = to_mont(v1[i]);
+    uint32_t *t = nullptr;
+    PV_CUDA(ctx_alloc(c, &t, words));
+    PV_CUDA(dev_alloc(scratch, swords));
+    CodeDraws draws[2];
+    uint32_t *sc[2], *at = *scratch;
+    for (int k = 0; k < 2; ++k) {
+        CodeDev &d = *code[k];
+        for (uint32_t **p : {&d.pi1, &d.pi2, &d.v1, &d.v2, &d.pi1inv, &d.pi2inv, &d.v2p, &d.v2m, &d.v1pm, &d.v1m}) {
+            *p = t;
+            t += up(N[k]);
+        }
+        // code `which` reads tags kTagCodeX + 4 which + 0 .. 3
+        draws[k] = CodeDraws{N[k], kTagCodeX + 4u * (uint32_t)which[k], d.pi1, d.pi2, d.v1, d.v2, d.pi1inv, d.pi2inv,
+                             d.v2p, d.v2m, d.v1pm, d.v1m, {}};
+        sc[k] = at;
+        at += up(code_draw_scratch_words(N[k]));
     }
-    uint32_t **dst[10] = {&d.pi1, &d.pi2, &d.v1, &d.v2, &d.pi1inv, &d.pi2inv, &d.v2p, &d.v2m, &d.v1pm, &d.v1m};
-    const std::vector<uint32_t> *src[10] = {&pi1, &pi2, &v1, &v2, &pi1inv, &pi2inv, &v2p, &v2m, &v1pm, &v1m};
-    for (int i = 0; i < 10; ++i) {
-        PV_CUDA(ctx_alloc(c, dst[i], N));
-        PV_CUDA(cudaMemcpyAsync(*dst[i], src[i]->data(), (size_t)N * 4, cudaMemcpyHostToDevice, s));
-    }
-    // the host vectors are released on return; wait for the copies
-    PV_CUDA(cudaStreamSynchronize(s));
+    PV_CUDA(launch_code_draws(key, draws, 2, sc, s));
     return PVMVMD_OK;
 }
 
@@ -278,35 +288,50 @@ int encode_lanes_into(const CodeDev &d, uint32_t n, uint32_t r, const void *X, b
     return e == cudaSuccess ? PVMVMD_OK : PVMVMD_E_CUDA;
 }
 
-// Y (N x L lanes, row stride ldy) = G^T applied to the L lanes of X (n x L,
-// row stride ldx; row i holds message entry i of every lane; int8 or
-// uint32), in lane chunks with scratch allocated here (preprocessing only).
-int encode_lanes(const CodeDev &d, uint32_t n, uint32_t r, const void *X, bool x_is_i8, size_t ldx,
-                 uint32_t L, uint32_t *Y, size_t ldy, uint32_t *err, cudaStream_t s) {
-    const uint32_t N = n * r;
-    size_t lc = ((size_t)1 << 28) / N;  // lanes per chunk: about 1 GiB of scratch
-    lc = (lc / 256) * 256;
-    if (lc < 256) lc = 256;
-    if (lc > L) lc = L;
+// Scratch of encode_lanes, allocated once for all the encodings of a
+// preprocessing (a 512 MiB cudaMalloc and cudaFree take 0.44 ms).
+struct LaneScratch {
     uint32_t *S = nullptr, *ticket = nullptr;
     unsigned long long *status = nullptr;
-    const size_t sw = encode_scan_status_words(N, (uint32_t)lc);
-    int status_code = PVMVMD_OK;
-    if (dev_alloc(&S, (size_t)N * lc) != cudaSuccess || dev_alloc(&status, sw) != cudaSuccess ||
-        dev_alloc(&ticket, 1) != cudaSuccess) {
-        status_code = PVMVMD_E_NOMEM;
+    ~LaneScratch() {
+        cudaFree(S);
+        cudaFree(status);
+        cudaFree(ticket);
     }
-    for (uint32_t l0 = 0; status_code == PVMVMD_OK && l0 < L; l0 += (uint32_t)lc) {
+    static size_t lanes(uint32_t N, uint32_t L) {  // lanes per chunk: about 1 GiB of S
+        size_t lc = ((size_t)1 << 28) / N / 256 * 256;
+        if (lc < 256) lc = 256;
+        return lc < L ? lc : L;
+    }
+    // for encodings of length N[k] over L[k] lanes
+    int alloc(std::initializer_list<std::pair<uint32_t, uint32_t>> uses) {
+        size_t s = 0, w = 0;
+        for (const auto &u : uses) {
+            const size_t lc = lanes(u.first, u.second);
+            s = std::max(s, (size_t)u.first * lc);
+            w = std::max(w, encode_scan_status_words(u.first, (uint32_t)lc));
+        }
+        return dev_alloc(&S, s) == cudaSuccess && dev_alloc(&status, w) == cudaSuccess &&
+                       dev_alloc(&ticket, 1) == cudaSuccess
+                   ? PVMVMD_OK
+                   : PVMVMD_E_NOMEM;
+    }
+};
+
+// Y (N x L lanes, row stride ldy) = G^T applied to the L lanes of X (n x L,
+// row stride ldx; row i holds message entry i of every lane; int8 or
+// uint32), in lane chunks (preprocessing only).
+int encode_lanes(const CodeDev &d, uint32_t n, uint32_t r, const void *X, bool x_is_i8, size_t ldx,
+                 uint32_t L, uint32_t *Y, size_t ldy, const LaneScratch &sc, uint32_t *err, cudaStream_t s) {
+    const size_t lc = LaneScratch::lanes(n * r, L);
+    for (uint32_t l0 = 0; l0 < L; l0 += (uint32_t)lc) {
         const uint32_t nl = (uint32_t)((L - l0) < lc ? (L - l0) : lc);
         const void *Xl = x_is_i8 ? static_cast<const void *>(static_cast<const int8_t *>(X) + l0)
                                  : static_cast<const void *>(static_cast<const uint32_t *>(X) + l0);
-        status_code = encode_lanes_into(d, n, r, Xl, x_is_i8, ldx, nl, Y + l0, ldy, S, status, ticket, err, s);
+        const int st = encode_lanes_into(d, n, r, Xl, x_is_i8, ldx, nl, Y + l0, ldy, sc.S, sc.status, sc.ticket, err, s);
+        if (st != PVMVMD_OK) return st;
     }
-    if (cudaStreamSynchronize(s) != cudaSuccess) status_code = PVMVMD_E_CUDA;
-    cudaFree(S);
-    cudaFree(status);
-    cudaFree(ticket);
-    return status_code;
+    return PVMVMD_OK;
 }
 
 int read_and_clear_error() {
@@ -458,21 +483,61 @@ int preprocess_impl(const void *W_dev, bool w16, int m, int K, const pvmvmd_para
     c->sb = p.scratch_batch;
 
     auto fail = [&](int code) {
+        cudaStreamSynchronize(s);  // what is enqueued may still use the context
+        (void)cudaGetLastError();
         pvmvmd_destroy(c);
         return code;
     };
-    if ((st = upload_code(c, c->gx, *key, 0, c->Nx, s))) return fail(st);
-    if ((st = upload_code(c, c->gy, *key, 1, c->Ny, s))) return fail(st);
-    if (ctx_alloc(c, &c->PT, (size_t)c->Nx * m) != cudaSuccess ||
-        ctx_alloc(c, &c->Q, (size_t)c->Ny * K) != cudaSuccess ||
-        ctx_alloc(c, &c->F, (size_t)((c->sb + 3) & ~3) * c->Nx) != cudaSuccess ||  // lanes padded to 4
-        ctx_alloc(c, &c->Fy, (size_t)c->ell * c->Ny) != cudaSuccess ||
-        ctx_alloc(c, &c->chal, (size_t)c->ell * 2 * c->t_y) != cudaSuccess ||
-        ctx_alloc(c, &c->g, (size_t)c->ell * m) != cudaSuccess ||
-        ctx_alloc(c, &c->u, (size_t)c->ell * K) != cudaSuccess ||
-        ctx_alloc(c, &c->status, scan_status_words(c->Nx, c->sb)) != cudaSuccess ||
-        ctx_alloc(c, &c->status_y, scan_status_words(c->Ny, c->ell)) != cudaSuccess)
+    // temporaries: freed on every way out, once the stream has drained (the
+    // context's own memory too, where the call fails)
+    struct Temp {
+        uint32_t *draws = nullptr, *M32 = nullptr, *MT32 = nullptr;
+        int8_t *MT = nullptr;
+        LaneScratch lanes;
+        cudaStream_t s;
+        ~Temp() {
+            cudaStreamSynchronize(s);
+            cudaFree(draws);
+            cudaFree(M32);
+            cudaFree(MT32);
+            cudaFree(MT);
+        }
+    } tmp;
+    tmp.s = s;
+    CodeDev *const codes[2] = {&c->gx, &c->gy};
+    const int which[2] = {0, 1};
+    const uint32_t lengths[2] = {(uint32_t)c->Nx, (uint32_t)c->Ny};
+    if ((st = sample_codes(c, *key, codes, which, lengths, &tmp.draws, s))) return fail(st);
+    // the small arrays in one allocation
+    const size_t f = (size_t)((c->sb + 3) & ~3) * c->Nx;  // lanes padded to 4
+    const bool lanes = c->sb >= kLaneMinBatch;
+    uint32_t *small = nullptr;
+    size_t words = 0;
+    auto take = [&](size_t n) {  // on 256-byte boundaries
+        const size_t at = words;
+        words += (n + 63) & ~(size_t)63;
+        return at;
+    };
+    const size_t oF = take(f), oFy = take((size_t)c->ell * c->Ny), ochal = take((size_t)c->ell * 2 * c->t_y),
+                 og = take((size_t)c->ell * m), ou = take((size_t)c->ell * K),
+                 ostatus = take(2 * scan_status_words(c->Nx, c->sb)),
+                 ostatus_y = take(2 * scan_status_words(c->Ny, c->ell)),
+                 oS = take(lanes ? lane_state_words(c->t_x, c->sb) : 0),
+                 olaux = take(lanes ? lane_aux_words(c->Nx, c->sb) : 0);
+    if (ctx_alloc(c, &small, words) != cudaSuccess || ctx_alloc(c, &c->PT, (size_t)c->Nx * m) != cudaSuccess ||
+        ctx_alloc(c, &c->Q, (size_t)c->Ny * K) != cudaSuccess)
         return fail(PVMVMD_E_NOMEM);
+    c->F = small + oF;
+    c->Fy = small + oFy;
+    c->chal = small + ochal;
+    c->g = small + og;
+    c->u = small + ou;
+    c->status = reinterpret_cast<unsigned long long *>(small + ostatus);
+    c->status_y = reinterpret_cast<unsigned long long *>(small + ostatus_y);
+    if (lanes) {
+        c->S = small + oS;
+        c->laux = small + olaux;
+    }
     // the tiled syndrome finds its status words zero and leaves them zero
     if (cudaMemsetAsync(c->status, 0, scan_status_words(c->Nx, c->sb) * sizeof(unsigned long long), s) != cudaSuccess ||
         cudaMemsetAsync(c->status_y, 0, scan_status_words(c->Ny, c->ell) * sizeof(unsigned long long), s) !=
@@ -487,47 +552,29 @@ int preprocess_impl(const void *W_dev, bool w16, int m, int K, const pvmvmd_para
         cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->join, cudaEventDisableTiming) != cudaSuccess)
         return fail(PVMVMD_E_CUDA);
-    if (c->sb >= kLaneMinBatch &&
-        (ctx_alloc(c, &c->S, lane_state_words(c->t_x, c->sb)) != cudaSuccess ||
-         ctx_alloc(c, &c->laux, lane_aux_words(c->Nx, c->sb)) != cudaSuccess))
-        return fail(PVMVMD_E_NOMEM);
-
+    if ((st = tmp.lanes.alloc({{(uint32_t)c->Nx, (uint32_t)m}, {(uint32_t)c->Ny, (uint32_t)K}}))) return fail(st);
+    const void *rows = W_dev, *cols = nullptr;  // M by rows (lanes: its columns) and transposed
     if (w16) {
         // 16-bit M: lift it to F_q, then encode as uint32 lanes
-        uint32_t *M32 = nullptr, *MT32 = nullptr;
-        if (dev_alloc(&M32, (size_t)m * K) != cudaSuccess || dev_alloc(&MT32, (size_t)m * K) != cudaSuccess) {
-            cudaFree(M32);
+        if (dev_alloc(&tmp.M32, (size_t)m * K) != cudaSuccess || dev_alloc(&tmp.MT32, (size_t)m * K) != cudaSuccess)
             return fail(PVMVMD_E_NOMEM);
-        }
-        if (launch_lift_i16(static_cast<const int16_t *>(W_dev), (size_t)m * K, M32, s) != cudaSuccess ||
-            launch_transpose_u32(M32, m, K, MT32, s) != cudaSuccess) {
-            cudaFree(M32);
-            cudaFree(MT32);
+        if (launch_lift_i16(static_cast<const int16_t *>(W_dev), (size_t)m * K, tmp.M32, s) != cudaSuccess ||
+            launch_transpose_u32(tmp.M32, m, K, tmp.MT32, s) != cudaSuccess)
             return fail(PVMVMD_E_CUDA);
-        }
-        st = encode_lanes(c->gx, K, c->rate, MT32, false, (size_t)m, m, c->PT, (size_t)m, err, s);
-        if (!st) st = encode_lanes(c->gy, m, c->rate, M32, false, (size_t)K, K, c->Q, (size_t)K, err, s);
-        cudaFree(M32);
-        cudaFree(MT32);
-        if (st) return fail(st);
-        if ((st = read_and_clear_error())) return fail(st);
-        *out = c;
-        return PVMVMD_OK;
+        rows = tmp.M32;
+        cols = tmp.MT32;
+    } else {
+        if (dev_alloc(&tmp.MT, (size_t)m * K) != cudaSuccess) return fail(PVMVMD_E_NOMEM);
+        if (launch_transpose_i8(static_cast<const int8_t *>(W_dev), m, K, tmp.MT, s) != cudaSuccess)
+            return fail(PVMVMD_E_CUDA);
+        cols = tmp.MT;
     }
-    // P^T = G_x^T M^T: the m rows of M are the lanes, so transpose M first.
-    int8_t *MT = nullptr;
-    if (dev_alloc(&MT, (size_t)m * K) != cudaSuccess) return fail(PVMVMD_E_NOMEM);
-    if (launch_transpose_i8(static_cast<const int8_t *>(W_dev), m, K, MT, s) != cudaSuccess) {
-        cudaFree(MT);
-        return fail(PVMVMD_E_CUDA);
-    }
-    st = encode_lanes(c->gx, K, c->rate, MT, true, (size_t)m, m, c->PT, (size_t)m, err, s);
-    cudaFree(MT);
+    // P^T = G_x^T M^T: the m rows of M are the lanes; Q = G_y^T M: its K columns
+    st = encode_lanes(c->gx, K, c->rate, cols, !w16, (size_t)m, m, c->PT, (size_t)m, tmp.lanes, err, s);
+    if (!st) st = encode_lanes(c->gy, m, c->rate, rows, !w16, (size_t)K, K, c->Q, (size_t)K, tmp.lanes, err, s);
+    if (!st && cudaStreamSynchronize(s) != cudaSuccess) st = PVMVMD_E_CUDA;
+    if (!st) st = read_and_clear_error();
     if (st) return fail(st);
-    // Q = G_y^T M: the K columns of M are the lanes.
-    st = encode_lanes(c->gy, m, c->rate, W_dev, true, (size_t)K, K, c->Q, (size_t)K, err, s);
-    if (st) return fail(st);
-    if ((st = read_and_clear_error())) return fail(st);
     *out = c;
     return PVMVMD_OK;
 }
@@ -984,12 +1031,28 @@ int pvmvmd_bv_preprocess(const int8_t *W_dev, int B, int m, int n, const pvmvmd_
     c->B = B; c->m = m; c->n = n; c->rate = rate; c->N = (int)N; c->N2 = (int)N2;
     c->t = t; c->ell = ell; c->t2 = t2; c->ell2 = ell2;
     auto fail = [&](int code) {
+        cudaStreamSynchronize(s);
+        (void)cudaGetLastError();
         pvmvmd_bv_destroy(c);
         return code;
     };
     const uint32_t Bn = (uint32_t)B * n;
-    if ((st = upload_code(c, c->g, *key, 3, (uint32_t)N, s))) return fail(st);
-    if ((st = upload_code(c, c->g2, *key, 4, (uint32_t)N2, s))) return fail(st);
+    struct Temp {
+        uint32_t *draws = nullptr, *Qt = nullptr;
+        LaneScratch lanes;
+        cudaStream_t s;
+        ~Temp() {
+            cudaStreamSynchronize(s);
+            cudaFree(draws);
+            cudaFree(Qt);
+        }
+    } tmp;
+    tmp.s = s;
+    CodeDev *const codes[2] = {&c->g, &c->g2};
+    const int which[2] = {3, 4};
+    const uint32_t lengths[2] = {(uint32_t)N, (uint32_t)N2};
+    if ((st = sample_codes(c, *key, codes, which, lengths, &tmp.draws, s))) return fail(st);
+    if ((st = tmp.lanes.alloc({{(uint32_t)N, (uint32_t)n}, {(uint32_t)N2, (uint32_t)N}}))) return fail(st);
     const size_t sw = encode_scan_status_words((uint32_t)N, (uint32_t)B);
     if (ctx_alloc(c, &c->Qs, (size_t)N * Bn) != cudaSuccess ||
         ctx_alloc(c, &c->QauxT, (size_t)N2 * N) != cudaSuccess ||
@@ -1008,20 +1071,17 @@ int pvmvmd_bv_preprocess(const int8_t *W_dev, int B, int m, int n, const pvmvmd_
     // Q_b = G^T M_b into the column block b n of Qs (the lanes are M_b's columns)
     for (int b = 0; b < B; ++b) {
         st = encode_lanes(c->g, (uint32_t)m, (uint32_t)rate, W_dev + (size_t)b * m * n, true, (size_t)n,
-                          (uint32_t)n, c->Qs + (size_t)b * n, (size_t)Bn, err, s);
+                          (uint32_t)n, c->Qs + (size_t)b * n, (size_t)Bn, tmp.lanes, err, s);
         if (st) return fail(st);
     }
     // Qaux = Qt^T G': row i is G'^T applied to row i of Qs; encode with the
     // N rows of Qs as lanes, so Qs is transposed first (Qt, B n x N)
-    uint32_t *Qt = nullptr;
-    if (dev_alloc(&Qt, (size_t)Bn * N) != cudaSuccess) return fail(PVMVMD_E_NOMEM);
-    if (launch_transpose_u32(c->Qs, (int)N, (int)Bn, Qt, s) != cudaSuccess) {
-        cudaFree(Qt);
-        return fail(PVMVMD_E_CUDA);
-    }
-    st = encode_lanes(c->g2, Bn, (uint32_t)rate, Qt, false, (size_t)N, (uint32_t)N, c->QauxT, (size_t)N, err, s);
-    cudaFree(Qt);
+    if (dev_alloc(&tmp.Qt, (size_t)Bn * N) != cudaSuccess) return fail(PVMVMD_E_NOMEM);
+    if (launch_transpose_u32(c->Qs, (int)N, (int)Bn, tmp.Qt, s) != cudaSuccess) return fail(PVMVMD_E_CUDA);
+    st = encode_lanes(c->g2, Bn, (uint32_t)rate, tmp.Qt, false, (size_t)N, (uint32_t)N, c->QauxT, (size_t)N, tmp.lanes,
+                      err, s);
     if (st) return fail(st);
+    if (cudaStreamSynchronize(s) != cudaSuccess) return fail(PVMVMD_E_CUDA);
     if ((st = read_and_clear_error())) return fail(st);
     *out = c;
     return PVMVMD_OK;

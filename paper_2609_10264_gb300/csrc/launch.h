@@ -23,6 +23,22 @@ inline size_t scan_status_words(uint32_t N, uint32_t count) {
     return 1 + (size_t)count * scan_tiles(N);
 }
 
+// Device sampling of a public code (code_sample.cu): streams tag0 .. tag0 + 3
+// give pi1, pi2, v1, v2 (N words each); the others are the derived tables
+// (CodeDev in api.cu).  `perm` is filled in by the launch.
+struct PermScratch {
+    uint32_t *j, *head, *link, *next, *succ;
+};
+struct CodeDraws {
+    uint32_t N, tag0;
+    uint32_t *pi1, *pi2, *v1, *v2, *pi1inv, *pi2inv, *v2p, *v2m, *v1pm, *v1m;
+    PermScratch perm[2];
+};
+// One or two codes of one key; scratch[k] holds code_draw_scratch_words(N_k).
+size_t code_draw_scratch_words(uint32_t N);
+cudaError_t launch_code_draws(const pvmvmd_key &key, CodeDraws *codes, int count, uint32_t *const *scratch,
+                              cudaStream_t s);
+
 // Sample `count` vectors of E_t^N: vector j uses index idx0 + j, reading
 // nonces (tag, 2*idx) and (tag, 2*idx + 1).  out: [count][2t] (ascending
 // support, then values).  Also zeroes clear[0 .. clear_words) for the scan

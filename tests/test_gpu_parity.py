@@ -138,6 +138,27 @@ def test_tiled_syndrome_round_trip(pv, wl, m, K, B, kw):
     _full_round_trip(pv, W, x, seeds=(m + B, K, B), params=_params(pv, **kw), oracle_kw=okw)
 
 
+@pytest.mark.parametrize("N", [1, 2, 3, 33, 2047, 2048, 2049, 3073, 16384, 40000, 114688])
+def test_code_tables_sampled_on_device(pv, N):
+    """The codes drawn on the device equal the host's draw for draw, at lengths
+    around the batch (1024 indices), the last 2048 and a round of keystream
+    (16384 words), and the inverse permutations and scaled tables follow."""
+    W = np.ones((1, N), np.int8)
+    ctx = pv.pvmvmd_preprocess(to_dev(W), key=N + 5, params=_params(pv, rate=1, t_x=1, t_y=1, ell=1))
+    v, tabs = ctx_tables(pv, ctx)
+    assert (v.N_x, v.N_y) == (N, 1)
+    for which, name in ((0, "gx"), (1, "gy")):
+        exp = pv.pvmvmd_code_sample_host(N + 5, which, N if which == 0 else 1)
+        for f, e in zip(("pi1", "pi2", "v1", "v2"), exp):
+            assert np.array_equal(tabs[f"{name}_{f}"], e), f"{name}_{f}"
+    # an encoding uses the derived tables: G_x e for one vector, by the oracle
+    pp = oracle.PublicParams(W, oracle.key_from_seed(N + 5), t_x=1, t_y=1, ell=1, rate=1, with_tables=False)
+    Xh, st = pv.pvmvmd_encode(ctx, to_dev(np.zeros((1, N), np.uint32)), key=6)
+    assert np.array_equal(pv.as_u32(Xh)[0], pp.encrypt(np.zeros(N, np.uint32), oracle.key_from_seed(6), 0)[0])
+    assert pv.pvmvmd_device_status() == 0
+    ctx.destroy()
+
+
 def test_encode_chunking_matches(pv, wl):
     """Encoding in chunks of 3 vectors (scratch_batch) gives the same result."""
     W = wl.weights_uniform(64, 96, 1)
