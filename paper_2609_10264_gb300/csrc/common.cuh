@@ -27,8 +27,12 @@ constexpr uint32_t kSpinLimit = 1u << 22;
 
 // ---------------------------------------------------------------- field F_q
 __host__ __device__ __forceinline__ uint32_t fadd(uint32_t a, uint32_t b) {
-    uint32_t r = a + b;  // a, b < q < 2^31, so no wrap
+    const uint32_t r = a + b;  // a, b < q < 2^31, so no wrap
+#ifdef __CUDA_ARCH__
+    return min(r, r - kQ);  // r - q wraps above 2^31 where r < q
+#else
     return r >= kQ ? r - kQ : r;
+#endif
 }
 __host__ __device__ __forceinline__ uint32_t fsub(uint32_t a, uint32_t b) {
     return a >= b ? a - b : a + (kQ - b);
@@ -64,8 +68,12 @@ static_assert(PVMVMD_Q * qinv_mod_2_32() == 1u, "q^-1 mod 2^32");
 __host__ __device__ __forceinline__ uint32_t fmul_mont(uint32_t a, uint32_t b_m) {
     const uint64_t t = (uint64_t)a * b_m;
     const uint32_t m = (uint32_t)t * kQInvNeg;
-    const uint64_t u = (t + (uint64_t)m * kQ) >> 32;  // t + m q < 2^62 + 2^63
-    return (uint32_t)(u >= kQ ? u - kQ : u);
+    const uint32_t u = (uint32_t)((t + (uint64_t)m * kQ) >> 32);  // t + m q < 2^62 + 2^63: u < 2q
+#ifdef __CUDA_ARCH__
+    return min(u, u - kQ);
+#else
+    return u >= kQ ? u - kQ : u;
+#endif
 }
 // b -> b R mod q (host table preparation).
 __host__ __device__ __forceinline__ uint32_t to_mont(uint32_t b) {
