@@ -877,7 +877,11 @@ __global__ void __launch_bounds__(kFusedThreads) k_syndrome_fused(
 // tile and the lanes' values in separate arrays behind a fence and block
 // barriers, with warp 0 reading 32 flags at a time, took 0.755 ms per
 // 4096 x 4096 encoding.)  At 32 positions per tile the kernel is held to 64
-// registers, four CTAs per SM.
+// registers, four CTAs per SM.  Issue-bound: loads without predicates (a lane
+// past L reads the last one, a position past N row 0 with scale 0), one
+// shared-memory read per position for the row's byte offset and scale, and
+// the field additions by min took a launch at N = 32768, L = 4096 from 295 to
+// 200 us (int8) and 287 to 235 us (uint32).
 // -----------------------------------------------------------------------------
 __device__ __forceinline__ unsigned long long enc_status(uint32_t state, uint32_t v) {
     return ((unsigned long long)state << 32) | v;
@@ -891,8 +895,7 @@ __global__ void __launch_bounds__(256, 4) k_encode_scan(const void *__restrict__
                                                     unsigned long long *status, uint32_t *ticket_ctr,
                                                     uint32_t *__restrict__ err) {
     __shared__ uint32_t s_ticket;
-    __shared__ unsigned long long s_off[kEncTile];  // source row offset (row * ldx) of each position
-    __shared__ uint32_t s_vs[kEncTile];
+    __shared__ ulonglong2 s_row[kEncTile];  // byte offset of the source row and scale of each position
     const int tid = threadIdx.x;
     const uint32_t nlb = (L + 255) / 256;
     const uint32_t ntiles = (N + kEncTile - 1) / kEncTile;
@@ -909,25 +912,30 @@ __global__ void __launch_bounds__(256, 4) k_encode_scan(const void *__restrict__
     const uint32_t j0 = tile * kEncTile;
     if (tid < kEncTile) {
         const uint32_t j = j0 + tid;
-        s_off[tid] = (unsigned long long)(j < N ? __ldg(perm + j) / div : 0u) * ldx;
-        s_vs[tid] = j < N ? __ldg(vscale_m + j) : 0u;  // 0 past N: adds nothing
+        // scale 0 past N: adds nothing
+        const unsigned long long row = j < N ? __ldg(perm + j) / div : 0u;
+        s_row[tid] = make_ulonglong2(row * ldx * (kI8 ? 1 : 4), j < N ? __ldg(vscale_m + j) : 0u);
     }
     __syncthreads();
 
+    // an idle lane reads a neighbour's column; nothing of it is stored
+    const uint32_t lr = lane_ok ? l : L - 1;
     uint32_t v[kEncTile];
+    if (kI8) {
+        const int8_t *X = static_cast<const int8_t *>(Xv) + lr;
 #pragma unroll
-    for (int u = 0; u < kEncTile; ++u) {
-        const bool ok = lane_ok && j0 + u < N;
-        const size_t src = (size_t)s_off[u] + l;
-        if (kI8)
-            v[u] = ok ? flift_i8(static_cast<const int8_t *>(Xv)[src]) : 0u;
-        else
-            v[u] = ok ? static_cast<const uint32_t *>(Xv)[src] : 0u;
+        for (int u = 0; u < kEncTile; ++u) v[u] = (uint32_t)(int32_t)X[s_row[u].x];
+#pragma unroll
+        for (int u = 0; u < kEncTile; ++u) v[u] = min(v[u], v[u] + kQ);  // the lift: w mod q
+    } else {
+        const char *X = static_cast<const char *>(Xv) + (size_t)lr * 4;
+#pragma unroll
+        for (int u = 0; u < kEncTile; ++u) v[u] = *reinterpret_cast<const uint32_t *>(X + s_row[u].x);
     }
     uint32_t run = 0;
 #pragma unroll
     for (int u = 0; u < kEncTile; ++u) {
-        run = fadd(run, fmul_mont(v[u], s_vs[u]));
+        run = fadd(run, fmul_mont(v[u], (uint32_t)s_row[u].y));
         v[u] = run;
     }
 
@@ -958,24 +966,48 @@ __global__ void __launch_bounds__(256, 4) k_encode_scan(const void *__restrict__
     }
     if (lane_ok) {
         uint32_t *yp = Y + (size_t)j0 * ldy + l;
-        const uint32_t nu = N - j0 < (uint32_t)kEncTile ? N - j0 : (uint32_t)kEncTile;
+        if (j0 + kEncTile <= N) {
 #pragma unroll
-        for (int u = 0; u < kEncTile; ++u, yp += ldy)
-            if ((uint32_t)u < nu) *yp = fadd(v[u], prefix);
+            for (int u = 0; u < kEncTile; ++u, yp += ldy) *yp = fadd(v[u], prefix);
+        } else {
+            const uint32_t nu = N - j0;
+#pragma unroll
+            for (int u = 0; u < kEncTile; ++u, yp += ldy)
+                if ((uint32_t)u < nu) *yp = fadd(v[u], prefix);
+        }
     }
 }
 
-__global__ void k_transpose_i8(const int8_t *__restrict__ in, int R, int C, int8_t *__restrict__ out) {
-    __shared__ int8_t tile[32][33];
-    const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int r = r0 + i, c = c0 + threadIdx.x;
-        if (r < R && c < C) tile[i][threadIdx.x] = in[(size_t)r * C + c];
+// 128 x 128 tiles (256 threads): a thread reads 16 rows' four bytes, and writes
+// 16 rows' four bytes picked from the tile, 128 bytes per warp both ways.
+// (32 x 32 tiles a byte at a time: 31.6 us at 4096 x 4096.)
+__global__ void __launch_bounds__(256) k_transpose_i8(const int8_t *__restrict__ in, int R, int C, int8_t *__restrict__ out,
+                                                     bool words) {
+    __shared__ __align__(16) int8_t tile[128][132];
+    const int c0 = blockIdx.x * 128, r0 = blockIdx.y * 128;
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+    for (int i = y; i < 128; i += 8) {
+        const int r = r0 + i, c = c0 + 4 * x;
+        if (words && r < R && c + 4 <= C) {
+            *reinterpret_cast<uint32_t *>(&tile[i][4 * x]) = __ldg(reinterpret_cast<const uint32_t *>(in + (size_t)r * C + c));
+        } else {
+            for (int b = 0; b < 4; ++b)
+                if (r < R && c + b < C) tile[i][4 * x + b] = in[(size_t)r * C + c + b];
+        }
     }
     __syncthreads();
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int c = c0 + i, r = r0 + threadIdx.x;
-        if (r < R && c < C) out[(size_t)c * R + r] = tile[threadIdx.x][i];
+    for (int i = y; i < 128; i += 8) {
+        const int c = c0 + i, r = r0 + 4 * x;
+        if (c >= C) continue;
+        if (words && r + 4 <= R) {
+            uint32_t w = 0;
+#pragma unroll
+            for (int b = 0; b < 4; ++b) w |= (uint32_t)(uint8_t)tile[4 * x + b][i] << (8 * b);
+            *reinterpret_cast<uint32_t *>(out + (size_t)c * R + r) = w;
+        } else {
+            for (int b = 0; b < 4; ++b)
+                if (r + b < R) out[(size_t)c * R + r + b] = tile[4 * x + b][i];
+        }
     }
 }
 
@@ -1484,9 +1516,11 @@ cudaError_t launch_encode_scan(const void *X, bool x_is_i8, size_t ldx, const ui
 
 cudaError_t launch_transpose_i8(const int8_t *in, int R, int C, int8_t *out, cudaStream_t s) {
     if (R <= 0 || C <= 0) return cudaSuccess;
-    dim3 grid((C + 31) / 32, (R + 31) / 32), block(32, 8);
+    dim3 grid((C + 127) / 128, (R + 127) / 128);
     if (grid.y > 65535u) return cudaErrorInvalidValue;
-    k_transpose_i8<<<grid, block, 0, s>>>(in, R, C, out); note_launch();
+    const bool words = C % 4 == 0 && R % 4 == 0 &&
+                       ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 3u) == 0;
+    k_transpose_i8<<<grid, 256, 0, s>>>(in, R, C, out, words); note_launch();
     return cudaGetLastError();
 }
 
