@@ -778,11 +778,15 @@ struct GroupJob {
     unsigned long long *acc;  // B x m partial sums when split > 1
     int m, K, B, nkb, nvt, mp, split, per, item0;
     const uint32_t *Xhat;     // for the digit-tile kernel
+    unsigned dblk0, fblk0;    // first block of the job in the digit-tile and split-finish grids
 };
 struct GroupArgs {
     CUtensorMap map[kMaxGroupJobs];  // M of each job as a K x m tensor of bytes
     GroupJob job[kMaxGroupJobs];
     int njobs, total_items;
+    uint4 *acc;               // the split jobs' partial sums, one after the other
+    size_t acc_chunks;        // 16-byte chunks of them
+    unsigned zero0, zeros;    // blocks of the digit-tile grid that clear them
 };
 
 struct Item {
@@ -810,18 +814,24 @@ __device__ __forceinline__ int group_item_index(int r, int c, int C, int total) 
     return idx < total ? idx : -1;
 }
 
-// Digit tiles of every job (as k_digit_tiles, blockIdx.y = job) and zeroed
-// partial-sum buffers of the split jobs.
+// Digit tiles of every job (as k_digit_tiles; job j has the blocks from
+// dblk0), and zeroed partial sums of the split jobs (the blocks from zero0).
 template <int V>
 __global__ void __launch_bounds__(256) k_digit_tiles_grouped(const __grid_constant__ GroupArgs args) {
     using T = GTile<V>;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const GroupJob &g = args.job[blockIdx.y];
-    const size_t gid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g.split > 1) {
-        const size_t n = (size_t)g.B * g.m;
-        for (size_t i = gid; i < n; i += (size_t)gridDim.x * blockDim.x) g.acc[i] = 0ull;
+    // x_hat comes from the kernel before, which may also still use the scratch
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (blockIdx.x >= args.zero0) {
+        for (size_t i = (size_t)(blockIdx.x - args.zero0) * 256 + threadIdx.x; i < args.acc_chunks;
+             i += (size_t)args.zeros * 256)
+            args.acc[i] = make_uint4(0u, 0u, 0u, 0u);
+        return;
     }
+    int j = 0;
+    while (j + 1 < args.njobs && blockIdx.x >= args.job[j + 1].dblk0) ++j;
+    const GroupJob &g = args.job[j];
+    const size_t gid = (size_t)(blockIdx.x - g.dblk0) * 256 + threadIdx.x;
     const size_t per_vec = (size_t)g.nkb * 8;
     const size_t total = (size_t)g.nvt * T::kBV * per_vec;
     if (gid >= total) return;
@@ -862,13 +872,21 @@ __global__ void __launch_bounds__(256) k_digit_tiles_grouped(const __grid_consta
     }
 }
 
-// Y = acc mod q for the split jobs (blockIdx.y = job).
+// Y = acc mod q for the split jobs (job j has the blocks from fblk0, four
+// outputs per thread).
+constexpr int kFinishPer = 4;
 __global__ void __launch_bounds__(256) k_split_finish(const __grid_constant__ GroupArgs args) {
-    const GroupJob &g = args.job[blockIdx.y];
-    if (g.split <= 1) return;
-    const size_t n = (size_t)g.B * g.m;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        g.Y[i] = fred(g.acc[i]);
+    int j = 0;
+    while (j + 1 < args.njobs && blockIdx.x >= args.job[j + 1].fblk0) ++j;
+    const GroupJob &g = args.job[j];
+    const size_t n = (size_t)g.B * g.m, i0 = (size_t)(blockIdx.x - g.fblk0) * (256 * kFinishPer) + threadIdx.x;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    unsigned long long v[kFinishPer];
+#pragma unroll
+    for (int u = 0; u < kFinishPer; ++u) v[u] = i0 + 256 * u < n ? g.acc[i0 + 256 * u] : 0ull;
+#pragma unroll
+    for (int u = 0; u < kFinishPer; ++u)
+        if (i0 + 256 * u < n) g.Y[i0 + 256 * u] = fred(v[u]);
 }
 
 template <int V>
@@ -895,6 +913,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int c = (int)(blockIdx.x >> 1), C = (int)(gridDim.x >> 1);
     const int total = args.total_items;
 
+    // k_split_finish may be put in place beside this kernel; it waits for it
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (tid == 0) {
         for (int s = 0; s < kGStages; ++s) {
             // every converter warp (both groups), the digit copies' arrival
@@ -1281,6 +1301,7 @@ cudaError_t launch_grouped_v(const BatchJob *jobs, int count, uint32_t *err, cud
             dbytes += (size_t)j.nvt * j.nkb * T::kBTile;
             if (j.split > 1) abytes += (size_t)j.B * j.m * 8;
         }
+        abytes = (abytes + 15) & ~(size_t)15;
         void *buf = nullptr;
         cudaError_t e = stream_scratch(kScratchDigitTiles, dbytes + abytes, s, &buf);
         if (e != cudaSuccess) return e;
@@ -1290,7 +1311,8 @@ cudaError_t launch_grouped_v(const BatchJob *jobs, int count, uint32_t *err, cud
         memset(&args, 0, sizeof(args));
         uint8_t *dp = static_cast<uint8_t *>(buf);
         unsigned long long *ap = reinterpret_cast<unsigned long long *>(dp + dbytes);
-        int item0 = 0, any_split = 0, max_threads = 0, max_acc = 0;
+        int item0 = 0;
+        unsigned dblk = 0, fblk = 0;
         for (int i = 0; i < (int)plan.size(); ++i) {
             const PlanJob &p = plan[i];
             const BatchJob &b = jobs[p.src];
@@ -1302,8 +1324,6 @@ cudaError_t launch_grouped_v(const BatchJob *jobs, int count, uint32_t *err, cud
             if (p.split > 1) {
                 g.acc = ap;
                 ap += (size_t)p.B * p.m;
-                any_split = 1;
-                max_acc = std::max(max_acc, p.B * p.m);
             }
             g.m = p.m;
             g.K = p.K;
@@ -1316,7 +1336,10 @@ cudaError_t launch_grouped_v(const BatchJob *jobs, int count, uint32_t *err, cud
             g.item0 = item0;
             g.Xhat = b.Xhat;
             item0 += p.items;
-            max_threads = std::max(max_threads, p.nvt * T::kBV * p.nkb * 8);
+            g.dblk0 = dblk;
+            dblk += (unsigned)(((size_t)p.nvt * T::kBV * p.nkb * 8 + 255) / 256);
+            g.fblk0 = fblk;
+            if (p.split > 1) fblk += (unsigned)(((size_t)p.B * p.m + 256 * kFinishPer - 1) / (256 * kFinishPer));
             const cuuint64_t gdim[2] = {(cuuint64_t)p.K, (cuuint64_t)p.m};
             const cuuint64_t gstride[1] = {(cuuint64_t)p.K};
             const cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)kBM};
@@ -1329,10 +1352,21 @@ cudaError_t launch_grouped_v(const BatchJob *jobs, int count, uint32_t *err, cud
         args.njobs = (int)plan.size();
         args.total_items = item0;
         if (item0 == 0) continue;
-        // digit tiles (and zeroed partial sums); enough CTAs for the largest job
-        const int dblocks = std::max((max_threads + 255) / 256, any_split ? std::min(1024, (max_acc + 255) / 256) : 1);
-        k_digit_tiles_grouped<V><<<dim3((unsigned)dblocks, (unsigned)args.njobs), 256, 0, s>>>(args); note_launch();
-        e = cudaGetLastError();
+        // digit tiles, and 1 KiB or more of the partial sums per further block
+        args.acc = reinterpret_cast<uint4 *>(static_cast<uint8_t *>(buf) + dbytes);
+        args.acc_chunks = abytes / 16;
+        args.zero0 = dblk;
+        args.zeros = (unsigned)std::min<size_t>(1024, (args.acc_chunks + 255) / 256);
+        cudaLaunchAttribute pdl[1];
+        pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        pdl[0].val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t dcfg = {};
+        dcfg.gridDim = dim3(dblk + args.zeros, 1, 1);
+        dcfg.blockDim = dim3(256, 1, 1);
+        dcfg.stream = s;
+        dcfg.attrs = pdl;
+        dcfg.numAttrs = 1;
+        e = counted_launch(cudaLaunchKernelEx(&dcfg, k_digit_tiles_grouped<V>, args));
         if (e != cudaSuccess) return e;
         const int C = std::min(best_c, item0);
         cudaLaunchConfig_t cfg = {};
@@ -1354,12 +1388,16 @@ cudaError_t launch_grouped_v(const BatchJob *jobs, int count, uint32_t *err, cud
         const uint64_t wait_ns = dbg.site == PVMVMD_DEBUG_WAIT_PRODUCT ? dbg.limit : kWaitNs;
         e = counted_launch(cudaLaunchKernelEx(&cfg, k_batched_grouped<V>, args, err, skip_report, wait_ns));
         if (e != cudaSuccess) return e;
-        if (any_split) {
-            int dev = 0, sms = 0;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            k_split_finish<<<dim3((unsigned)(2 * sms), (unsigned)args.njobs), 256, 0, s>>>(args); note_launch();
-            e = cudaGetLastError();
+        if (fblk) {
+            // jobs without splits before a split one share its first block
+            // index; the last such job is the one the kernel finds
+            cudaLaunchConfig_t fcfg = {};
+            fcfg.gridDim = dim3(fblk, 1, 1);
+            fcfg.blockDim = dim3(256, 1, 1);
+            fcfg.stream = s;
+            fcfg.attrs = pdl;
+            fcfg.numAttrs = 1;
+            e = counted_launch(cudaLaunchKernelEx(&fcfg, k_split_finish, args));
             if (e != cudaSuccess) return e;
         }
     }
