@@ -187,6 +187,7 @@ struct CodeDev {
     uint32_t *pi1inv = nullptr, *pi2inv = nullptr, *v2p = nullptr;
     uint32_t *v2m = nullptr, *v1pm = nullptr;  // Montgomery-scaled v2 and v1 o pi1^-1
     uint32_t *v1m = nullptr;                   // Montgomery-scaled v1
+    uint32_t *slices = nullptr;                // the sliced syndrome's tables (G_x, where it is used)
 };
 
 }  // namespace
@@ -508,6 +509,12 @@ int preprocess_impl(const void *W_dev, bool w16, int m, int K, const pvmvmd_para
     const int which[2] = {0, 1};
     const uint32_t lengths[2] = {(uint32_t)c->Nx, (uint32_t)c->Ny};
     if ((st = sample_codes(c, *key, codes, which, lengths, &tmp.draws, s))) return fail(st);
+    if (!syndrome_fused_fits(c->Nx, c->t_x) && syndrome_sliced_fits(c->Nx, K, c->rate, c->t_x)) {
+        CodeDev &d = c->gx;
+        if (ctx_alloc(c, &d.slices, slice_table_words(c->Nx)) != cudaSuccess) return fail(PVMVMD_E_NOMEM);
+        if (launch_slice_tables(d.pi1, d.pi2, d.v2m, c->Nx, c->rate, d.slices, s) != cudaSuccess)
+            return fail(PVMVMD_E_CUDA);
+    }
     // the small arrays in one allocation
     const size_t f = (size_t)((c->sb + 3) & ~3) * c->Nx;  // lanes padded to 4
     const bool lanes = c->sb >= kLaneMinBatch;
@@ -685,6 +692,17 @@ int encode_batch(pvmvmd_ctx *ctx, const uint32_t *X_dev, int B, const pvmvmd_key
     uint32_t *stp = static_cast<uint32_t *>(st_dev);
     const CodeDev &d = ctx->gx;
     const bool fits = syndrome_fused_fits(ctx->Nx, ctx->t_x);
+    // A code too long for that, and vectors enough for the SMs: a CTA per
+    // vector, two per SM.  Against the lanes, back to back and alone (one
+    // encode and a field add, about 8 us of it launches): K = 8192, B = 256: 55
+    // against 83 us and 71 against 85; B = 100: 23 / 45 and 44 / 46; B = 64: 15 /
+    // 40 but 44 / 42; K = 5700, B = 32: 7 / 36 and 36 / 37; K = 13000, B = 152:
+    // 54 / 97 and 74 / 99, B = 128: 47 / 68 but 74 / 70.  The lines keep both.
+    if (d.slices && B >= (ctx->Nx <= 48 * 1024 ? kLaneMinBatch : ctx->Nx <= 80 * 1024 ? 2 * sm_count() / 3 : sm_count())) {
+        PV_CUDA(launch_syndrome_sliced(*key, kTagMask, 0, ctx->Nx, ctx->t_x, (uint32_t)B, d.slices, d.v1m, ctx->K, stp,
+                                       X_dev, Xhat_dev, s));
+        return PVMVMD_OK;
+    }
     if (B >= kLaneMinBatch && ctx->laux && !fits) {
         // vectors as lanes: every permutation step moves whole rows (a code
         // that fits one CTA's shared memory stays on chip in the fused kernel)

@@ -71,6 +71,17 @@ cudaError_t launch_syndrome_fused(const pvmvmd_key &key, uint32_t tag, uint64_t 
                                   uint32_t n, uint32_t r, uint32_t *sparse_out,
                                   const uint32_t *addend, uint32_t *out, cudaStream_t s);
 
+// Sliced syndrome, one CTA per vector with the code taken slice by slice, as
+// launch_syndrome_fused otherwise.  tables: slice_table_words(N) words, 16-byte
+// aligned, from launch_slice_tables; v1m = v1 R.
+bool syndrome_sliced_fits(uint32_t N, uint32_t n, uint32_t r, uint32_t t);
+size_t slice_table_words(uint32_t N);
+cudaError_t launch_slice_tables(const uint32_t *pi1, const uint32_t *pi2, const uint32_t *v2m, uint32_t N, uint32_t r,
+                                uint32_t *tables, cudaStream_t s);
+cudaError_t launch_syndrome_sliced(const pvmvmd_key &key, uint32_t tag, uint64_t idx0, uint32_t N, uint32_t t,
+                                   uint32_t count, const uint32_t *tables, const uint32_t *v1m, uint32_t n,
+                                   uint32_t *sparse_out, const uint32_t *addend, uint32_t *out, cudaStream_t s);
+
 // Lane-parallel syndrome for L vectors (vector b uses index idx0 + b, as
 // launch_sample_sparse): sparse_out [L][2t] as there, S lane_state_words(t,
 // L) words (suffix sums of the values, then a bucket index into the sorted

@@ -860,6 +860,165 @@ __global__ void __launch_bounds__(kFusedThreads) k_syndrome_fused(
 }
 
 // -----------------------------------------------------------------------------
+// Sliced syndrome: x' = G e, one CTA of 512 threads per vector and two per SM,
+// for codes longer than one CTA's shared memory.  The positions are taken in
+// slices of kSlice from the end of the vector, so that the suffix sum of a
+// slice starts from the carry of those before it, and only one slice and the n
+// outputs are held:
+//   c over the slice, scattered from the positions k with pi2(k) in it, which
+//     a table lists in ascending order (k << kSliceBits | pi2(k) mod kSlice, so
+//     that a warp's lookups of (A e)_k meet in one or two supports);
+//   a block-wide suffix scan of eight positions per thread, in registers;
+//   out_{pi1(i) / r} += v1_i d_i by shared-memory atomics: the sum mod 2^32 and,
+//     from the value an addition finds, its carries (a byte per output).
+// Nothing of length N goes through memory (the lanes below move 20 bytes per
+// vector and position); bound by instruction issue and shared-memory conflicts
+// of the two permutations.  256 vectors at N = 65536: 83 -> 55 us (outputs from
+// a second pass over the slice in shared memory: 67; 1024 threads, one CTA per
+// SM: 74).
+// -----------------------------------------------------------------------------
+constexpr int kSliceBits = 12;
+constexpr uint32_t kSlice = 1u << kSliceBits;
+constexpr int kSliceThreads = 512;
+constexpr int kSliceItems = (int)kSlice / kSliceThreads;  // consecutive positions of a thread
+static_assert(kSliceItems == 8, "two 16-byte reads of a table");
+
+// t[0 .. 8) = p[at .. at + 8), zero from index `end`
+__device__ __forceinline__ void slice_read(const uint32_t *__restrict__ p, uint32_t at, uint32_t end, uint32_t (&t)[8]) {
+    if (at + 8 <= end) {
+        const uint4 a = __ldg(reinterpret_cast<const uint4 *>(p + at)), b = __ldg(reinterpret_cast<const uint4 *>(p + at + 4));
+        t[0] = a.x; t[1] = a.y; t[2] = a.z; t[3] = a.w;
+        t[4] = b.x; t[5] = b.y; t[6] = b.z; t[7] = b.w;
+    } else {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) t[u] = at + u < end ? __ldg(p + at + u) : 0u;
+    }
+}
+
+__global__ void __launch_bounds__(kSliceThreads, 2) k_syndrome_sliced(
+    pvmvmd_key key, uint32_t tag, uint64_t idx0, uint32_t N, uint32_t t, const uint32_t *__restrict__ kp,
+    const uint32_t *__restrict__ v2s, const uint32_t *__restrict__ v1m, const uint32_t *__restrict__ oj, uint32_t n,
+    uint32_t *__restrict__ sparse_out, const uint32_t *addend, uint32_t *out) {
+    extern __shared__ uint32_t sm[];
+    constexpr int nw = kSliceThreads / 32;
+    __shared__ uint32_t s_wtot[nw];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint32_t *F = sm;                         // padded slice
+    uint32_t *lo = F + fpad(kSlice);          // n: sums mod 2^32
+    uint32_t *hi = lo + n;                    // n bytes: their carries
+    uint32_t *supp = hi + (n + 3) / 4;        // t
+    uint32_t *suf = supp + t;                 // t + 1
+    uint32_t *bitmap = suf + t + 1;           // the support, and below it per 32 positions
+    uint16_t *cnt = reinterpret_cast<uint16_t *>(bitmap + (N + 31) / 32);
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // the keystream words pass through F (kSlice >= 1024)
+    sample_sorted<kSliceThreads>(key, tag, idx0 + blockIdx.x, N, t, bitmap, cnt, F, supp, suf, s_wtot);
+    for (uint32_t j = tid; j < n + (n + 3) / 4; j += kSliceThreads) lo[j] = 0u;
+    uint32_t carry = 0;
+    uint32_t s = (N + kSlice - 1) / kSlice - 1;
+    uint32_t at = s * kSlice + tid * kSliceItems;
+    uint32_t kk[8], vv[8];
+    slice_read(kp, at, N, kk);
+    slice_read(v2s, at, N, vv);
+    for (;; --s, at -= kSlice) {
+        // c over the slice; a short one (the last) has zeros above its end
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            if (at + u < N)
+                F[fpad(kk[u] & (kSlice - 1))] =
+                    fmul_mont(suf[support_rank(bitmap, cnt, kk[u] >> kSliceBits)], vv[u]);
+            else
+                F[fpad(tid * kSliceItems + u)] = 0u;
+        }
+        uint32_t ww[8];
+        slice_read(v1m, at, N, ww);
+        const uint4 o4 = __ldg(reinterpret_cast<const uint4 *>(oj) + at / 8);
+        __syncthreads();
+        uint32_t f[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) f[u] = F[fpad(tid * kSliceItems + u)];
+#pragma unroll
+        for (int u = 6; u >= 0; --u) f[u] = fadd(f[u], f[u + 1]);
+        uint32_t incl = f[0];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_down_sync(kFull, incl, o);
+            if (lane + o < 32) incl = fadd(incl, y);
+        }
+        if (lane == 0) s_wtot[warp] = incl;
+        if (s > 0) {  // tables of the next slice
+            slice_read(kp, at - kSlice, N, kk);
+            slice_read(v2s, at - kSlice, N, vv);
+        }
+        __syncthreads();  // F is read: the next slice may be scattered after this
+        // every warp: the totals of the warps after it, and all of them
+        const uint32_t wv = lane < nw ? s_wtot[lane] : 0u;
+        uint32_t winc = wv;
+#pragma unroll
+        for (int o = 1; o < nw; o <<= 1) {
+            const uint32_t y = __shfl_down_sync(kFull, winc, o);
+            if (lane + o < 32) winc = fadd(winc, y);
+        }
+        const uint32_t after = __shfl_sync(kFull, fsub(winc, wv), warp), all = __shfl_sync(kFull, winc, 0);
+        const uint32_t add = fadd(fadd(fsub(incl, f[0]), after), carry);
+        carry = fadd(carry, all);
+        const uint32_t oo[4] = {o4.x, o4.y, o4.z, o4.w};
+        uint32_t old[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const uint32_t j = u & 1 ? oo[u / 2] >> 16 : oo[u / 2] & 0xffffu;
+            f[u] = fmul_mont(fadd(f[u], add), ww[u]);  // 0 above the end of a short slice (scale 0)
+            old[u] = atomicAdd(lo + j, f[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (old[u] + f[u] < old[u]) {
+                const uint32_t j = u & 1 ? oo[u / 2] >> 16 : oo[u / 2] & 0xffffu;
+                atomicAdd(hi + (j >> 2), 1u << (8 * (j & 3)));
+            }
+        if (s == 0) break;
+    }
+    __syncthreads();
+    fused_publish<kSliceThreads>(sparse_out + (size_t)blockIdx.x * 2 * t, supp, suf, t, tid);
+    for (uint32_t j = tid; j < n; j += kSliceThreads) {
+        const uint32_t h = (hi[j >> 2] >> (8 * (j & 3))) & 0xffu;
+        const uint32_t x = fred(((uint64_t)h << 32) | lo[j]);
+        const size_t o = (size_t)blockIdx.x * n + j;
+        out[o] = addend ? fadd(addend[o], x) : x;
+    }
+}
+
+// The tables of k_syndrome_sliced, one CTA per slice: kp and v2s list the
+// positions k with pi2(k) in the slice in ascending order.
+__global__ void __launch_bounds__(1024) k_slice_tables(const uint32_t *__restrict__ pi1,
+                                                       const uint32_t *__restrict__ pi2,
+                                                       const uint32_t *__restrict__ v2m, uint32_t N, uint32_t r,
+                                                       uint32_t *__restrict__ kp, uint32_t *__restrict__ v2s,
+                                                       uint16_t *__restrict__ oj) {
+    __shared__ uint32_t s_wsum[2][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t at = blockIdx.x * kSlice;
+    int buf = 0;
+    for (uint32_t k0 = 0; k0 < N; k0 += 1024, buf ^= 1) {
+        const uint32_t k = k0 + threadIdx.x;
+        const uint32_t p = k < N ? __ldg(pi2 + k) : 0xffffffffu;
+        const bool in = k < N && p >> kSliceBits == blockIdx.x;
+        const uint32_t mask = __ballot_sync(kFull, in);
+        if (lane == 0) s_wsum[buf][warp] = __popc(mask);
+        __syncthreads();
+        const uint32_t wv = s_wsum[buf][lane];
+        const uint32_t e = at + __reduce_add_sync(kFull, lane < warp ? wv : 0u) + __popc(mask & lanemask_lt());
+        if (in) {
+            kp[e] = k << kSliceBits | (p & (kSlice - 1));
+            v2s[e] = v2m[k];
+        }
+        at += __reduce_add_sync(kFull, wv);
+    }
+    for (uint32_t i = blockIdx.x * kSlice + threadIdx.x; i < (blockIdx.x + 1) * kSlice; i += 1024)
+        oj[i] = i < N ? (uint16_t)(__ldg(pi1 + i) / r) : (uint16_t)0;
+}
+
+// -----------------------------------------------------------------------------
 // One accumulate stage of G^T w (App. B, encoding direction) over L lanes:
 //   Y[j][l] = sum_{j' <= j} vscale[j'] * X[perm[j'] / div][l]
 // With (perm, div, vscale) = (pi1, r, v1) this is A^T V1 Pi1^T R^T; with
@@ -1551,6 +1710,44 @@ cudaError_t launch_syndrome_fused(const pvmvmd_key &key, uint32_t tag, uint64_t 
     void *args[] = {(void *)&key, &tag, &idx0, &N, &t, &slice, &pi1inv, &n, &r, &sparse_out, &addend, &out,
                     &pi2, &v2m, &v1pm};
     return launch_pdl((const void *)k_syndrome_fused, dim3(count), dim3(kFusedThreads), fused_smem(slice, t), s, args);
+}
+
+namespace {
+size_t sliced_smem(uint32_t N, uint32_t n, uint32_t t) {
+    const size_t nbw = (N + 31) / 32;
+    return ((size_t)kSlice + kSlice / 32 + n + (n + 3) / 4 + 2 * (size_t)t + 1 + nbw + (nbw + 1) / 2) * sizeof(uint32_t);
+}
+constexpr size_t kSlicedMaxSmem = 110 * 1024;  // two CTAs per SM
+}  // namespace
+
+bool syndrome_sliced_fits(uint32_t N, uint32_t n, uint32_t r, uint32_t t) {
+    // k in 32 - kSliceBits bits, outputs in 16, carries of r terms in 8
+    return N <= (1u << (32 - kSliceBits)) && n <= 65536u && r <= 255u && sliced_smem(N, n, t) <= kSlicedMaxSmem;
+}
+size_t slice_table_words(uint32_t N) {
+    return 2 * (((size_t)N + 3) & ~(size_t)3) + (((size_t)N + kSlice - 1) / kSlice * kSlice) / 2;
+}
+
+cudaError_t launch_slice_tables(const uint32_t *pi1, const uint32_t *pi2, const uint32_t *v2m, uint32_t N, uint32_t r,
+                                uint32_t *tables, cudaStream_t s) {
+    const size_t Np = ((size_t)N + 3) & ~(size_t)3;
+    k_slice_tables<<<(N + kSlice - 1) / kSlice, 1024, 0, s>>>(pi1, pi2, v2m, N, r, tables, tables + Np,
+                                                              reinterpret_cast<uint16_t *>(tables + 2 * Np));
+    note_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t launch_syndrome_sliced(const pvmvmd_key &key, uint32_t tag, uint64_t idx0, uint32_t N, uint32_t t,
+                                   uint32_t count, const uint32_t *tables, const uint32_t *v1m, uint32_t n,
+                                   uint32_t *sparse_out, const uint32_t *addend, uint32_t *out, cudaStream_t s) {
+    if (count == 0) return cudaSuccess;
+    const cudaError_t attr = func_attr((const void *)k_syndrome_sliced, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)kSlicedMaxSmem);
+    if (attr != cudaSuccess) return attr;
+    const size_t Np = ((size_t)N + 3) & ~(size_t)3;
+    const uint32_t *kp = tables, *v2s = tables + Np, *oj = tables + 2 * Np;
+    void *args[] = {(void *)&key, &tag, &idx0, &N, &t, &kp, &v2s, &v1m, &oj, &n, &sparse_out, &addend, &out};
+    return launch_pdl((const void *)k_syndrome_sliced, dim3(count), dim3(kSliceThreads), sliced_smem(N, n, t), s, args);
 }
 
 size_t lane_state_words(uint32_t t, uint32_t L) {

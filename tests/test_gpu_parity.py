@@ -159,6 +159,36 @@ def test_code_tables_sampled_on_device(pv, N):
     ctx.destroy()
 
 
+@pytest.mark.parametrize("K,B,kw", [
+    (6000, 32, {}),                                # a last slice of 2944 positions
+    (6144, 33, dict(t_x=257)),                     # whole slices
+    (6000, 300, dict(scratch_batch=300)),          # more vectors than CTAs at once, lanes' scratch at hand
+    (16001, 40, dict(rate=3, t_x=1)),              # N_x = 48003: ragged tables, odd outputs, one support
+    (8200, 99, {}), (8200, 110, {}),               # lanes and slices, on both sides of the rule
+    (13000, 160, {}),                              # the longest codes that two CTAs per SM hold
+    (15000, 300, dict(scratch_batch=270)),         # beyond them: lanes, in chunks of 270 and 30
+])
+def test_sliced_encode(pv, wl, K, B, kw):
+    """Masks of a large batch on codes longer than one CTA's shared memory."""
+    W = wl.weights_uniform(16, K, K)
+    X = field(wl.int8_vectors(B, K, B))
+    okw = dict(rate=kw.get("rate", 8), **({"t_x": kw["t_x"]} if "t_x" in kw else {}))
+    pp = oracle.PublicParams(W, oracle.key_from_seed(K), with_tables=False, **okw)
+    ctx = pv.pvmvmd_preprocess(to_dev(W), key=K, params=_params(pv, **kw))
+    Xh, st = pv.pvmvmd_encode(ctx, to_dev(X), key=B)
+    Xh, st = pv.as_u32(Xh), pv.as_u32(st)
+    for b in sorted({0, 1, B // 2, B - 2, B - 1}):
+        xh_o, s_o, v_o = pp.encrypt(X[b], oracle.key_from_seed(B), b)
+        assert np.array_equal(Xh[b], xh_o), b
+        assert np.array_equal(st[b], np.concatenate([s_o, v_o])), b
+    # in place, and every vector against a second encoding of the same batch
+    Xi = to_dev(X)
+    pv.pvmvmd_encode(ctx, Xi, key=B, Xhat=Xi)
+    assert np.array_equal(pv.as_u32(Xi), Xh)
+    assert pv.pvmvmd_device_status() == 0
+    ctx.destroy()
+
+
 def test_encode_chunking_matches(pv, wl):
     """Encoding in chunks of 3 vectors (scratch_batch) gives the same result."""
     W = wl.weights_uniform(64, 96, 1)
