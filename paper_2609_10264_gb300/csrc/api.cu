@@ -210,6 +210,7 @@ struct pvmvmd_ctx {
     // streams P^T
     cudaStream_t side = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr;
+    uint32_t *sync = nullptr;  // of the one-kernel decode
     std::vector<void *> owned;
 };
 
@@ -528,7 +529,7 @@ int preprocess_impl(const void *W_dev, bool w16, int m, int K, const pvmvmd_para
     const size_t oF = take(f), oFy = take((size_t)c->ell * c->Ny), ochal = take((size_t)c->ell * 2 * c->t_y),
                  og = take((size_t)c->ell * m), ou = take((size_t)c->ell * K),
                  ostatus = take(2 * scan_status_words(c->Nx, c->sb)),
-                 ostatus_y = take(2 * scan_status_words(c->Ny, c->ell)),
+                 ostatus_y = take(2 * scan_status_words(c->Ny, c->ell)), osync = take(kDecodeSyncWords),
                  oS = take(lanes ? lane_state_words(c->t_x, c->sb) : 0),
                  olaux = take(lanes ? lane_aux_words(c->Nx, c->sb) : 0);
     if (ctx_alloc(c, &small, words) != cudaSuccess || ctx_alloc(c, &c->PT, (size_t)c->Nx * m) != cudaSuccess ||
@@ -541,12 +542,14 @@ int preprocess_impl(const void *W_dev, bool w16, int m, int K, const pvmvmd_para
     c->u = small + ou;
     c->status = reinterpret_cast<unsigned long long *>(small + ostatus);
     c->status_y = reinterpret_cast<unsigned long long *>(small + ostatus_y);
+    c->sync = small + osync;
     if (lanes) {
         c->S = small + oS;
         c->laux = small + olaux;
     }
-    // the tiled syndrome finds its status words zero and leaves them zero
-    if (cudaMemsetAsync(c->status, 0, scan_status_words(c->Nx, c->sb) * sizeof(unsigned long long), s) != cudaSuccess ||
+    // the tiled syndrome and the one-kernel decode find these zero and leave them so
+    if (cudaMemsetAsync(c->sync, 0, kDecodeSyncWords * sizeof(uint32_t), s) != cudaSuccess ||
+        cudaMemsetAsync(c->status, 0, scan_status_words(c->Nx, c->sb) * sizeof(unsigned long long), s) != cudaSuccess ||
         cudaMemsetAsync(c->status_y, 0, scan_status_words(c->Ny, c->ell) * sizeof(unsigned long long), s) !=
             cudaSuccess)
         return fail(PVMVMD_E_CUDA);
@@ -880,6 +883,20 @@ int decode_verify_batch(pvmvmd_ctx *ctx, const void *st_dev, const uint32_t *mas
                         const pvmvmd_key *challenge_key, uint32_t *Y_dev, int32_t *accept_dev,
                         cudaStream_t s) {
     const bool in_place = overlaps(Y_dev, Yhat_dev, (size_t)B * ctx->m * sizeof(uint32_t));
+    if (!in_place && !mask_out_dev && decode_wins(ctx->m, B, ctx->t_x, ctx->t_y, ctx->ell)) {
+        uint32_t *err = error_word();
+        if (!err) return PVMVMD_E_CUDA;
+        const CodeDev &d = ctx->gy;
+        const DecodeCall c{*challenge_key, kTagChallenge, (uint32_t)ctx->Ny, (uint32_t)ctx->t_y, (uint32_t)ctx->ell,
+                           (uint32_t)ctx->rate, (uint32_t)ctx->t_x, (uint32_t)ctx->Nx, d.pi2inv, d.v2p, d.v1m,
+                           d.pi1inv, ctx->Fy, ctx->status_y, err, ctx->sync, ctx->Q, ctx->u, ctx->g, ctx->PT,
+                           static_cast<const uint32_t *>(st_dev), Xhat_dev, Yhat_dev, Y_dev, accept_dev, ctx->m,
+                           ctx->K, B};
+        // the side stream's last use of the scratch was joined to the
+        // caller's stream by the call that made it
+        PV_CUDA(launch_decode(c, s));
+        return PVMVMD_OK;
+    }
     const cudaStream_t cs = in_place ? s : ctx->side;
     if (!in_place) {
         PV_CUDA(cudaEventRecord(ctx->fork, s));

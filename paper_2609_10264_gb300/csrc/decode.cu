@@ -21,6 +21,7 @@
 
 #include "common.cuh"
 #include "launch.h"
+#include "syndrome.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -167,19 +168,17 @@ __device__ __forceinline__ void pe_cols(const uint32_t *__restrict__ PT, int m, 
 // several vectors' supports is read from HBM once and then from L2.
 // ---------------------------------------------------------------------------
 template <bool kBoost, int kDecGroups>
-__global__ void __launch_bounds__(kDecThreads) k_decrypt(const uint32_t *__restrict__ PT, int m,
-                                                        const uint32_t *__restrict__ st, uint32_t t_x,
-                                                        uint32_t Nx, const uint32_t *Yhat, uint32_t *Y,
-                                                        const uint32_t *__restrict__ mask, bool vec) {
+__device__ __forceinline__ void decrypt_cta(const uint32_t *__restrict__ PT, int m, const uint32_t *__restrict__ st,
+                                            uint32_t t_x, uint32_t Nx, const uint32_t *Yhat, uint32_t *Y,
+                                            const uint32_t *__restrict__ mask, bool vec, size_t b, uint32_t yblk) {
     constexpr int kDecColThreads = kDecThreads / kDecGroups;
     constexpr int kDecCols = 4 * kDecColThreads;
     extern __shared__ uint32_t sm[];  // support[t_x], values[t_x]
     __shared__ uint4 s_part[kDecGroups > 1 ? kDecGroups - 1 : 1][kDecColThreads];
     const int tid = threadIdx.x;
-    const size_t b = blockIdx.x;
     const int grp = tid / kDecColThreads, ct = tid % kDecColThreads;
     // boost mode: no rows to split, every thread owns 4 of 1024 columns
-    const int i = kBoost ? ((int)blockIdx.y * kDecThreads + tid) * 4 : (int)blockIdx.y * kDecCols + ct * 4;
+    const int i = kBoost ? ((int)yblk * kDecThreads + tid) * 4 : (int)yblk * kDecCols + ct * 4;
     uint32_t pe[4] = {0u, 0u, 0u, 0u};
     if (!kBoost) {
         const uint32_t *stb = st + b * 2 * t_x;
@@ -225,6 +224,14 @@ __global__ void __launch_bounds__(kDecThreads) k_decrypt(const uint32_t *__restr
         for (int q2 = 0; q2 < 4; ++q2)
             if (i + q2 < m) yo[i + q2] = fsub(yh[i + q2], pe[q2]);
     }
+}
+
+template <bool kBoost, int kDecGroups>
+__global__ void __launch_bounds__(kDecThreads) k_decrypt(const uint32_t *__restrict__ PT, int m,
+                                                        const uint32_t *__restrict__ st, uint32_t t_x,
+                                                        uint32_t Nx, const uint32_t *Yhat, uint32_t *Y,
+                                                        const uint32_t *__restrict__ mask, bool vec) {
+    decrypt_cta<kBoost, kDecGroups>(PT, m, st, t_x, Nx, Yhat, Y, mask, vec, blockIdx.x, blockIdx.y);
 }
 
 // ---------------------------------------------------------------------------
@@ -327,6 +334,169 @@ __global__ void __launch_bounds__(kCheckThreads, 4) k_check(const uint32_t *__re
     if (rank == 0 && tid == 0) accept[b] = ok;
 }
 
+// ---------------------------------------------------------------------------
+// A large decode in one kernel: CTAs of 256 threads, by index
+//   the challenges' tiles and u = e^T Q (syndrome_tile),
+//   g = G_y e from the finished tiles,
+//   the decrypt, all but its last wave of resident CTAs,
+//   the check of one vector each, from u and g,
+//   the rest of the decrypt.
+// A CTA waits only for CTAs of lower index, which the GPU starts first; the
+// verification is done while P^T streams, and nothing is left between two
+// decodes but one launch (a side stream for the verification, forked and
+// joined by events, kept them 6 to 10 us apart).  sync: the finished tiles of
+// each challenge, the finished CTAs of u and g, the finished checks; all zero
+// at launch, and set back, with the tiles' status words, by the last check.
+// ---------------------------------------------------------------------------
+constexpr int kSyncReady = 16, kSyncFinished = 17;
+static_assert(kSyncFinished < kDecodeSyncWords, "sync words");
+
+struct DecodeArgs {
+    TileArgs tile;
+    const uint32_t *pi1inv;
+    uint32_t r, B, tiles, gather, first, decrypt;  // CTAs of each part; `first` of the decrypt's before the checks
+    uint32_t *g;
+    const uint32_t *PT, *st, *Xhat, *Yhat;
+    uint32_t *Y;
+    int m;
+    uint32_t t_x, Nx;
+    int32_t *accept;
+    uint32_t *sync;
+    bool vec;
+};
+
+// The CTA's writes before this are visible to a CTA whose sync_await sees it.
+__device__ __forceinline__ void sync_signal(uint32_t *p) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(p, 1u);
+    }
+}
+__device__ __forceinline__ void sync_await(const uint32_t *p, uint32_t n, uint32_t *err) {
+    if (threadIdx.x == 0) {
+        uint32_t spins = 0;
+        while (ld_acquire_u32(p) < n) {
+            if (++spins > kSpinLimit) {
+                record_error(err, kErrScanTimeout);
+                break;
+            }
+            __nanosleep(64);
+        }
+    }
+    __syncthreads();
+}
+
+// accept_b, by one CTA (as k_check with a cluster of one)
+__device__ __forceinline__ void check_cta(const DecodeArgs &a, uint32_t b) {
+    __shared__ uint32_t s_part[4][kDecThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int K = a.tile.K, m = a.m, n = K > m ? K : m;
+    const uint32_t *xh = a.Xhat + (size_t)b * K, *yh = a.Yhat + (size_t)b * m;
+    int ok = 1;
+    for (uint32_t q = 0; q < a.tile.count; q += 2) {
+        const bool two = q + 1 < a.tile.count;
+        const uint32_t *u0 = a.tile.u + (size_t)q * K, *g0 = a.g + (size_t)q * m;
+        const uint32_t *u1 = two ? u0 + K : u0, *g1 = two ? g0 + m : g0;
+        uint64_t l0 = 0, l1 = 0, r0 = 0, r1 = 0;
+        for (int k0 = tid; k0 < n; k0 += 4 * kDecThreads) {
+            uint32_t x[4], y[4], a0[4], a1[4], c0[4], c1[4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const int k = k0 + v * kDecThreads;
+                const bool kx = k < K, ky = k < m;
+                x[v] = kx ? xh[k] : 0u;
+                a0[v] = kx ? __ldcg(u0 + k) : 0u;
+                a1[v] = kx ? __ldcg(u1 + k) : 0u;
+                y[v] = ky ? yh[k] : 0u;
+                c0[v] = ky ? __ldcg(g0 + k) : 0u;
+                c1[v] = ky ? __ldcg(g1 + k) : 0u;
+            }
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {  // four products and the reduced sum stay below 2^64
+                l0 += (uint64_t)a0[v] * x[v];
+                l1 += (uint64_t)a1[v] * x[v];
+                r0 += (uint64_t)c0[v] * y[v];
+                r1 += (uint64_t)c1[v] * y[v];
+            }
+            l0 = fred(l0);
+            l1 = fred(l1);
+            r0 = fred(r0);
+            r1 = fred(r1);
+        }
+        const uint32_t w[4] = {warp_fsum((uint32_t)l0), warp_fsum((uint32_t)l1), warp_fsum((uint32_t)r0),
+                               warp_fsum((uint32_t)r1)};
+        if (lane == 0)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) s_part[i][warp] = w[i];
+        __syncthreads();
+        if (tid == 0) {
+            uint32_t t[4] = {0u, 0u, 0u, 0u};
+            for (int i = 0; i < 4; ++i)
+                for (int v = 0; v < kDecThreads / 32; ++v) t[i] = fadd(t[i], s_part[i][v]);
+            ok &= (t[0] == t[2]);
+            if (two) ok &= (t[1] == t[3]);
+        }
+        __syncthreads();
+    }
+    if (tid == 0) a.accept[b] = ok;
+}
+
+template <int kDecGroups>
+__global__ void __launch_bounds__(kDecThreads, 4) k_decode(const __grid_constant__ DecodeArgs a) {
+    static_assert(kDecThreads == kScanThreads, "one block size for every part");
+    uint32_t blk = blockIdx.x;
+    const uint32_t ntiles = scan_tiles(a.tile.N), nscan = a.tile.count * ntiles;
+    if (blk < a.tiles) {
+        syndrome_tile(a.tile, blk);
+        sync_signal(a.sync + (blk < nscan ? blk / ntiles : (uint32_t)kSyncReady));
+        return;
+    }
+    blk -= a.tiles;
+    if (blk < a.gather) {
+        const uint32_t per = a.gather / a.tile.count, q = blk / per, j = blk % per * kDecThreads + threadIdx.x;
+        const uint32_t *p = a.pi1inv + (size_t)j * a.r;
+        uint32_t at[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+        if (a.r == 8 && j < (uint32_t)a.m) {
+            const uint4 x = __ldg(reinterpret_cast<const uint4 *>(p)), y = __ldg(reinterpret_cast<const uint4 *>(p + 4));
+            at[0] = x.x; at[1] = x.y; at[2] = x.z; at[3] = x.w;
+            at[4] = y.x; at[5] = y.y; at[6] = y.z; at[7] = y.w;
+        }
+        sync_await(a.sync + q, ntiles, a.tile.err);
+        if (j < (uint32_t)a.m) {
+            const uint32_t *F = a.tile.F + (size_t)q * a.tile.N;
+            uint32_t s = 0;
+            if (a.r == 8) {
+                uint32_t f[8];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) f[c] = __ldcg(F + at[c]);
+#pragma unroll
+                for (int c = 0; c < 8; ++c) s = fadd(s, f[c]);
+            } else {
+                for (uint32_t c = 0; c < a.r; ++c) s = fadd(s, __ldcg(F + __ldg(p + c)));
+            }
+            a.g[(size_t)q * a.m + j] = s;
+        }
+        sync_signal(a.sync + kSyncReady);
+        return;
+    }
+    blk -= a.gather;
+    if (blk >= a.first && blk < a.first + a.B) {
+        __shared__ bool s_last;
+        sync_await(a.sync + kSyncReady, a.tiles - nscan + a.gather, a.tile.err);
+        check_cta(a, blk - a.first);
+        if (threadIdx.x == 0) s_last = atomicAdd(a.sync + kSyncFinished, 1u) == a.B - 1;
+        __syncthreads();
+        if (s_last) {  // every other part that uses them is done
+            for (uint32_t i = threadIdx.x; i < nscan; i += kDecThreads) a.tile.status[i] = 0ull;
+            if (threadIdx.x < kDecodeSyncWords) a.sync[threadIdx.x] = 0u;
+        }
+        return;
+    }
+    if (blk >= a.first) blk -= a.B;
+    decrypt_cta<false, kDecGroups>(a.PT, a.m, a.st, a.t_x, a.Nx, a.Yhat, a.Y, nullptr, a.vec, blk % a.B, blk / a.B);
+}
+
 // out[b][col] = (P e_x,b)_col for the columns of this CTA (1024 per CTA).
 __global__ void __launch_bounds__(kDecThreads) k_output_mask(const uint32_t *__restrict__ PT, int m,
                                                             const uint32_t *__restrict__ st, uint32_t t_x,
@@ -423,20 +593,8 @@ int decrypt_slots() {
     return cache[dev] = per_sm * sms;
 }
 
-cudaError_t launch_decrypt(const uint32_t *PT, int m, const uint32_t *st, uint32_t t_x, uint32_t Nx,
-                           const uint32_t *Yhat, int B, uint32_t *Y, cudaStream_t s, const uint32_t *mask) {
-    if (B <= 0 || m <= 0) return cudaSuccess;
-    const bool vec = (m % 4 == 0) &&
-                     ((reinterpret_cast<uintptr_t>(PT) | reinterpret_cast<uintptr_t>(Yhat) |
-                       reinterpret_cast<uintptr_t>(Y)) & 15u) == 0;
-    const size_t smem = mask ? 0 : 2 * (size_t)t_x * sizeof(uint32_t);
-    if (smem > 48 * 1024) return cudaErrorInvalidValue;
-    const dim3 grid_mask((unsigned)B, (m + 4 * kDecThreads - 1) / (4 * kDecThreads));
-    if (mask) {
-        k_decrypt<true, 2><<<grid_mask, kDecThreads, 0, s>>>(PT, m, nullptr, t_x, Nx, Yhat, Y, mask, vec);
-        note_launch();
-        return cudaGetLastError();
-    }
+// Columns per CTA of a decrypt.
+int decrypt_cols(int m, int B) {
     // Every CTA streams the same t_x row segments, so a last wave that is a
     // third full costs as much as a full one: 256-column CTAs are used when
     // they fill the last wave of resident CTAs clearly better than 512
@@ -453,7 +611,69 @@ cudaError_t launch_decrypt(const uint32_t *PT, int m, const uint32_t *st, uint32
         return waves / std::ceil(waves);
     };
     const bool once = slots > 0 && (double)B * (double)((m + 63) / 64) <= slots;
-    const int cols = once ? 64 : slots > 0 && fill(256) > fill(512) + 0.1 ? 256 : 512;
+    return once ? 64 : slots > 0 && fill(256) > fill(512) + 0.1 ? 256 : 512;
+}
+
+cudaError_t launch_decode(const DecodeCall &c, cudaStream_t s) {
+    const int cols = decrypt_cols(c.m, c.B);
+    const uint32_t ntiles = scan_tiles(c.Ny), ucols = (uint32_t)(c.K + kTileUCols - 1) / kTileUCols;
+    const uint64_t dec = (uint64_t)c.B * ((c.m + cols - 1) / cols);
+    const uint64_t tiles = (uint64_t)c.ell * (ntiles + ucols), gather = (uint64_t)c.ell * ((c.m + 255) / 256);
+    if (tiles + gather + dec + c.B > 0x7fffffffu) return cudaErrorInvalidValue;
+    const size_t smem = 2 * (size_t)c.t_x * sizeof(uint32_t);
+    if (smem > 32 * 1024) return cudaErrorInvalidValue;
+    const DebugWait dbg = debug_wait();
+    const bool inject = dbg.site == PVMVMD_DEBUG_WAIT_SCAN;
+    DecodeArgs a{};
+    a.tile = TileArgs{c.key, c.tag, c.Ny, c.t_y, c.ell, 0, c.pi2inv, c.v2p, c.v1m, nullptr, c.F, c.status, c.err,
+                      inject ? dbg.index : 0xFFFFFFFFu, inject ? (uint32_t)dbg.limit : kSpinLimit, c.Q, c.K, ucols, c.u};
+    a.pi1inv = c.pi1inv;
+    a.r = c.r;
+    a.B = (uint32_t)c.B;
+    a.tiles = (uint32_t)tiles;
+    a.gather = (uint32_t)gather;
+    a.decrypt = (uint32_t)dec;
+    a.first = dec > (uint64_t)decrypt_slots() ? (uint32_t)(dec - decrypt_slots()) : 0u;
+    a.g = c.g;
+    a.PT = c.PT;
+    a.st = c.st;
+    a.Xhat = c.Xhat;
+    a.Yhat = c.Yhat;
+    a.Y = c.Y;
+    a.m = c.m;
+    a.t_x = c.t_x;
+    a.Nx = c.Nx;
+    a.accept = c.accept;
+    a.sync = c.sync;
+    a.vec = c.m % 4 == 0 && ((reinterpret_cast<uintptr_t>(c.PT) | reinterpret_cast<uintptr_t>(c.Yhat) |
+                              reinterpret_cast<uintptr_t>(c.Y)) & 15u) == 0;
+    const auto kern = cols == 256 ? k_decode<4> : k_decode<2>;
+    kern<<<a.tiles + a.gather + a.decrypt + a.B, kDecThreads, smem, s>>>(a); note_launch();
+    return cudaGetLastError();
+}
+
+bool decode_wins(int m, int B, uint32_t t_x, uint32_t t_y, uint32_t ell) {
+    // a decrypt of more than one wave of resident CTAs
+    const int cols = decrypt_cols(m, B), slots = decrypt_slots();
+    return slots > 0 && cols > 64 && syndrome_tiles_eligible(t_y) && ell <= 16 && 2 * t_x * 4 <= 32 * 1024 &&
+           (uint64_t)B * ((m + cols - 1) / cols) > (uint64_t)slots;
+}
+
+cudaError_t launch_decrypt(const uint32_t *PT, int m, const uint32_t *st, uint32_t t_x, uint32_t Nx,
+                           const uint32_t *Yhat, int B, uint32_t *Y, cudaStream_t s, const uint32_t *mask) {
+    if (B <= 0 || m <= 0) return cudaSuccess;
+    const bool vec = (m % 4 == 0) &&
+                     ((reinterpret_cast<uintptr_t>(PT) | reinterpret_cast<uintptr_t>(Yhat) |
+                       reinterpret_cast<uintptr_t>(Y)) & 15u) == 0;
+    const size_t smem = mask ? 0 : 2 * (size_t)t_x * sizeof(uint32_t);
+    if (smem > 48 * 1024) return cudaErrorInvalidValue;
+    const dim3 grid_mask((unsigned)B, (m + 4 * kDecThreads - 1) / (4 * kDecThreads));
+    if (mask) {
+        k_decrypt<true, 2><<<grid_mask, kDecThreads, 0, s>>>(PT, m, nullptr, t_x, Nx, Yhat, Y, mask, vec);
+        note_launch();
+        return cudaGetLastError();
+    }
+    const int cols = decrypt_cols(m, B);
     if ((m + cols - 1) / cols > 65535) return cudaErrorInvalidValue;
     const dim3 grid((unsigned)B, (m + cols - 1) / cols);
     if (cols == 64)

@@ -220,6 +220,27 @@ cudaError_t launch_verify_u(const uint32_t *Qm, int K, const uint32_t *chal, uin
 cudaError_t launch_decrypt(const uint32_t *PT, int m, const uint32_t *st, uint32_t t_x, uint32_t Nx,
                            const uint32_t *Yhat, int B, uint32_t *Y, cudaStream_t s,
                            const uint32_t *mask = nullptr);
+// Verify and decrypt of a large batch in one kernel (see k_decode), where
+// decode_wins; sync: kDecodeSyncWords words, zero at the call and after it;
+// status as for launch_syndrome_tiles.  Y must not overlap Yhat.
+constexpr int kDecodeSyncWords = 32;
+struct DecodeCall {
+    pvmvmd_key key;
+    uint32_t tag, Ny, t_y, ell, r, t_x, Nx;
+    const uint32_t *pi2inv, *v2p, *v1m, *pi1inv;
+    uint32_t *F;
+    unsigned long long *status;
+    uint32_t *err, *sync;
+    const uint32_t *Q;
+    uint32_t *u, *g;
+    const uint32_t *PT, *st, *Xhat, *Yhat;
+    uint32_t *Y;
+    int32_t *accept;
+    int m, K, B;
+};
+bool decode_wins(int m, int B, uint32_t t_x, uint32_t t_y, uint32_t ell);
+cudaError_t launch_decode(const DecodeCall &c, cudaStream_t s);
+
 // Verify: accept[b] = AND_q (u_q . Xhat[b] == g_q . Yhat[b]) for the ell
 // challenges' u (ell x K) and g (ell x m).
 cudaError_t launch_check(const uint32_t *Xhat, int K, const uint32_t *Yhat, int m, const uint32_t *g,

@@ -884,6 +884,61 @@ def test_server_mvm_grouped_small_batches(pv, specs):
     assert pv.pvmvmd_device_status() == 0
 
 
+@pytest.mark.parametrize("m,K,B,kw", [
+    (300, 96, 700, {}),                            # more vectors than CTAs at once
+    (1030, 1001, 310, {}),                         # unaligned rows of P^T
+    (683, 64, 500, dict(rate=3, ell=3, t_y=1)),    # N_y = 2049, an odd number of challenges
+    (4096, 520, 100, dict(t_y=256, ell=1)),        # 256-column CTAs
+    (2048, 96, 300, dict(ell=16)),                 # the most challenges
+])
+def test_large_decode_in_one_kernel(pv, wl, m, K, B, kw):
+    """Decodes whose decrypt is more than one wave of CTAs run in one kernel:
+    outputs and verdicts exact, also after smaller and in-place decodes of the
+    same context and when a captured call is replayed."""
+    import torch
+    W = wl.weights_uniform(m, K, m + K)
+    x = wl.int8_vectors(B, K, B)
+    Wd = to_dev(W)
+    ctx = pv.pvmvmd_preprocess(Wd, key=41, params=_params(pv, **kw))
+    Xh, st = pv.pvmvmd_encode(ctx, to_dev(field(x)), key=42)
+    Yh = pv.pvmvmd_server_mvm(Wd, Xh)
+    exp = field(exact_product(W, x))
+    bad = Yh.clone()
+    wrong = sorted({0, B // 3, B - 1})
+    for b in wrong:
+        tamper(pv, bad, b, (7 * b) % m, 1 + b)
+    ok = np.ones(B, np.int32)
+    ok_bad = ok.copy()
+    ok_bad[wrong] = 0
+    n0 = pv.pvmvmd_kernel_launches()
+    Y, acc = pv.pvmvmd_decode_verify(ctx, st, Xh, Yh, challenge_key=43)
+    assert pv.pvmvmd_kernel_launches() - n0 == 1
+    assert_equal_report(pv.as_u32(Y), exp, "y")
+    assert np.array_equal(acc.cpu().numpy(), ok)
+    few, acc_few = pv.pvmvmd_decode_verify(ctx, st[:3].contiguous(), Xh[:3].contiguous(), bad[:3].contiguous(), 44)
+    assert_equal_report(pv.as_u32(few)[1:], exp[1:3], "three vectors")
+    assert acc_few.tolist() == [0, 1, 1]
+    _, acc_bad = pv.pvmvmd_decode_verify(ctx, st, Xh, bad, challenge_key=45)
+    assert np.array_equal(acc_bad.cpu().numpy(), ok_bad)
+    Yip = bad.clone()
+    _, acc_ip = pv.pvmvmd_decode_verify(ctx, st, Xh, Yip, challenge_key=46, Y=Yip)
+    assert np.array_equal(acc_ip.cpu().numpy(), ok_bad)
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    Yg, accg = torch.zeros_like(Y), torch.full_like(acc, 7)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        pv.pvmvmd_decode_verify(ctx, st, Xh, Yh, challenge_key=47, Y=Yg, accept=accg, stream=s)
+    for _ in range(3):
+        Yg.zero_()
+        accg.fill_(7)
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(Yg, Y) and np.array_equal(accg.cpu().numpy(), ok)
+    assert pv.pvmvmd_device_status() == 0
+    ctx.destroy()
+
+
 def test_decode_with_foreign_state_stays_in_bounds(pv, wl):
     """A mask state the encode did not write (support indices at and past
     N_x) gives wrong outputs for that vector only: every read stays inside
