@@ -223,7 +223,7 @@ struct pvmvmd_bv_ctx {
     uint32_t *QauxT = nullptr; // N' x N: Qaux transposed
     uint32_t *Yt = nullptr, *Z = nullptr;  // m x B, N x B
     uint32_t *chal2 = nullptr, *R = nullptr, *F2 = nullptr;
-    uint32_t *eS = nullptr, *eticket = nullptr;  // encode scratch: S, scan ticket
+    uint32_t *eS = nullptr;                      // encode scratch: S
     unsigned long long *estatus = nullptr;       // and scan status words
     unsigned long long *status = nullptr;
     std::vector<void *> owned;
@@ -275,33 +275,35 @@ int sample_codes(Ctx *c, const pvmvmd_key &key, CodeDev *const code[2], const in
 // Y (N x L lanes, row stride ldy) = G^T applied to the L lanes of X (n x L,
 // row stride ldx; row i holds message entry i of every lane), in lane chunks.
 // One chunk of lanes with caller-provided scratch (S: N x nl; status:
-// encode_scan_status_words(N, nl) 64-bit words; ticket: one word); no
+// encode_scan_status_words(N, nl) 64-bit words); no
 // allocation, no sync.
 int encode_lanes_into(const CodeDev &d, uint32_t n, uint32_t r, const void *X, bool x_is_i8, size_t ldx,
                       uint32_t nl, uint32_t *Y, size_t ldy, uint32_t *S, unsigned long long *status,
-                      uint32_t *ticket, uint32_t *err, cudaStream_t s) {
+                      uint32_t *err, cudaStream_t s) {
     const uint32_t N = n * r;
-    cudaError_t e = encode_scan_clear(status, ticket, N, nl, s);
+    cudaError_t e = encode_scan_clear(status, N, nl, s);
     if (e == cudaSuccess)  // S = A^T V1 Pi1^T R^T X
-        e = launch_encode_scan(X, x_is_i8, ldx, d.pi1, r, d.v1m, N, nl, S, nl, status, ticket, err, s);
-    if (e == cudaSuccess) e = encode_scan_clear(status, ticket, N, nl, s);
+        e = launch_encode_scan(X, x_is_i8, ldx, d.pi1, r, d.v1m, N, nl, S, nl, status, err, s);
+    if (e == cudaSuccess) e = encode_scan_clear(status, N, nl, s);
     if (e == cudaSuccess)  // Y = A^T V2 Pi2^T S
-        e = launch_encode_scan(S, false, nl, d.pi2, 1, d.v2m, N, nl, Y, ldy, status, ticket, err, s);
+        e = launch_encode_scan(S, false, nl, d.pi2, 1, d.v2m, N, nl, Y, ldy, status, err, s);
     return e == cudaSuccess ? PVMVMD_OK : PVMVMD_E_CUDA;
 }
 
 // Scratch of encode_lanes, allocated once for all the encodings of a
 // preprocessing (a 512 MiB cudaMalloc and cudaFree take 0.44 ms).
 struct LaneScratch {
-    uint32_t *S = nullptr, *ticket = nullptr;
+    uint32_t *S = nullptr;
     unsigned long long *status = nullptr;
     ~LaneScratch() {
         cudaFree(S);
         cudaFree(status);
-        cudaFree(ticket);
     }
-    static size_t lanes(uint32_t N, uint32_t L) {  // lanes per chunk: about 1 GiB of S
-        size_t lc = ((size_t)1 << 28) / N / 256 * 256;
+    // lanes per chunk: about 256 MiB of S (at 4096 x 4096 0.1 ms less to
+    // allocate and free than 512 MiB, at the same speed), 2048 lanes up to 1 GiB
+    static size_t lanes(uint32_t N, uint32_t L) {
+        const size_t few = ((size_t)1 << 26) / N, most = ((size_t)1 << 28) / N;
+        size_t lc = std::max(few, std::min<size_t>(2048, most)) / 256 * 256;
         if (lc < 256) lc = 256;
         return lc < L ? lc : L;
     }
@@ -313,8 +315,7 @@ struct LaneScratch {
             s = std::max(s, (size_t)u.first * lc);
             w = std::max(w, encode_scan_status_words(u.first, (uint32_t)lc));
         }
-        return dev_alloc(&S, s) == cudaSuccess && dev_alloc(&status, w) == cudaSuccess &&
-                       dev_alloc(&ticket, 1) == cudaSuccess
+        return dev_alloc(&S, s) == cudaSuccess && dev_alloc(&status, w) == cudaSuccess
                    ? PVMVMD_OK
                    : PVMVMD_E_NOMEM;
     }
@@ -330,7 +331,7 @@ int encode_lanes(const CodeDev &d, uint32_t n, uint32_t r, const void *X, bool x
         const uint32_t nl = (uint32_t)((L - l0) < lc ? (L - l0) : lc);
         const void *Xl = x_is_i8 ? static_cast<const void *>(static_cast<const int8_t *>(X) + l0)
                                  : static_cast<const void *>(static_cast<const uint32_t *>(X) + l0);
-        const int st = encode_lanes_into(d, n, r, Xl, x_is_i8, ldx, nl, Y + l0, ldy, sc.S, sc.status, sc.ticket, err, s);
+        const int st = encode_lanes_into(d, n, r, Xl, x_is_i8, ldx, nl, Y + l0, ldy, sc.S, sc.status, err, s);
         if (st != PVMVMD_OK) return st;
     }
     return PVMVMD_OK;
@@ -939,17 +940,16 @@ int pvmvmd_boost_decode_verify(pvmvmd_ctx *ctx, const uint32_t *mask_out_dev,
 namespace pv {
 namespace {
 // Scratch of pvmvmd_code_encode_lanes: S (N x L), the scan's 64-bit status
-// words and its ticket word, each at a 16-byte aligned offset.
+// words, each at a 16-byte aligned offset.
 struct EncodeScratch {
-    size_t s_off, status_off, ticket_off, bytes;
+    size_t s_off, status_off, bytes;
 };
 EncodeScratch encode_scratch_layout(uint32_t N, uint32_t L) {
     auto up = [](size_t b) { return (b + 15) & ~(size_t)15; };
     EncodeScratch e;
     e.s_off = 0;
     e.status_off = up((size_t)N * L * 4);
-    e.ticket_off = e.status_off + up(encode_scan_status_words(N, L) * 8);
-    e.bytes = e.ticket_off + 16;
+    e.bytes = e.status_off + up(encode_scan_status_words(N, L) * 8);
     return e;
 }
 }  // namespace
@@ -976,8 +976,7 @@ int pvmvmd_code_encode_lanes(const pvmvmd_ctx *ctx, int which, const uint32_t *X
     uint8_t *base = static_cast<uint8_t *>(scratch_dev);
     return encode_lanes_into(d, n, (uint32_t)ctx->rate, X_dev, false, (size_t)L, (uint32_t)L, Y_dev, (size_t)L,
                              reinterpret_cast<uint32_t *>(base + lay.s_off),
-                             reinterpret_cast<unsigned long long *>(base + lay.status_off),
-                             reinterpret_cast<uint32_t *>(base + lay.ticket_off), err,
+                             reinterpret_cast<unsigned long long *>(base + lay.status_off), err,
                              static_cast<cudaStream_t>(stream));
 }
 
@@ -1097,7 +1096,6 @@ int pvmvmd_bv_preprocess(const int8_t *W_dev, int B, int m, int n, const pvmvmd_
         ctx_alloc(c, &c->R, (size_t)ell2 * Bn) != cudaSuccess ||
         ctx_alloc(c, &c->F2, (size_t)ell2 * N2) != cudaSuccess ||
         ctx_alloc(c, &c->eS, (size_t)N * B) != cudaSuccess || ctx_alloc(c, &c->estatus, sw) != cudaSuccess ||
-        ctx_alloc(c, &c->eticket, 1) != cudaSuccess ||
         ctx_alloc(c, &c->status, scan_status_words((uint32_t)N2, (uint32_t)ell2)) != cudaSuccess)
         return fail(PVMVMD_E_NOMEM);
     if (cudaMemsetAsync(c->status, 0, scan_status_words((uint32_t)N2, (uint32_t)ell2) * sizeof(unsigned long long),
@@ -1150,7 +1148,7 @@ int pvmvmd_bv_check(pvmvmd_bv_ctx *ctx, const uint32_t *X_dev, const uint32_t *Y
     // z_b = G^T y_b (the B outputs as lanes)
     PV_CUDA(launch_transpose_u32(Y_dev, ctx->B, ctx->m, ctx->Yt, s));
     int st = encode_lanes_into(ctx->g, (uint32_t)ctx->m, (uint32_t)ctx->rate, ctx->Yt, false, (size_t)ctx->B,
-                               (uint32_t)ctx->B, ctx->Z, (size_t)ctx->B, ctx->eS, ctx->estatus, ctx->eticket,
+                               (uint32_t)ctx->B, ctx->Z, (size_t)ctx->B, ctx->eS, ctx->estatus,
                                err, s);
     if (st) return st;
     // secondary challenges, drawn after the responses, and r^(j) = G' e'^(j)

@@ -737,8 +737,7 @@ __global__ void __launch_bounds__(1024) k_slice_tables(const uint32_t *__restric
 // holds a state in its high half (1: the tile's own sum, 2: the inclusive
 // prefix through the tile) and the value in its low half, so a reader gets
 // state and value in one load and no fence or block barrier is needed.
-// Tiles are numbered in the order CTAs start (a global ticket), so every
-// predecessor of a tile is already running.  (The earlier form, one flag per
+// A tile's predecessors are CTAs of lower index, which the GPU starts first.  (The earlier form, one flag per
 // tile and the lanes' values in separate arrays behind a fence and block
 // barriers, with warp 0 reading 32 flags at a time, took 0.755 ms per
 // 4096 x 4096 encoding.)  At 32 positions per tile the kernel is held to 64
@@ -757,21 +756,12 @@ __global__ void __launch_bounds__(256, 4) k_encode_scan(const void *__restrict__
                                                     const uint32_t *__restrict__ perm, uint32_t div,
                                                     const uint32_t *__restrict__ vscale_m, uint32_t N,
                                                     uint32_t L, uint32_t *__restrict__ Y, size_t ldy,
-                                                    unsigned long long *status, uint32_t *ticket_ctr,
-                                                    uint32_t *__restrict__ err) {
-    __shared__ uint32_t s_ticket;
+                                                    unsigned long long *status, uint32_t *__restrict__ err) {
     __shared__ ulonglong2 s_row[kEncTile];  // byte offset of the source row and scale of each position
     const int tid = threadIdx.x;
     const uint32_t nlb = (L + 255) / 256;
     const uint32_t ntiles = (N + kEncTile - 1) / kEncTile;
-    if (tid == 0) s_ticket = atomicAdd(ticket_ctr, 1u);
-    __syncthreads();
-    const uint32_t ticket = s_ticket;
-    if (ticket >= nlb * ntiles) {  // ticket not cleared: never index past the data
-        if (tid == 0) record_error(err, kErrScanTimeout);
-        return;
-    }
-    const uint32_t tile = ticket / nlb, lb = ticket % nlb;
+    const uint32_t tile = blockIdx.x / nlb, lb = blockIdx.x % nlb;
     const uint32_t l = lb * 256 + tid;
     const bool lane_ok = l < L;
     const uint32_t j0 = tile * kEncTile;
@@ -1353,26 +1343,23 @@ size_t encode_scan_status_words(uint32_t N, uint32_t L) {
     return (size_t)((L + 255) / 256) * ((N + kEncTile - 1) / kEncTile) * 256;
 }
 
-cudaError_t encode_scan_clear(unsigned long long *status, uint32_t *ticket, uint32_t N, uint32_t L,
-                              cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(status, 0, encode_scan_status_words(N, L) * sizeof(unsigned long long), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(ticket, 0, sizeof(uint32_t), s);
-    return e;
+cudaError_t encode_scan_clear(unsigned long long *status, uint32_t N, uint32_t L, cudaStream_t s) {
+    return cudaMemsetAsync(status, 0, encode_scan_status_words(N, L) * sizeof(unsigned long long), s);
 }
 
 cudaError_t launch_encode_scan(const void *X, bool x_is_i8, size_t ldx, const uint32_t *perm,
                                uint32_t div, const uint32_t *vscale_m, uint32_t N, uint32_t L,
-                               uint32_t *Y, size_t ldy, unsigned long long *status, uint32_t *ticket,
-                               uint32_t *err, cudaStream_t s) {
+                               uint32_t *Y, size_t ldy, unsigned long long *status, uint32_t *err,
+                               cudaStream_t s) {
     const size_t ctas = encode_scan_status_words(N, L) / 256;
     if (ctas == 0) return cudaSuccess;
     if (ctas > 0x7fffffffu) return cudaErrorInvalidValue;
     if (x_is_i8)
         k_encode_scan<true><<<(unsigned)ctas, 256, 0, s>>>(X, ldx, perm, div, vscale_m, N, L, Y, ldy,
-                                                           status, ticket, err);
+                                                           status, err);
     else
         k_encode_scan<false><<<(unsigned)ctas, 256, 0, s>>>(X, ldx, perm, div, vscale_m, N, L, Y, ldy,
-                                                            status, ticket, err);
+                                                            status, err);
     note_launch();
     return cudaGetLastError();
 }
