@@ -30,8 +30,15 @@ namespace {
 
 constexpr int kDecThreads = 256;
 
+// A row of P^T is read once by a CTA, so L1 would only be filled in vain
+// (decode of 4096 x 4096, 100 vectors: 45.1 -> 41.2 us without; asking L2 for
+// 256 bytes at a time 43.0).
 __device__ __forceinline__ uint4 ldg4(const uint32_t *p) {
-    return __ldg(reinterpret_cast<const uint4 *>(p));
+    uint4 v;
+    asm("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+        : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+        : "l"(p));
+    return v;
 }
 
 // u[q][k] = sum_j chal_val[q][j] Q[chal_supp[q][j]][k]: a CTA covers 64
