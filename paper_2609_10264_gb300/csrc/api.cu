@@ -211,6 +211,8 @@ struct pvmvmd_ctx {
     cudaStream_t side = nullptr;
     cudaEvent_t fork = nullptr, join = nullptr;
     uint32_t *sync = nullptr;  // of the one-kernel decode
+    // the last verification ran on a caller's stream; a call was captured
+    bool on_caller = false, captured = false;
     std::vector<void *> owned;
 };
 
@@ -842,11 +844,10 @@ int pvmvmd_server_mvm_grouped(const pvmvmd_mvm_batch_job *jobs, int count, void 
 
 namespace pv {
 namespace {
-// The verification of a call: challenges e_q <- E_{t_y}^{N_y} shared by the
-// B vectors, g_q = G_y e_q, u_q = e_q^T Q, and accept_b from x_hat_b and
-// y_hat_b, all on stream cs.
-int verify_chain(pvmvmd_ctx *ctx, const pvmvmd_key *challenge_key, const uint32_t *Xhat_dev,
-                 const uint32_t *Yhat_dev, int B, int32_t *accept_dev, cudaStream_t cs) {
+// The challenges of a call: e_q <- E_{t_y}^{N_y}, shared by its vectors, and
+// g_q = G_y e_q, u_q = e_q^T Q from them, on stream cs.  They rest on the key and
+// the context alone.
+int challenge_chain(pvmvmd_ctx *ctx, const pvmvmd_key *challenge_key, cudaStream_t cs) {
     uint32_t *err = error_word();
     if (!err) return PVMVMD_E_CUDA;
     const CodeDev &d = ctx->gy;
@@ -863,8 +864,6 @@ int verify_chain(pvmvmd_ctx *ctx, const pvmvmd_key *challenge_key, const uint32_
                                        ctx->ell, cs));
         PV_CUDA(launch_verify_u(ctx->Q, ctx->K, ctx->chal, ctx->t_y, ctx->ell, ctx->u, cs));
     }
-    PV_CUDA(launch_check(Xhat_dev, ctx->K, Yhat_dev, ctx->m, ctx->g, ctx->u, (uint32_t)ctx->ell, B,
-                         accept_dev, cs));
     return PVMVMD_OK;
 }
 
@@ -874,15 +873,28 @@ bool overlaps(const void *a, const void *b, size_t bytes) {
 }
 
 // Verify and decrypt: Y = Yhat - P e_x from st, or Y = Yhat - mask_out when
-// mask_out is given (boost mode).  The verification depends on the key,
-// x_hat and y_hat but not on Y, so it runs on the context's side stream
-// while the decrypt streams P^T on the caller's stream; the caller's stream
-// then waits for the side stream.  When Y overwrites Yhat the verification
-// must read Yhat first, and both run in order on the caller's stream.
+// mask_out is given (boost mode).
+//  * A large decrypt: one kernel on the caller's stream (launch_decode).
+//  * Else the verification runs on the context's side stream while the
+//    decrypt runs on the caller's, which then waits for the side stream.
+//    Only the check reads what the caller's stream produced, so only it waits
+//    for that stream: the challenges are formed while, say, the server's
+//    product still runs (round trip of 1030 x 1001, 70 vectors 36.5 -> 29 us).
+//    Their scratch is free by then, since every earlier verification ran on
+//    the side stream too -- or on a caller's stream, as a replay of a captured
+//    call also does: then they wait as well.
+//  * When Y overwrites Yhat the verification must read Yhat first, and both
+//    run in order on the caller's stream.
 int decode_verify_batch(pvmvmd_ctx *ctx, const void *st_dev, const uint32_t *mask_out_dev,
                         const uint32_t *Xhat_dev, const uint32_t *Yhat_dev, int B,
                         const pvmvmd_key *challenge_key, uint32_t *Y_dev, int32_t *accept_dev,
                         cudaStream_t s) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) {  // the legacy stream, while another is captured
+        (void)cudaGetLastError();
+        capture = cudaStreamCaptureStatusActive;
+    }
+    if (capture != cudaStreamCaptureStatusNone) ctx->captured = true;
     const bool in_place = overlaps(Y_dev, Yhat_dev, (size_t)B * ctx->m * sizeof(uint32_t));
     if (!in_place && !mask_out_dev && decode_wins(ctx->m, B, ctx->t_x, ctx->t_y, ctx->ell)) {
         uint32_t *err = error_word();
@@ -895,16 +907,24 @@ int decode_verify_batch(pvmvmd_ctx *ctx, const void *st_dev, const uint32_t *mas
                            ctx->K, B};
         // the side stream's last use of the scratch was joined to the
         // caller's stream by the call that made it
+        ctx->on_caller = true;
         PV_CUDA(launch_decode(c, s));
         return PVMVMD_OK;
     }
     const cudaStream_t cs = in_place ? s : ctx->side;
+    int st = PVMVMD_OK;
     if (!in_place) {
+        const bool early = !ctx->captured && !ctx->on_caller;
+        if (early && (st = challenge_chain(ctx, challenge_key, cs))) return st;
         PV_CUDA(cudaEventRecord(ctx->fork, s));
-        PV_CUDA(cudaStreamWaitEvent(ctx->side, ctx->fork, 0));
+        PV_CUDA(cudaStreamWaitEvent(cs, ctx->fork, 0));
+        if (!early && (st = challenge_chain(ctx, challenge_key, cs))) return st;
+        ctx->on_caller = false;
+    } else {
+        ctx->on_caller = true;
+        if ((st = challenge_chain(ctx, challenge_key, cs))) return st;
     }
-    int st = verify_chain(ctx, challenge_key, Xhat_dev, Yhat_dev, B, accept_dev, cs);
-    if (st) return st;
+    PV_CUDA(launch_check(Xhat_dev, ctx->K, Yhat_dev, ctx->m, ctx->g, ctx->u, (uint32_t)ctx->ell, B, accept_dev, cs));
     PV_CUDA(launch_decrypt(ctx->PT, ctx->m, static_cast<const uint32_t *>(st_dev), ctx->t_x, (uint32_t)ctx->Nx,
                            Yhat_dev, B, Y_dev, s, mask_out_dev));
     if (!in_place) {

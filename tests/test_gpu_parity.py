@@ -939,6 +939,58 @@ def test_large_decode_in_one_kernel(pv, wl, m, K, B, kw):
     ctx.destroy()
 
 
+def test_decodes_of_every_route_in_turn(pv, wl):
+    """Decodes of one context that take the side stream, the caller's stream (Y
+    over Y_hat), one kernel (a large batch), boost mode and a captured graph,
+    queued one after the other without a wait: the challenges' shared scratch
+    is handed from one to the next, and every output and verdict is exact."""
+    import torch
+    m, K, B = 600, 520, 400
+    W = wl.weights_uniform(m, K, 81)
+    x = wl.int8_vectors(B, K, 82)
+    Wd = to_dev(W)
+    ctx = pv.pvmvmd_preprocess(Wd, key=83)
+    Xh, st = pv.pvmvmd_encode(ctx, to_dev(field(x)), key=84)
+    Yh = pv.pvmvmd_server_mvm(Wd, Xh)
+    bad = Yh.clone()
+    tamper(pv, bad, 1, 17, 5)
+    mask_in, mask_out, _ = pv.pvmvmd_boost_prepare(ctx, B, key=84)
+    exp = to_dev(field(exact_product(W, x)))
+    exp_bad = pv.pvmvmd_decode_verify(ctx, st, Xh, bad, 85)[0]
+    small = [t[:4].contiguous() for t in (st, Xh, bad)]
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    Yg, ag = torch.empty((4, m), dtype=torch.int32, device="cuda"), torch.empty(4, dtype=torch.int32, device="cuda")
+    graph = None
+    for turn in range(3):
+        got = []
+        for i in range(40):
+            key = 100 + 50 * turn + i
+            if i % 5 == 0:
+                got.append((4, *pv.pvmvmd_decode_verify(ctx, *small, key)))
+            elif i % 5 == 1:
+                Yip = small[2].clone()
+                got.append((4, *pv.pvmvmd_decode_verify(ctx, *small, key, Y=Yip)) if i % 2 else
+                           (4, Yip, pv.pvmvmd_decode_verify(ctx, small[0], small[1], Yip, key, Y=Yip)[1]))
+            elif i % 5 == 2:
+                got.append((B, *pv.pvmvmd_decode_verify(ctx, st, Xh, bad, key)))
+            elif i % 5 == 3:
+                got.append((4, *pv.pvmvmd_boost_decode_verify(ctx, mask_out[:4].contiguous(), small[1], small[2], key)))
+            elif graph is not None:
+                graph.replay()
+                got.append((4, Yg.clone(), ag.clone()))
+        torch.cuda.synchronize()
+        for k, Y, acc in got:
+            assert torch.equal(Y, exp_bad[:k]) and torch.equal(Y[0], exp[0])
+            assert acc.tolist() == [0 if b == 1 else 1 for b in range(k)]
+        if turn == 0:  # from the second turn on with a captured call among them
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=s):
+                pv.pvmvmd_decode_verify(ctx, *small, 77, Y=Yg, accept=ag, stream=s)
+    assert pv.pvmvmd_device_status() == 0
+    ctx.destroy()
+
+
 def test_decode_with_foreign_state_stays_in_bounds(pv, wl):
     """A mask state the encode did not write (support indices at and past
     N_x) gives wrong outputs for that vector only: every read stays inside
