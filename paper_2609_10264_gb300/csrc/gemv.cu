@@ -301,6 +301,12 @@ __global__ void __launch_bounds__(kRingThreads, 2) k_gemv_ring(const __grid_cons
 #pragma unroll
         for (int d = 0; d < kRingBatches; ++d) load(ring + d * kBatchBytes);
         if (!waited) {
+            // x_hat may only be read after the wait; L2 may fetch it before
+            // (eight 8B-class layers 338.5 -> 334.7 us)
+#pragma unroll
+            for (int i = 0; i < CH; ++i)
+                if (grp == 0 && ct + i * T < nchunks)
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(job.xhat + (size_t)(ct + i * T) * 16));
             asm volatile("griddepcontrol.wait;" ::: "memory");
             waited = true;
         }
