@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(kGemvThreads, 1)
 // ---------------------------------------------------------------------------
 // Grouped persistent kernel: one launch computes a list of independent batch-1
 // products (jobs), each streaming its own matrix once.  One CTA of 512 threads
-// per SM takes whole rows: of one job where a few jobs split evenly over the
+// per SM (two for large products) takes whole rows: of one job where a few jobs split evenly over the
 // CTAs (the rows then run without a break), else an even share of all the
 // bytes, job after job.
 //
@@ -195,9 +195,9 @@ __global__ void __launch_bounds__(kGemvThreads, 1)
 //
 // Against a kernel with the digit planes in shared memory, M in registers and
 // two CTAs of 128 registers per SM: eight 8B-class layers of four dependent
-// launches 402 -> 338 us (5.18 TB/s), 100 requests of 4096 x 4096 252 -> 236
-// us (7.1 TB/s); dependent single calls, 4096 x 4096 5.8 -> 4.7 us, 4096 x
-// 14336 14.1 -> 11.0, 50000 x 64 15.0 -> 5.0, 256 x 256 2.05 -> 1.99.  Asking
+// launches 402 -> 322 us (5.4 TB/s), 100 requests of 4096 x 4096 252 -> 231
+// us (7.3 TB/s); dependent single calls, 4096 x 4096 5.8 -> 4.6 us, 4096 x
+// 14336 14.1 -> 12.0, 50000 x 64 15.0 -> 5.0, 256 x 256 2.05 -> 1.9.  Asking
 // L2 for more of M before the wait made a token slower (362 -> 378 us and up).
 // ---------------------------------------------------------------------------
 constexpr int kRingThreads = 512;
@@ -206,6 +206,7 @@ constexpr int kRingSlots = 4;    // 16-byte slots per thread and batch
 constexpr int kRingSumRows = 16 * (kRingThreads / 32);  // rows per block-wide reduction
 constexpr int kRingFewJobs = 8;
 constexpr int kRingMinBytes = 16384;  // of M per CTA (1024 x 1024: 2.4 us; 8 KiB 2.8, 64 KiB 2.7)
+constexpr long long kRingPairBytes = 256 << 10;  // of M per SM from which an SM takes two CTAs
 constexpr int kRingSmem = kRingThreads * kRingBatches * kRingSlots * 16;
 
 template <int NJ>
@@ -423,9 +424,21 @@ cudaError_t run_gemv_ring(const MvmJob *jobs, int count, cudaStream_t s) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    // one CTA per SM where every CTA gets enough of M
+    // One CTA per SM where every CTA gets enough of M, so that the next
+    // launch's fill their rings beside it; two for a few jobs that are large.
+    // Two are placed evenly whatever ran before (every slot of an SM takes
+    // one), one need not be: a launch that comes while the one before it ends,
+    // as the second after a pause does, puts two CTAs on the SMs that are
+    // empty, and the launches that depend on it inherit that (a token through
+    // eight 8B-class layers after a pause: 356 or 485 us by turns, now 348; back
+    // to back 346 -> 336).  Below the line the rings hold much of the share
+    // and the overlap is worth more (dependent single calls, two CTAs against
+    // one: 8192 x 4096 8.3 and 6.8 us, 6144 x 6144 8.0 and 7.6; above it
+    // 4096 x 14336 12.0 and 10.9, 8192 x 8192 11.0 and 11.6, gate and up of
+    // 14336 x 4096 17.3 and 18.7; 100 requests 249 and 237).
     const long long total = args.base[count];
-    const int grid = (int)std::max(1LL, std::min({(long long)sms, rows, total / kRingMinBytes}));
+    const long long slots = count <= kRingFewJobs && total >= sms * kRingPairBytes ? 2LL * sms : sms;
+    const int grid = (int)std::max(1LL, std::min({slots, rows, total / kRingMinBytes}));
     args.split = 0;
     if (count <= kRingFewJobs && count * 8 <= grid) {
         // CTAs for each job, where that splits the bytes within 12 % of evenly

@@ -682,6 +682,8 @@ def test_qwen3_4b_block_8_tokens(pv, wl, name):
     [(5, 16400)],                                    # a second segment of one chunk
     [(5000, 32), (300, 4096), (2, 8192)],            # jobs that share CTAs
     [(2048, 4096), (2048, 4096), (2048, 4096)],      # jobs with CTAs of their own
+    [(4863, 8192)], [(4865, 8192)],                  # one CTA per SM, two
+    [(9001, 4096), (777, 4096), (5, 16384)],         # two, and jobs that share them
     [(1000 + i, 16 * (1 + i)) for i in range(9)],    # more jobs than the small parameter block holds
 ])
 def test_gemv_ring_edges(pv, shapes):
