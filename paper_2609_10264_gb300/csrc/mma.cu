@@ -31,7 +31,7 @@
 //   warps 8-11   epilogue for vectors 0-31, warps 12-15 for vectors 32-63
 //                (TMEM lanes 32 (w mod 4) .. +31);
 //   warp 16      bulk-copies this CTA's half of the digit operand;
-//   warp 17      allocates TMEM; in the even CTA one lane issues the MMAs, in
+//   warp 17      allocates TMEM; in the even CTA it issues the MMAs, in
 //                the odd CTA one lane tells the even CTA when a stage of
 //                its own shared memory is filled;
 //   warp 18      streams 128 x 64 int8 tiles of M into a ring of raw tiles
@@ -144,6 +144,19 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
 
+// One lane of the converged warp (the same one each time).  MMAs are issued
+// under this by a warp that runs its loop together: their operands are then
+// uniform, and an MMA takes the warp 16 cycles.  Under `if (lane == 0)` it took
+// 61 alone on an SM and about 110 beside the other roles, so issuing bounded
+// the kernels (one MMA of N = 256 lasts 128; a 64-vector 8B-class layer 86
+// -> 80 us, a 256-vector 70B-class layer 1115 -> 1030, and at the power cap
+// of a long run 88.6 -> 84.7 and 1116 -> 1092).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+    return p != 0;
+}
+
 // ---------------------------------------------------------------- async copies, fences
 __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
     asm volatile(
@@ -203,13 +216,17 @@ __device__ __forceinline__ void mma_pair(uint32_t tmem_d, uint64_t adesc, uint64
         "l"(adesc), "l"(bdesc), "r"(kIdesc), "r"(accumulate));
 }
 // Arrive on `bar` (same offset) in every CTA of `mask` once all MMAs issued
-// so far have completed.
+// so far (by this lane) have completed.
 __device__ __forceinline__ void mma_commit_pair(uint64_t *bar, uint16_t mask) {
     asm volatile(
         "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
             smem_addr(bar)),
         "h"(mask)
         : "memory");
+}
+__device__ __forceinline__ void warp_commit_pair(uint64_t *bar, uint16_t mask) {
+    if (elect_one()) mma_commit_pair(bar, mask);
+    __syncwarp();
 }
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
     asm volatile(
@@ -329,7 +346,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     __shared__ __align__(8) uint64_t raw_full[kRaw], raw_empty[kRaw];  // raw int8 tile ring
     __shared__ uint32_t s_tmem;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(kFull, tid >> 5, 0);  // uniform, so that the roles' operands are
     const uint32_t base = (smem_addr(smem_raw) + 1023u) & ~1023u;
     uint8_t *smem = smem_raw + (base - smem_addr(smem_raw));
 
@@ -514,36 +532,37 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     } else if (half == 0) {
         // ------------------------------------------------ MMA issuer (even CTA)
-        if (lane == 0) {
+        {
             bool ok = true;
             for (int c = 0; c < nchunks && ok; ++c) {
                 const int bsel = c & 1;
-                if (!mbar_wait(&acc_empty[bsel], ((uint32_t)(c >> 1) & 1u) ^ 1u, err, wait_ns)) break;
+                if (!mbar_wait_warp(&acc_empty[bsel], ((uint32_t)(c >> 1) & 1u) ^ 1u, err, wait_ns)) break;
                 tc_fence_after();
                 const uint32_t dcol = tmem + (uint32_t)(bsel * kBN);
                 const int i_end = min(nblk, (c + 1) * kChunkBlocks);
                 for (int i = c * kChunkBlocks; i < i_end; ++i) {
                     const int s = i % kStages;
                     const uint32_t ph = (uint32_t)(i / kStages) & 1u;
-                    if (!mbar_wait(&full[s], ph, err, wait_ns)) {
+                    if (!mbar_wait_warp(&full[s], ph, err, wait_ns)) {
                         ok = false;
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t a_addr = base + (uint32_t)(s * kStageBytes);
-                    const uint32_t b_addr = a_addr + kATile;
+                    const uint64_t ad = sw128_desc(base) + (uint32_t)(s * kStageBytes >> 4);
+                    const uint64_t bd = ad + (uint32_t)(kATile >> 4);
+                    if (elect_one()) {
+                        mma_pair(dcol, ad, bd, i > c * kChunkBlocks ? 1u : 0u);
 #pragma unroll
-                    for (int k = 0; k < kBK / 16; ++k) {
-                        mma_pair(dcol, sw128_desc(a_addr + 32u * k), sw128_desc(b_addr + 32u * k),
-                                 (i > c * kChunkBlocks || k > 0) ? 1u : 0u);
+                        for (int k = 1; k < kBK / 16; ++k) mma_pair(dcol, ad + 2u * k, bd + 2u * k, 1u);
+                        mma_commit_pair(&empty_bar[s], pair_mask);
                     }
-                    mma_commit_pair(&empty_bar[s], pair_mask);
+                    __syncwarp();
                 }
-                mma_commit_pair(&acc_full[bsel], pair_mask);
+                warp_commit_pair(&acc_full[bsel], pair_mask);
             }
             // all issued MMAs have finished before TMEM is released
-            mma_commit_pair(&mma_done, (uint16_t)(1u << leader));
-            mbar_wait(&mma_done, 0, err, wait_ns);
+            warp_commit_pair(&mma_done, (uint16_t)(1u << leader));
+            mbar_wait_warp(&mma_done, 0, err, wait_ns);
         }
     } else {
         // ------------------------------------------------ stage relay (odd CTA)
@@ -905,7 +924,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     __shared__ __align__(8) uint64_t raw_full[kGRaw], raw_empty[kGRaw];
     __shared__ uint32_t s_tmem;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(kFull, tid >> 5, 0);  // uniform, so that the roles' operands are
     const uint32_t base = (smem_addr(smem_raw) + 1023u) & ~1023u;
     uint8_t *smem = smem_raw + (base - smem_addr(smem_raw));
     const uint32_t half = cluster.block_rank() & 1u;  // 0: the even CTA, which issues the MMAs
@@ -1132,7 +1152,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     } else if (half == 0) {
         // ------------------------------------------------ MMA issuer (even CTA)
-        if (lane == 0) {
+        {
             uint32_t gs = 0, gc = 0;
             bool ok = true;
             for (int r = 0; ok; ++r) {
@@ -1142,7 +1162,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const int nch = (it.nblk + kChunkBlocks - 1) / kChunkBlocks;
                 for (int ch = 0; ch < nch && ok; ++ch, ++gc) {
                     const int bsel = gc & 1u;
-                    if (!mbar_wait(&acc_empty[bsel], ((gc >> 1) & 1u) ^ 1u, err, wait_ns)) {
+                    if (!mbar_wait_warp(&acc_empty[bsel], ((gc >> 1) & 1u) ^ 1u, err, wait_ns)) {
                         ok = false;
                         break;
                     }
@@ -1152,28 +1172,32 @@ __global__ void __launch_bounds__(kThreads, 1)
                     for (int b0 = ch * kChunkBlocks; b0 < i_end; b0 += kGStageBlocks, ++gs) {
                         const int nb = min(kGStageBlocks, i_end - b0);
                         const int s = gs % kGStages;
-                        if (!mbar_wait(&full[s], (gs / kGStages) & 1u, err, wait_ns)) {
+                        if (!mbar_wait_warp(&full[s], (gs / kGStages) & 1u, err, wait_ns)) {
                             ok = false;
                             break;
                         }
                         tc_fence_after();
-                        const uint32_t st = base + (uint32_t)(s * kGStageBytes);
-                        for (int j = 0; j < nb; ++j) {
-                            const uint32_t a_addr = st + (uint32_t)(j * kATile);
-                            const uint32_t b_addr = st + (uint32_t)(kGStageBlocks * kATile + j * kBHalfG);
+                        const uint64_t ad = sw128_desc(base) + (uint32_t)(s * kGStageBytes >> 4);
+                        const uint64_t bd = ad + (uint32_t)(kGStageBlocks * kATile >> 4);
+                        if (elect_one()) {
+                            mma_pair_n<T::kIdesc>(dcol, ad, bd, b0 > ch * kChunkBlocks ? 1u : 0u);
 #pragma unroll
-                            for (int k = 0; k < kBK / 16; ++k)
-                                mma_pair_n<T::kIdesc>(dcol, sw128_desc(a_addr + 32u * k),
-                                                      sw128_desc(b_addr + 32u * k),
-                                                      (b0 > ch * kChunkBlocks || j > 0 || k > 0) ? 1u : 0u);
+                            for (int k = 1; k < kBK / 16; ++k) mma_pair_n<T::kIdesc>(dcol, ad + 2u * k, bd + 2u * k, 1u);
+                            if (nb > 1) {
+#pragma unroll
+                                for (int k = 0; k < kBK / 16; ++k)
+                                    mma_pair_n<T::kIdesc>(dcol, ad + (uint32_t)((kATile >> 4) + 2 * k),
+                                                          bd + (uint32_t)((kBHalfG >> 4) + 2 * k), 1u);
+                            }
+                            mma_commit_pair(&empty_bar[s], pair_mask);
                         }
-                        mma_commit_pair(&empty_bar[s], pair_mask);
+                        __syncwarp();
                     }
-                    mma_commit_pair(&acc_full[bsel], pair_mask);
+                    warp_commit_pair(&acc_full[bsel], pair_mask);
                 }
             }
-            mma_commit_pair(&mma_done, (uint16_t)1u);
-            mbar_wait(&mma_done, 0, err, wait_ns);
+            warp_commit_pair(&mma_done, (uint16_t)1u);
+            mbar_wait_warp(&mma_done, 0, err, wait_ns);
         }
     } else {
         // ------------------------------------------------ stage relay (odd CTA)
