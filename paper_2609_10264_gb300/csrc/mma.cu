@@ -174,13 +174,6 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, i
         "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_addr(bar))
         : "memory");
 }
-// Ask L2 to fetch the same box ahead of its load (no shared memory used).
-__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap *map, int x, int y) {
-    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(
-                     reinterpret_cast<uint64_t>(map)),
-                 "r"(x), "r"(y)
-                 : "memory");
-}
 __device__ __forceinline__ void fence_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
@@ -741,8 +734,7 @@ cudaError_t batched_launch(const int8_t *W, int m, int K, const uint32_t *Xhat, 
 // products (for example the projections of a decoder layer).  Work items are
 // (job, pair of 128-row tiles, 64-vector tile, K-split); one CTA pair of a
 // thread-block cluster stays resident and walks its items, its pipelines
-// (stages, raw ring, double-buffered TMEM accumulator) running on from one
-// item to the next, so that the pipeline fill, TMEM allocation and barrier
+// (stages, raw ring, TMEM accumulators) running on from one item to the next, so that the pipeline fill, TMEM allocation and barrier
 // set-up are paid once per launch and an item's epilogue overlaps the next
 // item's MMAs.  Items are ordered longest first (jobs by blocks per item),
 // and within a job by row pair, then K-split, then vector tile, so that the
@@ -754,41 +746,81 @@ cudaError_t batched_launch(const int8_t *W, int m, int K, const uint32_t *Xhat, 
 // the epilogue warp that adds the last part reduce its block instead, behind
 // a fence and a counter, held the epilogue up and was slower: 8B layer
 // 84 -> 97 us.)
+//
+// The converted M goes to TMEM, not to shared memory: a converter thread
+// takes one row's 64 bytes of a K-block, writes the fp16 values to its TMEM
+// lane, and the MMAs read A from there.  In shared memory M's K-block cost 128
+// write and 128 read wavefronts of the about 710 that a 64-vector K-block came
+// to, against 512 cycles of MMA, and left room for 3 stages and 4 raw tiles.
+// TMEM holds M only if the accumulators leave columns: a 64-vector tile is
+// computed as two parts of N = 128, whose exact chunks of 16 K-blocks end in
+// turn every 8, so that three accumulators of 128 columns do where two of 256
+// did, and the epilogue still reads one while the MMAs go on.  A ring of raw
+// tiles that deep (96 or 160 KiB) needs no L2 prefetch beside it; the requests
+// of that, from one lane, had held the loads up.
+// One 8B-class layer for 64 vectors 84.7 -> 79.5 us, for 16 vectors 59.4 ->
+// 46.4; one 70B-class layer for 256 vectors 1092 -> 1020 us (1.72 PFLOP/s of
+// the four digits, at the power cap; a plain bf16 GEMM sustains 1.73).  Tiles of
+// two K-blocks (128-byte rows) in the raw ring measured the same.
 // ---------------------------------------------------------------------------
 constexpr int kMaxGroupJobs = 8;
 constexpr int kMaxSplit = 8;
 constexpr int kNarrowMaxB = 16;  // batches up to this size use 16-vector tiles
-constexpr int kGPrefetch = 12;   // blocks of M asked of L2 ahead of their load
 
-// Tile geometry of the grouped kernel for V vectors per tile: 64 (N = 256
-// digit rows, the batched configurations) or 16 (N = 64, small batches,
-// where a 64-vector tile would leave three quarters of the MMA idle).  A
-// stage holds two K-blocks (A0 A1 B0 B1); the smaller digit operand of
-// V = 16 leaves room for four stages and eight raw tiles.
+// Tile geometry of the grouped kernel for V vectors per tile: 64 (256 digit
+// rows, the batched configurations) or 16 (64, small batches, where a
+// 64-vector tile would leave three quarters of the MMA idle).  A stage holds
+// one K-block for each group of four converter warps: two for V = 64; four for
+// V = 16, where HBM bounds and a K-block's conversion takes longer than its
+// share of the stream (8B-class layer, 16 vectors: 46.4 us; two groups 51.8).
 template <int V>
 struct GTile {
     static constexpr int kBV = V;
     static constexpr int kBN = 4 * V;                      // MMA N (digit rows)
     static constexpr int kBTile = kBN * kBK * 2;           // digit bytes per K-block (pair)
     static constexpr int kBHalf = kBTile / 2;              // one CTA's half
-    static constexpr int kStages = V == 64 ? 3 : 4;
-    static constexpr int kRaw = V == 64 ? 4 : 8;
-    static constexpr int kStageBytes = 2 * (kATile + kBHalf);
+    static constexpr int kGroups = V == 64 ? 2 : 4;        // converter groups of four warps = K-blocks of a stage
+    static constexpr int kConvWarps = 4 * kGroups;
+    static constexpr int kThreads = 32 * (kConvWarps + 8 + 3);
+    static constexpr int kStages = 4;                      // of the digit operand, in shared memory
+    static constexpr int kAStages = V == 64 ? 2 : 3;       // of M, in TMEM
+    static constexpr int kRaw = V == 64 ? 12 : 20;         // K-blocks of int8 M in flight
+    static constexpr int kStageBytes = kGroups * kBHalf;
     static constexpr int kRawOff = kStages * kStageBytes;
     static constexpr int kSmem = kRawOff + kRaw * kRawTile + 1024;  // + alignment slack
-    static constexpr int kTmemCols = 2 * kBN;              // double-buffered accumulator
+    static constexpr int kParts = V == 64 ? 2 : 1;         // accumulators a tile is split over
+    static constexpr int kPartN = kBN / kParts;            // digit rows (MMA N) of a part
+    static constexpr int kPartBlocks = kChunkBlocks / kParts;  // K-blocks from one part's end to the next
+    static constexpr int kAccs = kParts + 1;               // accumulators in TMEM
+    static constexpr int kACol = kAccs * kPartN;           // first TMEM column of M
+    static constexpr int kAStageCols = kGroups * kBK / 2;  // two fp16 a column
+    static constexpr int kTmemCols = 512;
     static constexpr int kVecs = V / 2;                    // vectors per epilogue thread
-    static constexpr uint32_t kIdesc = (1u << 4) | ((uint32_t)(kBN >> 3) << 17) | ((uint32_t)(2 * kBM >> 4) << 24);
-    static_assert(kSmem <= 232448, "shared memory per CTA");
-    static_assert(kTmemCols == 128 || kTmemCols == 512, "TMEM allocation");
+    static constexpr uint32_t kIdesc = (1u << 4) | ((uint32_t)(kPartN >> 3) << 17) | ((uint32_t)(2 * kBM >> 4) << 24);
+    static_assert(kSmem <= 231424, "shared memory per CTA, beside the barriers");
+    static_assert(kACol + kAStages * kAStageCols <= kTmemCols, "TMEM allocation");
+    static_assert(kAStages <= kStages, "a stage of M is free before its barrier comes round");
 };
 
+// A from TMEM: lane = row, a 32-bit column holds two fp16 of K.
 template <uint32_t IDESC>
-__device__ __forceinline__ void mma_pair_n(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
+__device__ __forceinline__ void mma_pair_ta(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t accumulate) {
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(IDESC), "r"(accumulate));
+        " tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(tmem_d),
+        "r"(tmem_a), "l"(bdesc), "r"(IDESC), "r"(accumulate)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};" ::"r"(taddr),
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
+        "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]),
+        "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]),
+        "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
+        : "memory");
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
 struct GroupJob {
@@ -909,18 +941,20 @@ __global__ void __launch_bounds__(256) k_split_finish(const __grid_constant__ Gr
 }
 
 template <int V>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(GTile<V>::kThreads, 1)
     k_batched_grouped(const __grid_constant__ GroupArgs args, uint32_t *__restrict__ err, int skip_report,
                       uint64_t wait_ns) {
     using T = GTile<V>;
-    constexpr int kGStageBlocks = 2;
+    constexpr int kGStageBlocks = T::kGroups, kConvW = T::kConvWarps;
     constexpr int kGStages = T::kStages, kGRaw = T::kRaw, kGStageBytes = T::kStageBytes, kGRawOff = T::kRawOff;
-    constexpr int kBHalfG = T::kBHalf, kBTileG = T::kBTile, kBNG = T::kBN, kBVG = T::kBV;
-    static_assert(kChunkBlocks % kGStageBlocks == 0, "chunks end on stage boundaries");
+    constexpr int kBHalfG = T::kBHalf, kBTileG = T::kBTile, kBVG = T::kBV;
+    constexpr int kLoadW = kConvW + 8, kMmaW = kConvW + 9, kWLoadW = kConvW + 10;
+    constexpr int kParts = T::kParts, kPartN = T::kPartN, kPartBlocks = T::kPartBlocks, kAccs = T::kAccs;
+    static_assert(kPartBlocks % kGStageBlocks == 0, "parts end on stage boundaries");
     cg::cluster_group cluster = cg::this_cluster();
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full[kGStages], empty_bar[kGStages];
-    __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2], mma_done;
+    __shared__ __align__(8) uint64_t acc_full[kAccs], acc_empty[kAccs], mma_done;
     __shared__ __align__(8) uint64_t raw_full[kGRaw], raw_empty[kGRaw];
     __shared__ uint32_t s_tmem;
 
@@ -937,23 +971,23 @@ __global__ void __launch_bounds__(kThreads, 1)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (tid == 0) {
         for (int s = 0; s < kGStages; ++s) {
-            // every converter warp (both groups), the digit copies' arrival
-            // and, in the even CTA, the odd CTA's report
-            mbar_init(&full[s], kConvThreads / 32 + 1 + (half == 0 ? 1 : 0));
+            // the digit copies' arrival and, in the even CTA, the odd CTA's
+            // report of its own and every converter warp of both CTAs
+            mbar_init(&full[s], half == 0 ? 2 * kConvW + 2 : 1);
             mbar_init(&empty_bar[s], 1);
         }
-        for (int b = 0; b < 2; ++b) {
+        for (int b = 0; b < kAccs; ++b) {
             mbar_init(&acc_full[b], 1);
             mbar_init(&acc_empty[b], 2 * kEpiThreads / 32);
         }
         mbar_init(&mma_done, 1);
         for (int r = 0; r < kGRaw; ++r) {
             mbar_init(&raw_full[r], 1);
-            mbar_init(&raw_empty[r], kConvThreads / 64);
+            mbar_init(&raw_empty[r], 4);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == kWarpMma) {
+    if (warp == kMmaW) {
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          smem_addr(&s_tmem)), "n"(T::kTmemCols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
@@ -963,11 +997,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_after();
     const uint32_t tmem = s_tmem;
 
-    if (warp < 8) {
+    if (warp < kConvW) {
         // ------------------------------------------------ converters: group j fills block j of each stage
         const int grp = warp >> 2;
-        const int t = tid & 127;
-        const int r0 = t >> 2, qk = t & 3;
+        const int row = tid & 127;  // = the TMEM lane
+        const uint32_t full_leader = cluster_addr(&full[0], 0);
+        const uint32_t ta = tmem + ((uint32_t)(row & 96) << 16) + (uint32_t)(T::kACol + grp * (kBK / 2));
         uint32_t gs = 0, gb = 0;
         bool ok = true;
         for (int r = 0; ok; ++r) {
@@ -976,55 +1011,51 @@ __global__ void __launch_bounds__(kThreads, 1)
             const Item it = group_item(args, idx);
             for (int b0 = 0; b0 < it.nblk; b0 += kGStageBlocks, ++gs) {
                 const int nb = min(kGStageBlocks, it.nblk - b0);
-                const int s = gs % kGStages;
-                const uint32_t ph = (gs / kGStages) & 1u;
                 const uint32_t rb = gb + (uint32_t)grp;
                 gb += (uint32_t)nb;
+                uint32_t o[kBK / 2];
+                // an item's last stage may be short of blocks: the rest only arrive
                 if (grp < nb) {
                     const int rs = rb % kGRaw;
-                    if (!mbar_wait_warp(&raw_full[rs], (rb / kGRaw) & 1u, err, wait_ns) ||
-                        !mbar_wait_warp(&empty_bar[s], ph ^ 1u, err, wait_ns)) {
+                    if (!mbar_wait_warp(&raw_full[rs], (rb / kGRaw) & 1u, err, wait_ns)) {
                         ok = false;
                         break;
                     }
-                    const uint8_t *raw = smem + kGRawOff + rs * kRawTile;
-                    uint8_t *a = smem + s * kGStageBytes + grp * kATile;
+                    // rows of 64 bytes, 64-byte swizzle: eight lanes' chunks lie in distinct banks
+                    const uint8_t *raw = smem + kGRawOff + rs * kRawTile + row * kBK;
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const uint4 w = *reinterpret_cast<const uint4 *>(raw + (r0 + 32 * j) * kBK + 16 * qk);
-                        uint32_t o[8];
-                        i8x4_to_f16x4(w.x, o[0], o[1]);
-                        i8x4_to_f16x4(w.y, o[2], o[3]);
-                        i8x4_to_f16x4(w.z, o[4], o[5]);
-                        i8x4_to_f16x4(w.w, o[6], o[7]);
-                        const int row = r0 + 32 * j;
-                        *reinterpret_cast<uint4 *>(a + sw128_off(row, 2 * qk)) = make_uint4(o[0], o[1], o[2], o[3]);
-                        *reinterpret_cast<uint4 *>(a + sw128_off(row, 2 * qk + 1)) =
-                            make_uint4(o[4], o[5], o[6], o[7]);
+                    for (int q = 0; q < 4; ++q) {
+                        const uint4 w = *reinterpret_cast<const uint4 *>(raw + ((q ^ ((row >> 1) & 3)) << 4));
+                        i8x4_to_f16x4(w.x, o[8 * q], o[8 * q + 1]);
+                        i8x4_to_f16x4(w.y, o[8 * q + 2], o[8 * q + 3]);
+                        i8x4_to_f16x4(w.z, o[8 * q + 4], o[8 * q + 5]);
+                        i8x4_to_f16x4(w.w, o[8 * q + 6], o[8 * q + 7]);
                     }
-                    fence_async_smem();
                     __syncwarp();
-                    if (lane == 0) {
-                        mbar_arrive(&full[s]);
-                        mbar_arrive(&raw_empty[rs]);
-                    }
-                } else {
-                    // no block for this group in the stage (an item's odd
-                    // last block): arrive in the stage's current phase
-                    if (!mbar_wait_warp(&empty_bar[s], ph ^ 1u, err, wait_ns)) {
-                        ok = false;
-                        break;
-                    }
-                    if (lane == 0) mbar_arrive(&full[s]);
+                    if (lane == 0) mbar_arrive(&raw_empty[rs]);
                 }
+                // the MMAs that read this stage of TMEM are done
+                const uint32_t gp = gs - (uint32_t)T::kAStages;
+                if (gs >= (uint32_t)T::kAStages &&
+                    !mbar_wait_warp(&empty_bar[gp % kGStages], (gp / kGStages) & 1u, err, wait_ns)) {
+                    ok = false;
+                    break;
+                }
+                if (grp < nb) {
+                    tc_fence_after();
+                    tmem_st32(ta + (gs % (uint32_t)T::kAStages) * (uint32_t)T::kAStageCols, o);
+                    tc_fence_before();
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(full_leader + 8u * (gs % kGStages));
             }
         }
-    } else if (warp < 16) {
+    } else if (warp < kConvW + 8) {
         // ------------------------------------------------ epilogue: TMEM -> mod-q sums -> Y
         const int q = warp & 3;
-        const int grp = (warp - 8) >> 2;
+        const int grp = (warp - kConvW) >> 2;
         const uint32_t acc_empty_leader = cluster_addr(&acc_empty[0], 0);
-        uint32_t gc = 0;
+        uint32_t ev = 0;  // accumulators read
         bool ok = true;
         for (int r = 0; ok; ++r) {
             const int idx = group_item_index(r, c, C, total);
@@ -1034,22 +1065,21 @@ __global__ void __launch_bounds__(kThreads, 1)
             uint32_t run[T::kVecs];
 #pragma unroll
             for (int v = 0; v < T::kVecs; ++v) run[v] = 0u;
-            const int nch = (it.nblk + kChunkBlocks - 1) / kChunkBlocks;
-            for (int ch = 0; ch < nch; ++ch, ++gc) {
-                const int bsel = gc & 1u;
-                if (!mbar_wait_warp(&acc_full[bsel], (gc >> 1) & 1u, err, wait_ns)) {
+            auto part = [&](uint32_t *sum) {  // the next accumulator, into a part's sums
+                const uint32_t a = ev % kAccs;
+                if (!mbar_wait_warp(&acc_full[a], (ev / kAccs) & 1u, err, wait_ns)) {
                     ok = false;
-                    break;
+                    return;
                 }
                 tc_fence_after();
 #pragma unroll
-                for (int j = 0; j < T::kVecs / 8; ++j) {
+                for (int j = 0; j < kPartN / 64; ++j) {
                     uint32_t rr[32];
-                    tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) +
-                                  (uint32_t)(bsel * kBNG + (kBNG / 2) * grp + 32 * j), rr);
+                    tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + a * kPartN + (uint32_t)((kPartN / 2) * grp + 32 * j),
+                              rr);
 #pragma unroll
                     for (int v = 0; v < 8; ++v) {
-                        run[8 * j + v] = fadd(run[8 * j + v],
+                        sum[8 * j + v] = fadd(sum[8 * j + v],
                                               digits_redc(__float2int_rn(__uint_as_float(rr[4 * v])),
                                                           __float2int_rn(__uint_as_float(rr[4 * v + 1])),
                                                           __float2int_rn(__uint_as_float(rr[4 * v + 2])),
@@ -1058,7 +1088,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive_cluster(acc_empty_leader + 8u * (uint32_t)bsel);
+                if (lane == 0) mbar_arrive_cluster(acc_empty_leader + 8u * a);
+                ++ev;
+            };
+            const int nev = (it.nblk + kPartBlocks - 1) / kPartBlocks + kParts - 1;
+            for (int i = 0; i < nev && ok; i += kParts) {
+                part(run);
+                if (kParts == 2 && ok && i + 1 < nev) part(run + T::kVecs / 2);
             }
             if (!ok) break;
             const int row = it.p * (2 * kBM) + (int)half * kBM + 32 * q + lane;
@@ -1077,123 +1113,129 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
             }
         }
-    } else if (warp == kWarpLoader) {
+    } else if (warp == kLoadW) {
         // ------------------------------------------------ this CTA's half of the digit operand
-        if (lane == 0) {
-            // the digit tiles come from the kernel launched just before this one
-            asm volatile("griddepcontrol.wait;" ::: "memory");
-            uint32_t gs = 0;
-            bool ok = true;
-            for (int r = 0; ok; ++r) {
-                const int idx = group_item_index(r, c, C, total);
-                if (idx < 0) break;
-                const Item it = group_item(args, idx);
-                const GroupJob &job = args.job[it.j];
-                const uint8_t *src = job.D + ((size_t)it.v * job.nkb + it.kb0) * kBTileG + (size_t)half * kBHalfG;
-                for (int b0 = 0; b0 < it.nblk; b0 += kGStageBlocks, ++gs) {
-                    const int nb = min(kGStageBlocks, it.nblk - b0);
-                    const int s = gs % kGStages;
-                    if (!mbar_wait(&empty_bar[s], ((gs / kGStages) & 1u) ^ 1u, err, wait_ns)) {
-                        ok = false;
-                        break;
-                    }
-                    mbar_arrive_tx(&full[s], (uint32_t)nb * kBHalfG);
-                    uint8_t *dst = smem + s * kGStageBytes + kGStageBlocks * kATile;
-                    for (int j = 0; j < nb; ++j)
-                        bulk_g2s(dst + j * kBHalfG, src + (size_t)(b0 + j) * kBTileG, kBHalfG, &full[s]);
+        // the digit tiles come from the kernel launched just before this one
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        uint32_t gs = 0;
+        bool ok = true;
+        for (int r = 0; ok; ++r) {
+            const int idx = group_item_index(r, c, C, total);
+            if (idx < 0) break;
+            const Item it = group_item(args, idx);
+            const GroupJob &job = args.job[it.j];
+            const uint8_t *src = job.D + ((size_t)it.v * job.nkb + it.kb0) * kBTileG + (size_t)half * kBHalfG;
+            for (int b0 = 0; b0 < it.nblk; b0 += kGStageBlocks, ++gs) {
+                const int nb = min(kGStageBlocks, it.nblk - b0);
+                const int s = gs % kGStages;
+                if (!mbar_wait_warp(&empty_bar[s], ((gs / kGStages) & 1u) ^ 1u, err, wait_ns)) {
+                    ok = false;
+                    break;
                 }
+                if (elect_one()) {
+                    mbar_arrive_tx(&full[s], (uint32_t)nb * kBHalfG);
+                    uint8_t *dst = smem + s * kGStageBytes;
+#pragma unroll
+                    for (int j = 0; j < kGStageBlocks; ++j)
+                        if (j < nb) bulk_g2s(dst + j * kBHalfG, src + (size_t)(b0 + j) * kBTileG, kBHalfG, &full[s]);
+                }
+                __syncwarp();
             }
-            // copies in flight complete before the CTA may exit
-            for (uint32_t i = gs > (uint32_t)kGStages ? gs - kGStages : 0u; i < gs; ++i)
-                mbar_wait(&full[i % kGStages], (i / kGStages) & 1u, err, wait_ns);
         }
-    } else if (warp == kWarpWLoad) {
+        // copies in flight complete before the CTA may exit
+        for (uint32_t i = gs > (uint32_t)kGStages ? gs - kGStages : 0u; i < gs; ++i)
+            mbar_wait_warp(&full[i % kGStages], (i / kGStages) & 1u, err, wait_ns);
+    } else if (warp == kWLoadW) {
         // ------------------------------------------------ raw int8 tiles of M by TMA
-        if (lane == 0) {
-            uint32_t gb = 0;
-            bool ok = true;
-            // L2 prefetches run kGPrefetch blocks ahead of the loads, into the
-            // next item near the end of this one: the raw ring alone holds too
-            // few blocks to cover the latency of HBM when the weights stream
-            // at the rate a 64-vector tile consumes them
-            const int idx0 = group_item_index(0, c, C, total);
-            Item nxt = idx0 >= 0 ? group_item(args, idx0) : Item{0, 0, 0, 0, 0};
-            int nxt_idx = idx0;
-            auto prefetch = [&](const Item &t, int i) {
-                const int y = t.p * (2 * kBM) + (int)half * kBM;
-                if (i < t.nblk && y < args.job[t.j].m) tma_prefetch_2d(&args.map[t.j], (t.kb0 + i) * kBK, y);
-            };
-            if (idx0 >= 0)
-                for (int i = 0; i < kGPrefetch; ++i) prefetch(nxt, i);
-            for (int r = 0; ok; ++r) {
-                const int idx = nxt_idx;
-                if (idx < 0) break;
-                const Item it = nxt;
-                nxt_idx = group_item_index(r + 1, c, C, total);
-                if (nxt_idx >= 0) nxt = group_item(args, nxt_idx);
-                const int m0 = it.p * (2 * kBM) + (int)half * kBM;
-                const CUtensorMap *map = &args.map[it.j];
-                for (int i = 0; i < it.nblk; ++i, ++gb) {
-                    if (i + kGPrefetch < it.nblk)
-                        prefetch(it, i + kGPrefetch);
-                    else if (nxt_idx >= 0)
-                        prefetch(nxt, i + kGPrefetch - it.nblk);
-                    const int rs = gb % kGRaw;
-                    if (!mbar_wait(&raw_empty[rs], ((gb / kGRaw) & 1u) ^ 1u, err, wait_ns)) {
-                        ok = false;
-                        break;
-                    }
+        uint32_t gb = 0;
+        bool ok = true;
+        for (int r = 0; ok; ++r) {
+            const int idx = group_item_index(r, c, C, total);
+            if (idx < 0) break;
+            const Item it = group_item(args, idx);
+            const int m0 = it.p * (2 * kBM) + (int)half * kBM;
+            const CUtensorMap *map = &args.map[it.j];
+            for (int i = 0; i < it.nblk; ++i, ++gb) {
+                const int rs = gb % kGRaw;
+                if (!mbar_wait_warp(&raw_empty[rs], ((gb / kGRaw) & 1u) ^ 1u, err, wait_ns)) {
+                    ok = false;
+                    break;
+                }
+                if (elect_one()) {
                     mbar_arrive_tx(&raw_full[rs], kRawTile);
                     tma_load_2d(smem + kGRawOff + rs * kRawTile, map, (it.kb0 + i) * kBK, m0, &raw_full[rs]);
                 }
+                __syncwarp();
             }
-            for (uint32_t i = gb > (uint32_t)kGRaw ? gb - kGRaw : 0u; i < gb; ++i)
-                mbar_wait(&raw_full[i % kGRaw], (i / kGRaw) & 1u, err, wait_ns);
         }
+        for (uint32_t i = gb > (uint32_t)kGRaw ? gb - kGRaw : 0u; i < gb; ++i)
+            mbar_wait_warp(&raw_full[i % kGRaw], (i / kGRaw) & 1u, err, wait_ns);
     } else if (half == 0) {
         // ------------------------------------------------ MMA issuer (even CTA)
         {
-            uint32_t gs = 0, gc = 0;
+            uint32_t gs = 0, ev = 0;  // stages, accumulators finished
             bool ok = true;
+            // Accumulators are opened, finished and read in one order, round the
+            // kAccs of them.  A segment of kPartBlocks ends one: of two parts the
+            // older, whose chunk began a segment earlier (part 0's first chunk is
+            // one segment, so no chunk is longer than kChunkBlocks); the younger
+            // opens with the segment.  An item's end finishes both.
+            // issue: the MMAs of a stage for one part, into accumulator e
+            auto issue = [&](uint32_t e, int part, int nb, bool first) {
+                if (first) {
+                    if (!mbar_wait_warp(&acc_empty[e % kAccs], ((e / kAccs) & 1u) ^ 1u, err, wait_ns)) return false;
+                    tc_fence_after();
+                }
+                const uint32_t d = tmem + (e % kAccs) * kPartN;
+                const uint32_t a = tmem + (uint32_t)T::kACol + (gs % (uint32_t)T::kAStages) * (uint32_t)T::kAStageCols;
+                const uint64_t bd =
+                    sw128_desc(base) + (((gs % kGStages) * kGStageBytes + part * (kPartN / 2) * 2 * kBK) >> 4);
+                if (elect_one()) {
+                    mma_pair_ta<T::kIdesc>(d, a, bd, first ? 0u : 1u);
+#pragma unroll
+                    for (int k = 1; k < kBK / 16; ++k) mma_pair_ta<T::kIdesc>(d, a + 8u * k, bd + 2u * k, 1u);
+#pragma unroll
+                    for (int j = 1; j < kGStageBlocks; ++j)
+                        if (j < nb) {
+#pragma unroll
+                            for (int k = 0; k < kBK / 16; ++k)
+                                mma_pair_ta<T::kIdesc>(d, a + (uint32_t)(j * (kBK / 2) + 8 * k),
+                                                       bd + (uint32_t)(j * (kBHalfG >> 4) + 2 * k), 1u);
+                        }
+                }
+                __syncwarp();
+                return true;
+            };
             for (int r = 0; ok; ++r) {
                 const int idx = group_item_index(r, c, C, total);
                 if (idx < 0) break;
                 const Item it = group_item(args, idx);
-                const int nch = (it.nblk + kChunkBlocks - 1) / kChunkBlocks;
-                for (int ch = 0; ch < nch && ok; ++ch, ++gc) {
-                    const int bsel = gc & 1u;
-                    if (!mbar_wait_warp(&acc_empty[bsel], ((gc >> 1) & 1u) ^ 1u, err, wait_ns)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint32_t dcol = tmem + (uint32_t)(bsel * kBNG);
-                    const int i_end = min(it.nblk, (ch + 1) * kChunkBlocks);
-                    for (int b0 = ch * kChunkBlocks; b0 < i_end; b0 += kGStageBlocks, ++gs) {
-                        const int nb = min(kGStageBlocks, i_end - b0);
-                        const int s = gs % kGStages;
-                        if (!mbar_wait_warp(&full[s], (gs / kGStages) & 1u, err, wait_ns)) {
+                const int nseg = (it.nblk + kPartBlocks - 1) / kPartBlocks;
+                for (int sg = 0; sg < nseg && ok; ++sg, ++ev) {
+                    const int b_first = sg * kPartBlocks, b_end = min(it.nblk, b_first + kPartBlocks);
+                    const int older = kParts == 2 ? sg & 1 : 0;  // the part that ends with this segment
+                    for (int b0 = b_first; b0 < b_end; b0 += kGStageBlocks, ++gs) {
+                        const int nb = min(kGStageBlocks, b_end - b0);
+                        if (!mbar_wait_warp(&full[gs % kGStages], (gs / kGStages) & 1u, err, wait_ns)) {
                             ok = false;
                             break;
                         }
                         tc_fence_after();
-                        const uint64_t ad = sw128_desc(base) + (uint32_t)(s * kGStageBytes >> 4);
-                        const uint64_t bd = ad + (uint32_t)(kGStageBlocks * kATile >> 4);
-                        if (elect_one()) {
-                            mma_pair_n<T::kIdesc>(dcol, ad, bd, b0 > ch * kChunkBlocks ? 1u : 0u);
-#pragma unroll
-                            for (int k = 1; k < kBK / 16; ++k) mma_pair_n<T::kIdesc>(dcol, ad + 2u * k, bd + 2u * k, 1u);
-                            if (nb > 1) {
-#pragma unroll
-                                for (int k = 0; k < kBK / 16; ++k)
-                                    mma_pair_n<T::kIdesc>(dcol, ad + (uint32_t)((kATile >> 4) + 2 * k),
-                                                          bd + (uint32_t)((kBHalfG >> 4) + 2 * k), 1u);
-                            }
-                            mma_commit_pair(&empty_bar[s], pair_mask);
+                        if (!issue(ev, older, nb, b0 == (kParts == 2 ? 0 : b_first))) {
+                            ok = false;
+                            break;
                         }
-                        __syncwarp();
+                        if (b0 + kGStageBlocks >= b_end) warp_commit_pair(&acc_full[ev % kAccs], pair_mask);
+                        if (kParts == 2 && !issue(ev + 1, 1 - older, nb, b0 == b_first)) {
+                            ok = false;
+                            break;
+                        }
+                        warp_commit_pair(&empty_bar[gs % kGStages], pair_mask);
                     }
-                    warp_commit_pair(&acc_full[bsel], pair_mask);
+                }
+                if (kParts == 2) {
+                    if (ok) warp_commit_pair(&acc_full[ev % kAccs], pair_mask);
+                    ++ev;
                 }
             }
             warp_commit_pair(&mma_done, (uint16_t)1u);
@@ -1226,7 +1268,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_before();
     __syncthreads();
     cluster.sync();  // the peer is done too: no MMA reads this CTA's memory any more
-    if (warp == kWarpMma) {
+    if (warp == kMmaW) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(T::kTmemCols));
     }
@@ -1369,7 +1411,7 @@ cudaError_t launch_grouped_v(const BatchJob *jobs, int count, uint32_t *err, cud
             const cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)kBM};
             const cuuint32_t estride[2] = {1, 1};
             if (encode(&args.map[i], CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<int8_t *>(b.W), gdim, gstride,
-                       box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                       box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
                 return cudaErrorInvalidValue;
         }
@@ -1395,7 +1437,7 @@ cudaError_t launch_grouped_v(const BatchJob *jobs, int count, uint32_t *err, cud
         const int C = std::min(best_c, item0);
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(2 * C, 1, 1);
-        cfg.blockDim = dim3(kThreads, 1, 1);
+        cfg.blockDim = dim3(T::kThreads, 1, 1);
         cfg.dynamicSmemBytes = T::kSmem;
         cfg.stream = s;
         cudaLaunchAttribute lattr[2];

@@ -886,6 +886,32 @@ def test_server_mvm_grouped_small_batches(pv, specs):
     assert pv.pvmvmd_device_status() == 0
 
 
+@pytest.mark.parametrize("specs", [
+    [(257, 64 * n, 64) for n in (1, 2, 7, 8, 9, 16, 17)],           # one segment of a part, its ends, a last odd block
+    [(300, 64 * n + 16, 33) for n in (15, 23, 24, 31, 32, 40)],     # chunks of both parts, K past a block
+    [(257, 64 * n, 16) for n in (1, 3, 4, 5, 16, 17, 33)],          # stages of four blocks, short last ones
+    [(5000, 1600, 256)],                                            # long items in turn on a pair
+])
+def test_grouped_product_segments(pv, specs):
+    """Where the grouped product's accumulators end, change over and drain:
+    item lengths round the segments, with the extreme sums of a chunk (weights
+    -128 and digits -128: 2^24 over 1024 columns)."""
+    import torch
+    rng = np.random.default_rng(specs[0][1] + specs[0][2])
+    ins = []
+    for m, K, B in specs:
+        W = rng.integers(-128, 128, size=(m, K), dtype=np.int8)
+        X = rng.integers(0, Q, size=(B, K)).astype(np.uint32)
+        W[:130] = -128
+        X[: B // 2] = (Q - 128 * (1 + 2**8 + 2**16)) % Q
+        ins.append((W, X, to_dev(W), to_dev(X), torch.full((B, m), -1, dtype=torch.int32, device="cuda")))
+    for rep in range(2):
+        pv.pvmvmd_server_mvm_grouped(pv.batch_jobs([(Wd, Xd, Yd) for _, _, Wd, Xd, Yd in ins]))
+        for W, X, _, _, Yd in ins:
+            assert_equal_report(pv.as_u32(Yd), oracle.server_mvm_batch(W, X), f"rep {rep} {W.shape} B={X.shape[0]}")
+    assert pv.pvmvmd_device_status() == 0
+
+
 @pytest.mark.parametrize("m,K,B,kw", [
     (300, 96, 700, {}),                            # more vectors than CTAs at once
     (1030, 1001, 310, {}),                         # unaligned rows of P^T
