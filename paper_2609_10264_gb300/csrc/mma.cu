@@ -790,7 +790,8 @@ struct GTile {
     static constexpr int kSmem = kRawOff + kRaw * kRawTile + 1024;  // + alignment slack
     static constexpr int kParts = V == 64 ? 2 : 1;         // accumulators a tile is split over
     static constexpr int kPartN = kBN / kParts;            // digit rows (MMA N) of a part
-    static constexpr int kPartBlocks = kChunkBlocks / kParts;  // K-blocks from one part's end to the next
+    static constexpr int kPartVecs = V / kParts;           // vectors of a part
+    static constexpr int kHalfVecs = kPartVecs / 2;        // of them in one CTA's half of the digit rows
     static constexpr int kAccs = kParts + 1;               // accumulators in TMEM
     static constexpr int kACol = kAccs * kPartN;           // first TMEM column of M
     static constexpr int kAStageCols = kGroups * kBK / 2;  // two fp16 a column
@@ -801,6 +802,15 @@ struct GTile {
     static_assert(kACol + kAStages * kAStageCols <= kTmemCols, "TMEM allocation");
     static_assert(kAStages <= kStages, "a stage of M is free before its barrier comes round");
 };
+
+// First digit row of vector vl in a tile: part by part and CTA by CTA, so that
+// a part holds consecutive vectors of the tile.
+template <int V>
+__device__ __forceinline__ uint32_t tile_row(int vl) {
+    using T = GTile<V>;
+    const int h = vl / T::kHalfVecs;  // 2 part + CTA
+    return (uint32_t)((h & 1) * (T::kBN / 2) + (h >> 1) * (T::kPartN / 2) + 4 * (vl % T::kHalfVecs));
+}
 
 // A from TMEM: lane = row, a 32-bit column holds two fp16 of K.
 template <uint32_t IDESC>
@@ -859,6 +869,14 @@ __device__ __forceinline__ Item group_item(const GroupArgs &a, int idx) {
     it.nblk = min(g.nkb, it.kb0 + g.per) - it.kb0;
     return it;
 }
+// Parts of an item's vector tile that hold vectors.  A tile of up to 32 of them
+// is one part: half the MMAs, digits and accumulators (an 8B-class layer for 32
+// vectors 71.9 -> 58.0 us, for 96 134.7 -> 118; a 70B-class one for 160 722 ->
+// 668).
+template <int V>
+__device__ __forceinline__ int item_parts(const GroupJob &g, const Item &it) {
+    return GTile<V>::kParts == 2 && g.B - it.v * V > GTile<V>::kPartVecs ? 2 : 1;
+}
 // The r-th item of pair c among C pairs (snake order); -1 past the end.
 __device__ __forceinline__ int group_item_index(int r, int c, int C, int total) {
     const int idx = r * C + ((r & 1) ? C - 1 - c : c);
@@ -887,6 +905,7 @@ __global__ void __launch_bounds__(256) k_digit_tiles_grouped(const __grid_consta
     const size_t total = (size_t)g.nvt * T::kBV * per_vec;
     if (gid >= total) return;
     const int v = (int)(gid / per_vec);
+    if (v / T::kPartVecs * T::kPartVecs >= g.B) return;  // a part without vectors is not read
     const int grp = (int)(gid % per_vec);
     const int kb = grp >> 3, chunk = grp & 7;
     const int k0 = kb * kBK + chunk * 8;
@@ -919,7 +938,7 @@ __global__ void __launch_bounds__(256) k_digit_tiles_grouped(const __grid_consta
             const __half2 d = __hadd2(*reinterpret_cast<const __half2 *>(&h), off);
             w[e] = *reinterpret_cast<const uint32_t *>(&d);
         }
-        *reinterpret_cast<uint4 *>(blk + sw128_off(4 * vl + l, chunk)) = make_uint4(w[0], w[1], w[2], w[3]);
+        *reinterpret_cast<uint4 *>(blk + sw128_off(tile_row<V>(vl) + l, chunk)) = make_uint4(w[0], w[1], w[2], w[3]);
     }
 }
 
@@ -949,8 +968,8 @@ __global__ void __launch_bounds__(GTile<V>::kThreads, 1)
     constexpr int kGStages = T::kStages, kGRaw = T::kRaw, kGStageBytes = T::kStageBytes, kGRawOff = T::kRawOff;
     constexpr int kBHalfG = T::kBHalf, kBTileG = T::kBTile, kBVG = T::kBV;
     constexpr int kLoadW = kConvW + 8, kMmaW = kConvW + 9, kWLoadW = kConvW + 10;
-    constexpr int kParts = T::kParts, kPartN = T::kPartN, kPartBlocks = T::kPartBlocks, kAccs = T::kAccs;
-    static_assert(kPartBlocks % kGStageBlocks == 0, "parts end on stage boundaries");
+    constexpr int kParts = T::kParts, kPartN = T::kPartN, kPartVecs = T::kPartVecs, kAccs = T::kAccs;
+    static_assert(kChunkBlocks / kParts % kGStageBlocks == 0, "chunks end on stage boundaries");
     cg::cluster_group cluster = cg::this_cluster();
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full[kGStages], empty_bar[kGStages];
@@ -1091,17 +1110,18 @@ __global__ void __launch_bounds__(GTile<V>::kThreads, 1)
                 if (lane == 0) mbar_arrive_cluster(acc_empty_leader + 8u * a);
                 ++ev;
             };
-            const int nev = (it.nblk + kPartBlocks - 1) / kPartBlocks + kParts - 1;
-            for (int i = 0; i < nev && ok; i += kParts) {
+            const int np = item_parts<V>(job, it), seg = kChunkBlocks / np;
+            const int nev = (it.nblk + seg - 1) / seg + np - 1;
+            for (int i = 0; i < nev && ok; i += np) {
                 part(run);
-                if (kParts == 2 && ok && i + 1 < nev) part(run + T::kVecs / 2);
+                if (np == 2 && ok && i + 1 < nev) part(run + (kParts - 1) * T::kHalfVecs);
             }
             if (!ok) break;
             const int row = it.p * (2 * kBM) + (int)half * kBM + 32 * q + lane;
             if (row < job.m) {
 #pragma unroll
                 for (int v = 0; v < T::kVecs; ++v) {
-                    const int b = it.v * kBVG + T::kVecs * grp + v;
+                    const int b = it.v * kBVG + v / T::kHalfVecs * kPartVecs + T::kHalfVecs * grp + v % T::kHalfVecs;
                     if (b < job.B) {
                         const uint32_t val = fmul_mont(run[v], kR2);
                         const size_t o = (size_t)b * job.m + row;
@@ -1125,6 +1145,7 @@ __global__ void __launch_bounds__(GTile<V>::kThreads, 1)
             const Item it = group_item(args, idx);
             const GroupJob &job = args.job[it.j];
             const uint8_t *src = job.D + ((size_t)it.v * job.nkb + it.kb0) * kBTileG + (size_t)half * kBHalfG;
+            const uint32_t bytes = (uint32_t)(kBHalfG / kParts * item_parts<V>(job, it));
             for (int b0 = 0; b0 < it.nblk; b0 += kGStageBlocks, ++gs) {
                 const int nb = min(kGStageBlocks, it.nblk - b0);
                 const int s = gs % kGStages;
@@ -1133,11 +1154,11 @@ __global__ void __launch_bounds__(GTile<V>::kThreads, 1)
                     break;
                 }
                 if (elect_one()) {
-                    mbar_arrive_tx(&full[s], (uint32_t)nb * kBHalfG);
+                    mbar_arrive_tx(&full[s], (uint32_t)nb * bytes);
                     uint8_t *dst = smem + s * kGStageBytes;
 #pragma unroll
                     for (int j = 0; j < kGStageBlocks; ++j)
-                        if (j < nb) bulk_g2s(dst + j * kBHalfG, src + (size_t)(b0 + j) * kBTileG, kBHalfG, &full[s]);
+                        if (j < nb) bulk_g2s(dst + j * kBHalfG, src + (size_t)(b0 + j) * kBTileG, bytes, &full[s]);
                 }
                 __syncwarp();
             }
@@ -1176,7 +1197,7 @@ __global__ void __launch_bounds__(GTile<V>::kThreads, 1)
             uint32_t gs = 0, ev = 0;  // stages, accumulators finished
             bool ok = true;
             // Accumulators are opened, finished and read in one order, round the
-            // kAccs of them.  A segment of kPartBlocks ends one: of two parts the
+            // kAccs of them.  A segment ends one: of two parts the
             // older, whose chunk began a segment earlier (part 0's first chunk is
             // one segment, so no chunk is longer than kChunkBlocks); the younger
             // opens with the segment.  An item's end finishes both.
@@ -1210,10 +1231,11 @@ __global__ void __launch_bounds__(GTile<V>::kThreads, 1)
                 const int idx = group_item_index(r, c, C, total);
                 if (idx < 0) break;
                 const Item it = group_item(args, idx);
-                const int nseg = (it.nblk + kPartBlocks - 1) / kPartBlocks;
+                const int np = item_parts<V>(args.job[it.j], it), seg = kChunkBlocks / np;
+                const int nseg = (it.nblk + seg - 1) / seg;
                 for (int sg = 0; sg < nseg && ok; ++sg, ++ev) {
-                    const int b_first = sg * kPartBlocks, b_end = min(it.nblk, b_first + kPartBlocks);
-                    const int older = kParts == 2 ? sg & 1 : 0;  // the part that ends with this segment
+                    const int b_first = sg * seg, b_end = min(it.nblk, b_first + seg);
+                    const int older = np == 2 ? sg & 1 : 0;  // the part that ends with this segment
                     for (int b0 = b_first; b0 < b_end; b0 += kGStageBlocks, ++gs) {
                         const int nb = min(kGStageBlocks, b_end - b0);
                         if (!mbar_wait_warp(&full[gs % kGStages], (gs / kGStages) & 1u, err, wait_ns)) {
@@ -1221,19 +1243,19 @@ __global__ void __launch_bounds__(GTile<V>::kThreads, 1)
                             break;
                         }
                         tc_fence_after();
-                        if (!issue(ev, older, nb, b0 == (kParts == 2 ? 0 : b_first))) {
+                        if (!issue(ev, older, nb, b0 == (np == 2 ? 0 : b_first))) {
                             ok = false;
                             break;
                         }
                         if (b0 + kGStageBlocks >= b_end) warp_commit_pair(&acc_full[ev % kAccs], pair_mask);
-                        if (kParts == 2 && !issue(ev + 1, 1 - older, nb, b0 == b_first)) {
+                        if (np == 2 && !issue(ev + 1, 1 - older, nb, b0 == b_first)) {
                             ok = false;
                             break;
                         }
                         warp_commit_pair(&empty_bar[gs % kGStages], pair_mask);
                     }
                 }
-                if (kParts == 2) {
+                if (np == 2) {
                     if (ok) warp_commit_pair(&acc_full[ev % kAccs], pair_mask);
                     ++ev;
                 }
@@ -1335,6 +1357,7 @@ cudaError_t launch_grouped_v(const BatchJob *jobs, int count, uint32_t *err, cud
             p.nkb = (b.K + kBK - 1) / kBK;
             p.nvt = (b.B + T::kBV - 1) / T::kBV;
             p.mp = (b.m + 2 * kBM - 1) / (2 * kBM);
+
             plan.push_back(p);
         }
         const cudaError_t attr =

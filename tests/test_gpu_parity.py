@@ -890,7 +890,8 @@ def test_server_mvm_grouped_small_batches(pv, specs):
     [(257, 64 * n, 64) for n in (1, 2, 7, 8, 9, 16, 17)],           # one segment of a part, its ends, a last odd block
     [(300, 64 * n + 16, 33) for n in (15, 23, 24, 31, 32, 40)],     # chunks of both parts, K past a block
     [(257, 64 * n, 16) for n in (1, 3, 4, 5, 16, 17, 33)],          # stages of four blocks, short last ones
-    [(5000, 1600, 256)],                                            # long items in turn on a pair
+    [(5000, 1600, 256), (5000, 1600, 70)],                          # long items in turn on a pair, of two parts and one
+    [(300, 64 * n, B) for n, B in ((1, 32), (16, 17), (17, 31), (33, 96), (5, 90), (40, 65))],  # tiles of one part
 ])
 def test_grouped_product_segments(pv, specs):
     """Where the grouped product's accumulators end, change over and drain:
