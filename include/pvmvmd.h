@@ -133,9 +133,9 @@ int pvmvmd_encode(pvmvmd_ctx *ctx, const uint32_t *X_dev, int B, const pvmvmd_ke
  * online work).  W_dev int8 m x K row-major, Xhat_dev B x K, Yhat_dev B x m.
  * Needs no context and no secret.  B == 1 runs the bandwidth-bound GEMV;
  * 2 <= B <= 16 (K a multiple of 16, 16-byte aligned W and Xhat) a GEMV that
- * reads M once per four vectors, or, for B >= 8 and m K B >= 2^27, the
- * tensor-core product with 16-vector tiles; larger B the byte-limb
- * tensor-core product.
+ * reads M once per four vectors, or, where it would read 12 MiB or more and
+ * the scratch can be had, the tensor-core product with 16-vector tiles;
+ * larger B the byte-limb tensor-core product.
  * 1 <= K <= PVMVMD_MAX_K.  The batch-1 GEMV and the 2 <= B <= 16 GEMV may
  * start reading M while the kernel before it on the stream finishes, when
  * that kernel signals its

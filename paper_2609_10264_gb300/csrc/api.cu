@@ -605,30 +605,50 @@ int pvmvmd_weights_split_i16(const int16_t *W_dev, int m, int K, int8_t *Whi_dev
 
 namespace pv {
 namespace {
-// The path of a product of 2 <= B <= 16 vectors: one pass over M per four
-// vectors with dp4a, unless the problem is large enough for the tensor-core
-// product with 16-vector tiles to win (measured: 14336 x 4096 with 8 vectors
-// 41.0 against 27.1 us, with 4 vectors 23.8 against 26.0 us; 4096 x 2560 with
-// 8 vectors 12.1 against 12.9 us).
-bool small_batch_wins(const void *W, int m, int K, const uint32_t *Xhat, int B) {
-    const bool tensor_small = B >= 8 && (double)m * K * B >= 128.0 * 1024 * 1024;
-    return B > 1 && B <= kSmallBatchMax && !tensor_small && K % 16 == 0 &&
+// The paths of a product of 2 <= B <= 16 vectors: one pass over M per four
+// vectors with dp4a, or the tensor-core product with 16-vector tiles (8 to 10 us
+// until M is large) from 12 MiB of M passed over that way.  GEMV against
+// tensor cores, us: 4096 x 2560 with 4 vectors 8.2 and 8.7, with 8 12.8 and
+// 9.2; 1024 x 4096 with 8 8.2 and 8.7, with 12 11.4 and 8.7; 4096 x 4096 with 2
+// 10.6 and 9.7; 14336 x 4096 with 4 23.6 and 15.4.  Both planes of a 16-bit
+// M: 4096 x 2560 with 4 12.8 and 12.8, with 8 20.0 and 12.8; 4096 x 4096 with 2
+// 17.0 and 13.8.  Where the scratch of the tensor-core product cannot be had
+// (memory, or a stream under capture that has not run as large a call), the
+// GEMV's smaller one serves.
+bool small_batch_ok(const void *W, int K, const uint32_t *Xhat, int B) {
+    return B > 1 && B <= kSmallBatchMax && K % 16 == 0 &&
            ((reinterpret_cast<uintptr_t>(W) | reinterpret_cast<uintptr_t>(Xhat)) & 15u) == 0;
+}
+bool small_batch_on_tensor(int m, int K, int B) {
+    return (double)m * K * ((B + 3) / 4) >= 12.0 * 1024 * 1024;
 }
 }  // namespace
 }  // namespace pv
 
-// Both planes in one launch where that needs no more scratch than a product:
-// of the small-batch kernel, which combines them itself (4096 x 2560, 8
-// vectors: 28.8 -> 19.8 us a call), or as two jobs of the batch-1 kernel (one
-// vector: 28.6 -> 17.5 us).
+// Both planes in one launch: of the small-batch kernel, which combines them
+// itself (4096 x 2560, 4 vectors: 18.9 -> 12.8 us a call), as two jobs of the
+// grouped tensor-core product (8 vectors: 28.8 -> 12.8; under capture only if its
+// scratch is there already) or of the batch-1 kernel (one vector: 28.6 ->
+// 17.5 us).
 int pvmvmd_server_mvm_i16(const int8_t *Whi_dev, const int8_t *Wlo_dev, int m, int K, const uint32_t *Xhat_dev,
                           int B, uint32_t *Yhat_dev, uint32_t *Ytmp_dev, void *stream) {
     using namespace pv;
     if (!Whi_dev || !Wlo_dev || !Ytmp_dev || !Xhat_dev || !Yhat_dev) return PVMVMD_E_ARG;
     if (m < 1 || K < 1 || K > PVMVMD_MAX_K || B < 1) return PVMVMD_E_SHAPE;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if (small_batch_wins(Whi_dev, m, K, Xhat_dev, B) && small_batch_wins(Wlo_dev, m, K, Xhat_dev, B)) {
+    if (small_batch_ok(Whi_dev, K, Xhat_dev, B) && small_batch_ok(Wlo_dev, K, Xhat_dev, B)) {
+        if (small_batch_on_tensor(m, K, B)) {
+            uint32_t *err = error_word();
+            if (!err) return PVMVMD_E_CUDA;
+            const BatchJob jobs[2] = {{Whi_dev, Xhat_dev, Yhat_dev, m, K, B}, {Wlo_dev, Xhat_dev, Ytmp_dev, m, K, B}};
+            const cudaError_t e = launch_batched_grouped(jobs, 2, err, s, true);
+            if (e == cudaSuccess) PV_CUDA(launch_combine_256(Yhat_dev, Ytmp_dev, (size_t)B * m, s));
+            if (e != cudaErrorNotReady && e != cudaErrorMemoryAllocation) {
+                PV_CUDA(e);
+                return PVMVMD_OK;
+            }
+            (void)cudaGetLastError();
+        }
         PV_CUDA(launch_gemv_small_batch(Wlo_dev, m, K, Xhat_dev, B, Yhat_dev, s, Whi_dev));
         return PVMVMD_OK;
     }
@@ -775,7 +795,16 @@ int pvmvmd_server_mvm(const int8_t *W_dev, int m, int K, const uint32_t *Xhat_de
         PV_CUDA(launch_gemv(W_dev, m, K, Xhat_dev, Yhat_dev, err, s));
         return PVMVMD_OK;
     }
-    if (small_batch_wins(W_dev, m, K, Xhat_dev, B)) {
+    if (small_batch_ok(W_dev, K, Xhat_dev, B)) {
+        if (small_batch_on_tensor(m, K, B)) {
+            const BatchJob job{W_dev, Xhat_dev, Yhat_dev, m, K, B};
+            const cudaError_t e = launch_batched_grouped(&job, 1, err, s, true);
+            if (e != cudaErrorNotReady && e != cudaErrorMemoryAllocation) {
+                PV_CUDA(e);
+                return PVMVMD_OK;
+            }
+            (void)cudaGetLastError();
+        }
         PV_CUDA(launch_gemv_small_batch(W_dev, m, K, Xhat_dev, B, Yhat_dev, s));
         return PVMVMD_OK;
     }

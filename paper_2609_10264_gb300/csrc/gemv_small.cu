@@ -281,7 +281,7 @@ cudaError_t launch_gemv_small_batch(const int8_t *W, int m, int K, const uint32_
     const int Bp = (B + kNbVec - 1) / kNbVec * kNbVec;
     const size_t row_words = (size_t)K / 4, job_words = 4 * kNbVec * row_words;
     void *pbuf = nullptr;
-    cudaError_t e = stream_scratch(kScratchDigitPlanes, (size_t)Bp / kNbVec * job_words * sizeof(uint32_t), s, &pbuf);
+    cudaError_t e = stream_scratch(kScratchDigits, (size_t)Bp / kNbVec * job_words * sizeof(uint32_t), s, &pbuf);
     if (e != cudaSuccess) return e;
     uint32_t *planes = static_cast<uint32_t *>(pbuf);
     {

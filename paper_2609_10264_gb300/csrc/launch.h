@@ -183,12 +183,17 @@ struct BatchJob {
     int m, K, B;
 };
 bool batched_grouped_eligible(const int8_t *W, const uint32_t *Xhat, int m, int K, int B);
-cudaError_t launch_batched_grouped(const BatchJob *jobs, int count, uint32_t *err, cudaStream_t s);
+// With ready_only, cudaErrorNotReady (and no launch) where scratch is not ready.
+cudaError_t launch_batched_grouped(const BatchJob *jobs, int count, uint32_t *err, cudaStream_t s,
+                                   bool ready_only = false);
 
 // Grow-only scratch of at least `need` bytes for `purpose` on the current
 // device, one buffer per stream (see scratch.cu).
-enum ScratchPurpose { kScratchDigitTiles = 0, kScratchDigitPlanes = 1 };
+enum ScratchPurpose { kScratchDigits = 0 };  // digit tiles or planes of the batched products
 cudaError_t stream_scratch(int purpose, size_t need, cudaStream_t s, void **out);
+// Whether stream_scratch would return a buffer here: one that is large enough
+// already, or a stream that is not being captured.
+bool stream_scratch_ready(int purpose, size_t need, cudaStream_t s);
 
 // cudaFuncSetAttribute for the current device, done once per (kernel,
 // attribute, device): function attributes belong to each device's instance

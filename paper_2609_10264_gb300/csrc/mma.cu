@@ -1342,7 +1342,7 @@ bool batched_grouped_eligible(const int8_t *W, const uint32_t *Xhat, int m, int 
 }
 
 template <int V>
-cudaError_t launch_grouped_v(const BatchJob *jobs, int count, uint32_t *err, cudaStream_t s) {
+cudaError_t launch_grouped_v(const BatchJob *jobs, int count, uint32_t *err, cudaStream_t s, bool ready_only) {
     using T = GTile<V>;
     for (int a = 0; a < count; a += kMaxGroupJobs) {
         const int n = std::min(count - a, kMaxGroupJobs);
@@ -1395,7 +1395,8 @@ cudaError_t launch_grouped_v(const BatchJob *jobs, int count, uint32_t *err, cud
         }
         abytes = (abytes + 15) & ~(size_t)15;
         void *buf = nullptr;
-        cudaError_t e = stream_scratch(kScratchDigitTiles, dbytes + abytes, s, &buf);
+        if (ready_only && !stream_scratch_ready(kScratchDigits, dbytes + abytes, s)) return cudaErrorNotReady;
+        cudaError_t e = stream_scratch(kScratchDigits, dbytes + abytes, s, &buf);
         if (e != cudaSuccess) return e;
         PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
         if (!encode) return cudaErrorNotSupported;
@@ -1496,16 +1497,15 @@ cudaError_t launch_grouped_v(const BatchJob *jobs, int count, uint32_t *err, cud
     return cudaSuccess;
 }
 
-cudaError_t launch_batched_grouped(const BatchJob *jobs, int count, uint32_t *err, cudaStream_t s) {
+cudaError_t launch_batched_grouped(const BatchJob *jobs, int count, uint32_t *err, cudaStream_t s, bool ready_only) {
     // small batches in 16-vector tiles, the rest in 64-vector tiles
     std::vector<BatchJob> narrow, wide;
     for (int i = 0; i < count; ++i) (jobs[i].B <= kNarrowMaxB ? narrow : wide).push_back(jobs[i]);
     cudaError_t e = cudaSuccess;
-    if (!wide.empty()) e = launch_grouped_v<64>(wide.data(), (int)wide.size(), err, s);
-    if (e == cudaSuccess && !narrow.empty()) e = launch_grouped_v<16>(narrow.data(), (int)narrow.size(), err, s);
+    if (!wide.empty()) e = launch_grouped_v<64>(wide.data(), (int)wide.size(), err, s, ready_only);
+    if (e == cudaSuccess && !narrow.empty()) e = launch_grouped_v<16>(narrow.data(), (int)narrow.size(), err, s, ready_only);
     return e;
 }
-
 
 cudaError_t launch_batched(const int8_t *W, int m, int K, const uint32_t *Xhat, int B,
                            uint32_t *Yhat, uint32_t *err, cudaStream_t s) {
@@ -1517,7 +1517,7 @@ cudaError_t launch_batched(const int8_t *W, int m, int K, const uint32_t *Xhat, 
     const int nkb = (K + kBK - 1) / kBK;
     const int nvt = (B + kBV - 1) / kBV;
     void *D = nullptr;
-    cudaError_t e = stream_scratch(kScratchDigitTiles, (size_t)nvt * nkb * kBTile, s, &D);
+    cudaError_t e = stream_scratch(kScratchDigits, (size_t)nvt * nkb * kBTile, s, &D);
     if (e != cudaSuccess) return e;
     return batched_launch(W, m, K, Xhat, B, Yhat, err, static_cast<uint8_t *>(D), s);
 }

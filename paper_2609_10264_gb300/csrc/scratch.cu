@@ -2,8 +2,10 @@
 //
 // Grow-only device scratch held per (purpose, device, stream).
 //
-// The batched product's digit tiles and the small-batch product's digit
-// planes live in library-owned buffers.  Keying them by stream lets calls on
+// The batched products' digit tiles and the small-batch product's digit
+// planes live in one library-owned buffer a stream: every kernel that writes
+// it waits for the kernel before, and a call that has sized it serves every
+// smaller one, whichever of the two paths that takes.  Keying by stream lets calls on
 // different streams overlap without sharing a buffer; calls on one stream
 // are ordered, so they may share one.  A buffer that must grow is replaced
 // after the stream has drained (the old one may still be read), which is
@@ -17,18 +19,33 @@
 
 namespace pv {
 
+namespace {
+struct Buf {
+    void *ptr = nullptr;
+    size_t bytes = 0;
+};
+std::mutex g_bufs_mu;
+std::map<std::tuple<int, int, cudaStream_t>, Buf> g_bufs;
+}  // namespace
+
+bool stream_scratch_ready(int purpose, size_t need, cudaStream_t s) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    {
+        std::lock_guard<std::mutex> lock(g_bufs_mu);
+        const auto it = g_bufs.find(std::make_tuple(purpose, dev, s));
+        if (it != g_bufs.end() && it->second.bytes >= need) return true;
+    }
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(s, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone;
+}
+
 cudaError_t stream_scratch(int purpose, size_t need, cudaStream_t s, void **out) {
-    struct Buf {
-        void *ptr = nullptr;
-        size_t bytes = 0;
-    };
-    static std::mutex mu;
-    static std::map<std::tuple<int, int, cudaStream_t>, Buf> bufs;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    std::lock_guard<std::mutex> lock(mu);
-    Buf &b = bufs[std::make_tuple(purpose, dev, s)];
+    std::lock_guard<std::mutex> lock(g_bufs_mu);
+    Buf &b = g_bufs[std::make_tuple(purpose, dev, s)];
     if (b.bytes < need) {
         if (b.ptr) {
             if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;

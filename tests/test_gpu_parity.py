@@ -357,11 +357,13 @@ def test_sixteen_bit_weights_round_trip(pv, wl, B):
     ctx.destroy()
 
 
-@pytest.mark.parametrize("m,K,B", [(33, 16, 2), (300, 6144 + 96, 5), (1025, 528, 16), (1, 512, 1), (40, 16400, 1)])
+@pytest.mark.parametrize("m,K,B", [(33, 16, 2), (300, 6144 + 96, 5), (1025, 528, 16), (1, 512, 1), (40, 16400, 1),
+                                   (1023, 4096, 12), (1025, 4096, 9), (3100, 2064, 5)])
 def test_sixteen_bit_product_one_launch(pv, m, K, B):
     """The 16-bit product where one launch takes both planes: few vectors (one
-    chunk of columns, two segments of K, the largest batch, an odd row) and
-    one vector (one launch, and two segments)."""
+    chunk of columns, two segments of K, the largest batch, an odd row), one
+    vector (one launch, and two segments), and both sides of the line from
+    which the tensor cores take the two planes."""
     rng = np.random.default_rng(m + K + B)
     W = rng.integers(-32768, 32640, size=(m, K)).astype(np.int16)
     W[0] = -32768
@@ -911,6 +913,33 @@ def test_grouped_product_segments(pv, specs):
         for W, X, _, _, Yd in ins:
             assert_equal_report(pv.as_u32(Yd), oracle.server_mvm_batch(W, X), f"rep {rep} {W.shape} B={X.shape[0]}")
     assert pv.pvmvmd_device_status() == 0
+
+
+def test_small_batches_captured_after_another_call(pv):
+    """Captured calls of 2 to 16 vectors on a stream whose scratch a call of
+    one plane, or of the GEMV path alone, has sized: whichever path they find
+    room for, they are captured and replay to the same results."""
+    import torch
+    rng = np.random.default_rng(81)
+    m, K = 4096, 2560
+    hi, lo = (to_dev(rng.integers(-128, 128, size=(m, K), dtype=np.int8)) for _ in range(2))
+    X = to_dev(rng.integers(0, Q, size=(8, K)).astype(np.uint32))
+    exp16, exp5 = pv.pvmvmd_server_mvm_i16(hi, lo, X), pv.pvmvmd_server_mvm(lo, X[:5])
+    for warm in ((lo, X), (lo[:100], X)):  # tensor cores; GEMV
+        s = torch.cuda.Stream()
+        s.wait_stream(torch.cuda.current_stream())
+        pv.pvmvmd_server_mvm(*warm, stream=s)
+        s.synchronize()
+        Y16, tmp, Y5 = torch.zeros_like(exp16), torch.zeros_like(exp16), torch.zeros_like(exp5)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            pv.pvmvmd_server_mvm_i16(hi, lo, X, Y16, tmp, stream=s)
+            pv.pvmvmd_server_mvm(lo, X[:5], Y5, stream=s)
+        for _ in range(2):
+            Y16.zero_(), Y5.zero_()
+            g.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(Y16, exp16) and torch.equal(Y5, exp5)
 
 
 @pytest.mark.parametrize("m,K,B,kw", [
