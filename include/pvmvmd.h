@@ -143,9 +143,10 @@ int pvmvmd_encode(pvmvmd_ctx *ctx, const uint32_t *X_dev, int B, const pvmvmd_ke
  * write M.  Kernels that do not use programmatic dependent launch, and all
  * of this library's kernels, are safe.  The B > 1 paths keep their digit
  * operand in library scratch held per stream: calls on different streams
- * may run concurrently, and a buffer grows (with a synchronisation of the
- * stream) only when a call needs more than any earlier call on that stream,
- * which must not happen while the stream is being captured. */
+ * may run concurrently, and a buffer grows only when a call needs more than any
+ * earlier call on that stream, which must not happen while the stream is being
+ * captured (outgrown buffers stay valid for captured graphs, unless memory runs
+ * short). */
 int pvmvmd_server_mvm(const int8_t *W_dev, int m, int K, const uint32_t *Xhat_dev, int B,
                       uint32_t *Yhat_dev, void *stream);
 
@@ -202,8 +203,7 @@ int pvmvmd_server_mvm_grouped(const pvmvmd_mvm_batch_job *jobs, int count, void 
  * memory is reserved up front by its own allocator or pool (a cudaMalloc
  * from inside the library could fail or fragment that pool), or a
  * latency-critical loop that cannot afford the regular call's first-use
- * allocation, or the device-wide synchronisation of replacing an outgrown
- * buffer.  It always runs the tensor-core digit product (also for B = 1),
+ * allocation, or that of replacing an outgrown buffer.  It always runs the tensor-core digit product (also for B = 1),
  * whose fp16 digit tiles then live in one file-scope __device__ array of
  * PVMVMD_NOALLOC_SCRATCH_BYTES (16 MiB) that every GPU which loads the
  * library holds until the process exits.  The tiles take

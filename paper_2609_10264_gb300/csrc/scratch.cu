@@ -7,13 +7,18 @@
 // it waits for the kernel before, and a call that has sized it serves every
 // smaller one, whichever of the two paths that takes.  Keying by stream lets calls on
 // different streams overlap without sharing a buffer; calls on one stream
-// are ordered, so they may share one.  A buffer that must grow is replaced
-// after the stream has drained (the old one may still be read), which is
-// not allowed while the stream is being captured: make one call of the
-// largest shape before capturing.
+// are ordered, so they may share one.  A buffer that must grow is replaced by
+// one of at least twice its size and kept beside it, since kernels in flight
+// and captured graphs may still use it; the kept ones come to less than the
+// one in use.  Only where memory is short are they given back, after the
+// stream has drained, for a buffer of just the size that is needed.  A buffer
+// cannot grow while the stream is being captured: make one call of the largest
+// shape before capturing.
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <tuple>
+#include <vector>
 
 #include "launch.h"
 
@@ -23,6 +28,7 @@ namespace {
 struct Buf {
     void *ptr = nullptr;
     size_t bytes = 0;
+    std::vector<void *> old;  // outgrown
 };
 std::mutex g_bufs_mu;
 std::map<std::tuple<int, int, cudaStream_t>, Buf> g_bufs;
@@ -47,14 +53,23 @@ cudaError_t stream_scratch(int purpose, size_t need, cudaStream_t s, void **out)
     std::lock_guard<std::mutex> lock(g_bufs_mu);
     Buf &b = g_bufs[std::make_tuple(purpose, dev, s)];
     if (b.bytes < need) {
-        if (b.ptr) {
-            if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
-            cudaFree(b.ptr);
-            b.ptr = nullptr;
-            b.bytes = 0;
+        size_t bytes = std::max(need, 2 * b.bytes);
+        void *p = nullptr;
+        e = cudaMalloc(&p, bytes);
+        if (e == cudaErrorMemoryAllocation) {
+            (void)cudaGetLastError();
+            if (b.ptr) {
+                if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
+                cudaFree(b.ptr);
+                for (void *o : b.old) cudaFree(o);
+                b = Buf{};
+            }
+            e = cudaMalloc(&p, bytes = need);
         }
-        if ((e = cudaMalloc(&b.ptr, need)) != cudaSuccess) return e;
-        b.bytes = need;
+        if (e != cudaSuccess) return e;
+        if (b.ptr) b.old.push_back(b.ptr);
+        b.ptr = p;
+        b.bytes = bytes;
     }
     *out = b.ptr;
     return cudaSuccess;

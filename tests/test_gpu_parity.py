@@ -940,6 +940,9 @@ def test_small_batches_captured_after_another_call(pv):
             g.replay()
             torch.cuda.synchronize()
             assert torch.equal(Y16, exp16) and torch.equal(Y5, exp5)
+            # the stream's scratch grows; the graph's stays valid
+            pv.pvmvmd_server_mvm(lo, X.repeat(9, 1), stream=s)
+            s.synchronize()
 
 
 @pytest.mark.parametrize("m,K,B,kw", [
