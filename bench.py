@@ -519,9 +519,11 @@ def run_ours(args):
     cur[0] = 0
     # encode: the fused syndrome kernel (standard), or k_field_add with masks
     # prepared ahead (boost; pipelined adds the preparation: fused syndrome +
-    # k_output_mask); decode: challenge syndrome, k_verify_u, k_decrypt, k_check
+    # k_output_mask); decode: k_decode (standard), or two challenge kernels,
+    # k_decrypt and k_check
     enc_launches = {"standard": 1, "boost": 1, "pipelined": 1 + 2}[args.mode]
-    expected_per_step = enc_launches + (1 if args.server_mode == "multi" else VECTORS) + 4
+    dec_launches = 1 if args.mode == "standard" else 4
+    expected_per_step = enc_launches + (1 if args.server_mode == "multi" else VECTORS) + dec_launches
     # the library's own count is what the line reports; the expected count is
     # a consistency check of the path the calls took
     launches_per_step = int(round(counted_per_step))

@@ -113,7 +113,8 @@ int pvmvmd_params_resolve(const pvmvmd_params *in, int m, int K, pvmvmd_params *
  * memory plus code tables and scratch; the call synchronises `stream` before
  * returning.  The context also owns one CUDA stream, created at the device's
  * highest stream priority, on which pvmvmd_decode_verify runs its short
- * verification kernels beside the decrypt.  On error *out is NULL. */
+ * verification kernels beside the decrypt (large calls run one kernel on the
+ * caller's stream instead).  On error *out is NULL. */
 int pvmvmd_preprocess(const int8_t *W_dev, int m, int K, const pvmvmd_params *params,
                       const pvmvmd_key *key, void *stream, pvmvmd_ctx **out);
 
@@ -187,7 +188,8 @@ typedef struct {
  * jobs per launch): one pair of CTAs per pair of SMs walks a list of tiles
  * of all the jobs, longest first, so that small matrices fill the GPU and
  * the pipeline is set up once.  Other jobs take the path pvmvmd_server_mvm
- * gives them (batch-1 requests together in one grouped GEMV).  `jobs` is a host array that may be freed on return; outputs must
+ * gives them (batch-1 requests together in one grouped GEMV).  `jobs` is a
+ * host array that may be freed on return; outputs must
  * not overlap any input or each other.  1 <= count, each 1 <= K <=
  * PVMVMD_MAX_K, 1 <= m, 1 <= B.  The digit operands live in library scratch
  * held per stream, as for pvmvmd_server_mvm. */
@@ -361,14 +363,14 @@ int pvmvmd_device_status(void *stream);
  * finishes (its results are then unspecified), instead of waiting forever.
  * This call lets a test make one such wait expire on purpose, with a short
  * limit, so that the expiry path itself runs:
- *   PVMVMD_DEBUG_WAIT_SCAN     the single-pass look-back scan of the syndrome
- *                              (encode of codes too long for a thread-block
- *                              cluster): tile `index` of every vector
+ *   PVMVMD_DEBUG_WAIT_SCAN     the single-pass look-back scans of the
+ *                              syndrome (a few vectors, challenges, or the
+ *                              longest codes): tile `index` of every vector
  *                              publishes no status word, and look-back spins
  *                              give up after `limit` polls;
  *   PVMVMD_DEBUG_WAIT_PRODUCT  the tensor-core batched product: the second
  *                              CTA of every pair withholds its report for
- *                              K-block `index`, and pipeline waits give up
+ *                              stage `index`, and pipeline waits give up
  *                              after `limit` nanoseconds;
  *   PVMVMD_DEBUG_WAIT_OFF      restore the normal behaviour (index and limit
  *                              ignored).

@@ -32,10 +32,10 @@ constexpr uint32_t kTagChallenge = 10;
 constexpr uint32_t kTagBvPrimary = 21;    // batch verification challenges
 constexpr uint32_t kTagBvSecondary = 22;
 // Encode batches of at least this many vectors as the lanes of N x B arrays
-// (launch_lane_syndrome) when the code needs a cluster per vector; smaller
-// batches and codes that fit one CTA use the fused kernel.
+// (launch_lane_syndrome) when the code does not fit one CTA's shared memory and
+// the sliced kernel does not take them.
 constexpr int kLaneMinBatch = 32;
-// Server products of at most this many vectors use the small-batch GEMV.
+// Server products of at most this many vectors use the small-batch paths.
 constexpr int kSmallBatchMax = 16;
 
 // --------------------------------------------------------------------------

@@ -1,11 +1,13 @@
 // Client decode and verification (Protocol 3, Verify and Decrypt).
 //
+//  * k_decode           a large call in one kernel: the challenges, then the
+//                       columns of k_decrypt and the checks.
 //  * k_verify_u         u_q = e_q^T Q for the ell shared challenges
 //                       (sum of t_y rows of Q, cost (2t-1)n per repetition,
 //                       the e^T Q row of the cost table in Sec. 5.3).
 //  * k_decrypt          Y_b = y_hat_b - P e_x,b (t_x rows of P^T), many
-//                       short CTAs: 512 columns of one vector each, the
-//                       rows split over two groups; in boost mode
+//                       short CTAs: 512, 256 or 64 columns of one vector
+//                       each, the rows split over groups; in boost mode
 //                       (Sec. 7.2) P e_x,b was prepared ahead and is read
 //                       instead of the t_x rows of P^T.
 //  * k_check            accept_b = AND_q (L_q == R_q), L_q = u_q . x_hat_b,

@@ -6,6 +6,10 @@
 //                         accumulator as a single-pass decoupled look-back scan.
 //  * k_syndrome_gather    second half: inverse permutation gather and the
 //                         block sums of R, fused with x_hat = x + x'.
+//  * k_syndrome_fused     the whole syndrome, a vector per CTA with its code in
+//                         shared memory.
+//  * k_syndrome_sliced    the same for longer codes and many vectors, slice by
+//                         slice (k_slice_tables orders the positions).
 //  * k_syndrome_tiles     the syndrome's first half for a few vectors, or a few
 //                         shared challenges: every CTA samples e itself and
 //                         takes one tile of 2048 positions.
@@ -133,7 +137,7 @@ __device__ void warp_bitmap_to_support(const uint32_t *bitmap, uint32_t nbw, uin
     }
 }
 
-// One warp per vector (the path for codes too long for one cluster).
+// One warp per vector (before k_syndrome_scan).
 __global__ void __launch_bounds__(32) k_sample_sparse(pvmvmd_key key, uint32_t tag, uint64_t idx0,
                                                      uint32_t N, uint32_t t,
                                                      uint32_t *__restrict__ out,
