@@ -611,7 +611,7 @@ namespace {
 // tensor cores, us: 4096 x 2560 with 4 vectors 8.2 and 8.7, with 8 12.8 and
 // 9.2; 1024 x 4096 with 8 8.2 and 8.7, with 12 11.4 and 8.7; 4096 x 4096 with 2
 // 10.6 and 9.7; 14336 x 4096 with 4 23.6 and 15.4.  Both planes of a 16-bit
-// M: 4096 x 2560 with 4 12.8 and 12.8, with 8 20.0 and 12.8; 4096 x 4096 with 2
+// M: 4096 x 2560 with 4 12.8 and 12.8, with 8 20.0 and 12.4; 4096 x 4096 with 2
 // 17.0 and 13.8.  Where the scratch of the tensor-core product cannot be had
 // (memory, or a stream under capture that has not run as large a call), the
 // GEMV's smaller one serves.
@@ -627,7 +627,7 @@ bool small_batch_on_tensor(int m, int K, int B) {
 
 // Both planes in one launch: of the small-batch kernel, which combines them
 // itself (4096 x 2560, 4 vectors: 18.9 -> 12.8 us a call), as two jobs of the
-// grouped tensor-core product (8 vectors: 28.8 -> 12.8; under capture only if its
+// grouped tensor-core product (8 vectors: 28.8 -> 12.4; under capture only if its
 // scratch is there already) or of the batch-1 kernel (one vector: 28.6 ->
 // 17.5 us).
 int pvmvmd_server_mvm_i16(const int8_t *Whi_dev, const int8_t *Wlo_dev, int m, int K, const uint32_t *Xhat_dev,

@@ -26,9 +26,12 @@ __global__ void k_lift_i16(const int16_t *__restrict__ W, size_t n, uint32_t *__
     out[i] = w < 0 ? kQ - (uint32_t)(-w) : (uint32_t)w;
 }
 
-// y = 256 y + y_lo over F_q (y holds y_hi on entry).
+// y = 256 y + y_lo over F_q (y holds y_hi on entry).  Launched beside the
+// product that writes them, which it waits for (a 4096 x 2560 product of 8
+// vectors 12.8 -> 12.4 us, its round trip 46.4 -> 45.0).
 __global__ void k_combine_256(uint32_t *__restrict__ y, const uint32_t *__restrict__ ylo, size_t n) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (i >= n) return;
     y[i] = fadd(fmul(y[i], 256u), ylo[i]);
 }
@@ -54,8 +57,16 @@ cudaError_t launch_lift_i16(const int16_t *W, size_t n, uint32_t *out, cudaStrea
 cudaError_t launch_combine_256(uint32_t *y, const uint32_t *ylo, size_t n, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
     if ((n + 255) / 256 > 0x7fffffffu) return cudaErrorInvalidValue;
-    k_combine_256<<<grid_of(n), 256, 0, s>>>(y, ylo, n); note_launch();
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid_of(n), 1, 1);
+    cfg.blockDim = dim3(256, 1, 1);
+    cfg.stream = s;
+    cudaLaunchAttribute attrs[1];
+    attrs[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attrs[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attrs;
+    cfg.numAttrs = 1;
+    return counted_launch(cudaLaunchKernelEx(&cfg, k_combine_256, y, ylo, n));
 }
 
 }  // namespace pv
