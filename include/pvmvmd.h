@@ -137,14 +137,15 @@ int pvmvmd_encode(pvmvmd_ctx *ctx, const uint32_t *X_dev, int B, const pvmvmd_ke
  * reads M once per four vectors, or, where it would read 12 MiB or more and
  * the scratch can be had, the tensor-core product with 16-vector tiles;
  * larger B the byte-limb tensor-core product.
- * 1 <= K <= PVMVMD_MAX_K.  The batch-1 GEMV and the 2 <= B <= 16 GEMV may
- * start reading M while the kernel before it on the stream finishes, when
- * that kernel signals its
+ * 1 <= K <= PVMVMD_MAX_K.  The batch-1 GEMV may start reading M while the
+ * kernel before it on the stream finishes, when that kernel signals its
  * dependents early (programmatic dependent launch); such a kernel must not
- * write M.  Kernels that do not use programmatic dependent launch, and all
- * of this library's kernels, are safe.  The B > 1 paths keep their digit
- * operand in library scratch held per stream: calls on different streams
- * may run concurrently, and a buffer grows only when a call needs more than any
+ * write M, also where only kernels of this library lie between it and the
+ * call.  Kernels that do not use programmatic dependent launch, and all
+ * of this library's kernels, are safe, and every product of B > 1 vectors
+ * reads M only once the kernels before the call have completed.  The B > 1
+ * paths keep their digit operand in library scratch held per stream: calls on
+ * different streams may run concurrently, and a buffer grows only when a call needs more than any
  * earlier call on that stream, which must not happen while the stream is being
  * captured (outgrown buffers stay valid for captured graphs, unless memory runs
  * short). */

@@ -79,7 +79,9 @@ struct NbArgs {
 // per four consecutive K-elements of one vector.
 __global__ void __launch_bounds__(256) k_nb_planes(const uint32_t *__restrict__ Xhat, int B, int K, int Bp,
                                                   uint32_t *__restrict__ planes) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");  // x_hat comes from the kernel before
+    // x_hat comes from the kernel before, and M may: the product, which reads M
+    // without a wait of its own, may start only after it
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const size_t gid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t per_vec = (size_t)K / 4;
@@ -119,9 +121,9 @@ __global__ void __launch_bounds__(kMultiThreads, 2) k_gemv_nb(const __grid_const
     const long long hi = total * (blockIdx.x + 1) / gridDim.x;
 
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    // The first loads of M go out before griddepcontrol.wait (M is the
-    // server's weight matrix, never written by a kernel of the chain); the
-    // planes and y_hat are touched only after it.
+    // The first loads of M go out before griddepcontrol.wait (whatever wrote M
+    // is done: k_nb_planes waits before it lets this kernel start); the planes
+    // and y_hat are touched only after it.
     bool waited = false;
 
     for (int j = 0; j < args.count; ++j) {

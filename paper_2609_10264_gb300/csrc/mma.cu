@@ -888,9 +888,11 @@ __device__ __forceinline__ int group_item_index(int r, int c, int C, int total) 
 template <int V>
 __global__ void __launch_bounds__(256) k_digit_tiles_grouped(const __grid_constant__ GroupArgs args) {
     using T = GTile<V>;
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    // x_hat comes from the kernel before, which may also still use the scratch
+    // x_hat comes from the kernel before, which may also still use the scratch.
+    // Only then may the product start: it reads M without a wait of its own,
+    // and the kernel before may be the one that writes M.
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (blockIdx.x >= args.zero0) {
         for (size_t i = (size_t)(blockIdx.x - args.zero0) * 256 + threadIdx.x; i < args.acc_chunks;
              i += (size_t)args.zeros * 256)

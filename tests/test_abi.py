@@ -144,3 +144,15 @@ def test_debug_wait_hook_arguments(pv):
     assert lib.pvmvmd_debug_expire_wait(pv.PVMVMD_DEBUG_WAIT_SCAN, 0, 0) == pv.PVMVMD_E_ARG
     assert lib.pvmvmd_debug_expire_wait(pv.PVMVMD_DEBUG_WAIT_PRODUCT, 3, 1000) == pv.PVMVMD_OK
     assert lib.pvmvmd_debug_expire_wait(pv.PVMVMD_DEBUG_WAIT_OFF, 0, 0) == pv.PVMVMD_OK
+
+
+def test_operand_kernels_wait_before_they_signal():
+    """The kernels that form a product's operand are launched early themselves,
+    and the product after them reads M without a wait: it may start only once
+    they have waited for the kernel before, which may have written M."""
+    csrc = os.path.join(ROOT, "paper_2609_10264_gb300", "csrc")
+    for name, kernel in (("mma.cu", "k_digit_tiles_grouped"), ("gemv_small.cu", "k_nb_planes")):
+        text = open(os.path.join(csrc, name)).read()
+        body = re.search(r"__global__[^;{]*\b" + kernel + r"\(.*?\n}\n", text, flags=re.S).group(0)
+        wait, signal = body.find("griddepcontrol.wait;"), body.find("griddepcontrol.launch_dependents;")
+        assert 0 <= wait < signal, kernel

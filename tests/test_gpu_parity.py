@@ -915,6 +915,36 @@ def test_grouped_product_segments(pv, specs):
     assert pv.pvmvmd_device_status() == 0
 
 
+@pytest.mark.parametrize("B,grouped", [(64, False), (64, True), (70, True), (8, False), (3, False)])
+def test_product_after_a_kernel_that_signals_early_and_writes_m(pv, wl, B, grouped):
+    """A product of B > 1 vectors reads M only once the kernel before it has
+    completed, also when that one lets its dependents start early.  The encode's
+    kernel is such a one: its output, read as int8 rows, is M here (1.6 MB from
+    100 vectors; for B = 8 and 3, both sides of the tensor cores' line, 13 MB)."""
+    import torch
+    rng = np.random.default_rng(B)
+    K, n = 4096, 100 if B > 16 else 800
+    ctx = pv.pvmvmd_preprocess(to_dev(wl.weights_uniform(16, K, 3)), key=91)
+    V = to_dev(rng.integers(0, Q, size=(n, K)).astype(np.uint32))
+    M = torch.empty((n, K), dtype=torch.int32, device="cuda")
+    W = M.view(torch.int8).view(4 * n, K)[: 4 * n if B != 3 else 300]
+    X = rng.integers(0, Q, size=(B, K)).astype(np.uint32)
+    Xd, Y = to_dev(X), torch.empty((B, W.shape[0]), dtype=torch.int32, device="cuda")
+    jobs = pv.batch_jobs([(W, Xd, Y)])
+    pv.pvmvmd_server_mvm(W.clone(), Xd)  # the scratch is there
+    for rep in range(4):
+        M.fill_(rep)  # what an early read would find
+        torch.cuda.synchronize()
+        pv.pvmvmd_encode(ctx, V, key=rep, Xhat=M)
+        if grouped:
+            pv.pvmvmd_server_mvm_grouped(jobs)
+        else:
+            pv.pvmvmd_server_mvm(W, Xd, Y)
+        assert_equal_report(pv.as_u32(Y), oracle.server_mvm_batch(W.cpu().numpy(), X), f"rep {rep}")
+    assert pv.pvmvmd_device_status() == 0
+    ctx.destroy()
+
+
 def test_small_batches_captured_after_another_call(pv):
     """Captured calls of 2 to 16 vectors on a stream whose scratch a call of
     one plane, or of the GEMV path alone, has sized: whichever path they find
