@@ -368,7 +368,11 @@ int pvmvmd_device_status(void *stream);
  *                              syndrome (a few vectors, challenges, or the
  *                              longest codes): tile `index` of every vector
  *                              publishes no status word, and look-back spins
- *                              give up after `limit` polls;
+ *                              give up after `limit` polls; in a decode of
+ *                              one kernel that tile does not report itself
+ *                              done either, and the waits on such reports
+ *                              give up after as many polls (an index past
+ *                              the tiles shortens the waits alone);
  *   PVMVMD_DEBUG_WAIT_PRODUCT  the tensor-core batched product: the second
  *                              CTA of every pair withholds its report for
  *                              stage `index`, and pipeline waits give up

@@ -354,8 +354,10 @@ __global__ void __launch_bounds__(kCheckThreads, 4) k_check(const uint32_t *__re
 // verification is done while P^T streams, and nothing is left between two
 // decodes but one launch (a side stream for the verification, forked and
 // joined by events, kept them 6 to 10 us apart).  sync: the finished tiles of
-// each challenge, the finished CTAs of u and g, the finished checks; all zero
-// at launch, and set back, with the tiles' status words, by the last check.
+// each challenge, the finished CTAs of u and g, the CTAs of the verification
+// that are through; all zero at launch, and set back, with the tiles' status
+// words, by the last of those.  A wait that runs out lets its CTA go on, so
+// only a count of all of them says that none will use the words again.
 // ---------------------------------------------------------------------------
 constexpr int kSyncReady = 16, kSyncFinished = 17;
 static_assert(kSyncFinished < kDecodeSyncWords, "sync words");
@@ -382,11 +384,11 @@ __device__ __forceinline__ void sync_signal(uint32_t *p) {
         atomicAdd(p, 1u);
     }
 }
-__device__ __forceinline__ void sync_await(const uint32_t *p, uint32_t n, uint32_t *err) {
+__device__ __forceinline__ void sync_await(const uint32_t *p, uint32_t n, uint32_t *err, uint32_t spin_limit) {
     if (threadIdx.x == 0) {
         uint32_t spins = 0;
         while (ld_acquire_u32(p) < n) {
-            if (++spins > kSpinLimit) {
+            if (++spins > spin_limit) {
                 record_error(err, kErrScanTimeout);
                 break;
             }
@@ -394,6 +396,21 @@ __device__ __forceinline__ void sync_await(const uint32_t *p, uint32_t n, uint32
         }
     }
     __syncthreads();
+}
+// The last thing that a CTA of the verification does with sync and the status
+// words; the last of them sets both back.  The fence orders a signal before it;
+// a check signals nothing and has read what it waits for.
+__device__ __forceinline__ void sync_leave(const DecodeArgs &a, uint32_t nscan, bool signalled) {
+    __shared__ bool s_last;
+    if (threadIdx.x == 0) {
+        if (signalled) __threadfence();
+        s_last = atomicAdd(a.sync + kSyncFinished, 1u) == a.tiles + a.gather + a.B - 1;
+        if (s_last) __threadfence();
+    }
+    __syncthreads();
+    if (!s_last) return;
+    for (uint32_t i = threadIdx.x; i < nscan; i += kDecThreads) a.tile.status[i] = 0ull;
+    if (threadIdx.x < kDecodeSyncWords) a.sync[threadIdx.x] = 0u;
 }
 
 // accept_b, by one CTA (as k_check with a cluster of one)
@@ -458,7 +475,12 @@ __global__ void __launch_bounds__(kDecThreads, 4) k_decode(const __grid_constant
     const uint32_t ntiles = scan_tiles(a.tile.N), nscan = a.tile.count * ntiles;
     if (blk < a.tiles) {
         syndrome_tile(a.tile, blk);
-        sync_signal(a.sync + (blk < nscan ? blk / ntiles : (uint32_t)kSyncReady));
+        // a failure-path test withholds one tile's signal too (off: skip_tile >= ntiles)
+        if (blk >= nscan || ntiles - 1 - blk % ntiles != a.tile.skip_tile)
+            sync_signal(a.sync + (blk < nscan ? blk / ntiles : (uint32_t)kSyncReady));
+        else
+            __syncthreads();
+        sync_leave(a, nscan, true);
         return;
     }
     blk -= a.tiles;
@@ -471,7 +493,7 @@ __global__ void __launch_bounds__(kDecThreads, 4) k_decode(const __grid_constant
             at[0] = x.x; at[1] = x.y; at[2] = x.z; at[3] = x.w;
             at[4] = y.x; at[5] = y.y; at[6] = y.z; at[7] = y.w;
         }
-        sync_await(a.sync + q, ntiles, a.tile.err);
+        sync_await(a.sync + q, ntiles, a.tile.err, a.tile.spin_limit);
         if (j < (uint32_t)a.m) {
             const uint32_t *F = a.tile.F + (size_t)q * a.tile.N;
             uint32_t s = 0;
@@ -487,19 +509,14 @@ __global__ void __launch_bounds__(kDecThreads, 4) k_decode(const __grid_constant
             a.g[(size_t)q * a.m + j] = s;
         }
         sync_signal(a.sync + kSyncReady);
+        sync_leave(a, nscan, true);
         return;
     }
     blk -= a.gather;
     if (blk >= a.first && blk < a.first + a.B) {
-        __shared__ bool s_last;
-        sync_await(a.sync + kSyncReady, a.tiles - nscan + a.gather, a.tile.err);
+        sync_await(a.sync + kSyncReady, a.tiles - nscan + a.gather, a.tile.err, a.tile.spin_limit);
         check_cta(a, blk - a.first);
-        if (threadIdx.x == 0) s_last = atomicAdd(a.sync + kSyncFinished, 1u) == a.B - 1;
-        __syncthreads();
-        if (s_last) {  // every other part that uses them is done
-            for (uint32_t i = threadIdx.x; i < nscan; i += kDecThreads) a.tile.status[i] = 0ull;
-            if (threadIdx.x < kDecodeSyncWords) a.sync[threadIdx.x] = 0u;
-        }
+        sync_leave(a, nscan, false);
         return;
     }
     if (blk >= a.first) blk -= a.B;

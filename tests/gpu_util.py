@@ -85,3 +85,23 @@ def tamper(pv, t, b: int, i: int, delta: int) -> None:
     v = int(pv.as_u32(t[b, i:i + 1])[0])
     nv = (v + int(delta)) % Q
     t[b, i] = nv - (1 << 32) if nv >= (1 << 31) else nv
+
+
+def key_bound_error(pp_seed: int, m: int, challenge_seed: int, at) -> list:
+    """Errors for the three outputs `at` that the two challenges of one key do
+    not see (g_q . error = 0 for both), so that a verification accepts them under
+    this key and, but for a chance of 2^-30, rejects them under any other: its
+    verdict tells whose challenges it used.  The paper's parameters."""
+    gy = oracle.Code.sample(oracle.key_from_seed(pp_seed), 1, m)
+    g = []
+    for q in range(2):
+        s, v = oracle.sample_sparse(oracle.key_from_seed(challenge_seed), oracle.TAG_CHALLENGE, q, gy.N,
+                                    oracle.T_Y_PAPER)
+        e = np.zeros(gy.N, np.uint32)
+        e[s] = v
+        row = gy.syndrome(e)
+        g.append([int(row[i]) for i in at])
+    (a0, a1, a2), (b0, b1, b2) = g
+    err = [(a1 * b2 - a2 * b1) % Q, (a2 * b0 - a0 * b2) % Q, (a0 * b1 - a1 * b0) % Q]
+    assert any(err) and all(sum(x * y for x, y in zip(r, err)) % Q == 0 for r in g)
+    return err
