@@ -147,8 +147,8 @@ int pvmvmd_encode(pvmvmd_ctx *ctx, const uint32_t *X_dev, int B, const pvmvmd_ke
  * paths keep their digit operand in library scratch held per stream: calls on
  * different streams may run concurrently, and a buffer grows only when a call needs more than any
  * earlier call on that stream, which must not happen while the stream is being
- * captured (outgrown buffers stay valid for captured graphs, unless memory runs
- * short). */
+ * captured (a buffer that a captured call was given stays valid for its graph,
+ * and is never given back). */
 int pvmvmd_server_mvm(const int8_t *W_dev, int m, int K, const uint32_t *Xhat_dev, int B,
                       uint32_t *Yhat_dev, void *stream);
 

@@ -10,10 +10,12 @@
 // are ordered, so they may share one.  A buffer that must grow is replaced by
 // one of at least twice its size and kept beside it, since kernels in flight
 // and captured graphs may still use it; the kept ones come to less than the
-// one in use.  Only where memory is short are they given back, after the
-// stream has drained, for a buffer of just the size that is needed.  A buffer
-// cannot grow while the stream is being captured: make one call of the largest
-// shape before capturing.
+// one in use.  Where memory is short those that no capture has been handed
+// are given back, after the stream has drained, for a buffer of just the size
+// that is needed; a graph may be replayed at any time, so a buffer that one was
+// handed is kept for good, and the call is refused if that leaves too little.  A
+// buffer cannot grow while the stream is being captured: make one call of the
+// largest shape before capturing.
 #include <algorithm>
 #include <map>
 #include <mutex>
@@ -28,7 +30,8 @@ namespace {
 struct Buf {
     void *ptr = nullptr;
     size_t bytes = 0;
-    std::vector<void *> old;  // outgrown
+    bool captured = false;    // handed to a call under capture
+    std::vector<void *> old;  // outgrown, of no capture
 };
 std::mutex g_bufs_mu;
 std::map<std::tuple<int, int, cudaStream_t>, Buf> g_bufs;
@@ -58,18 +61,31 @@ cudaError_t stream_scratch(int purpose, size_t need, cudaStream_t s, void **out)
         e = cudaMalloc(&p, bytes);
         if (e == cudaErrorMemoryAllocation) {
             (void)cudaGetLastError();
-            if (b.ptr) {
+            if ((b.ptr && !b.captured) || !b.old.empty()) {
                 if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
-                cudaFree(b.ptr);
                 for (void *o : b.old) cudaFree(o);
-                b = Buf{};
+                b.old.clear();
+                if (!b.captured) {
+                    cudaFree(b.ptr);
+                    b.ptr = nullptr;
+                    b.bytes = 0;
+                }
             }
             e = cudaMalloc(&p, bytes = need);
         }
         if (e != cudaSuccess) return e;
-        if (b.ptr) b.old.push_back(b.ptr);
+        if (b.ptr && !b.captured) b.old.push_back(b.ptr);
         b.ptr = p;
         b.bytes = bytes;
+        b.captured = false;
+    }
+    if (!b.captured) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) {  // the legacy stream, while another is captured
+            (void)cudaGetLastError();
+            capture = cudaStreamCaptureStatusActive;
+        }
+        b.captured = capture != cudaStreamCaptureStatusNone;
     }
     *out = b.ptr;
     return cudaSuccess;
