@@ -145,10 +145,11 @@ int pvmvmd_encode(pvmvmd_ctx *ctx, const uint32_t *X_dev, int B, const pvmvmd_ke
  * of this library's kernels, are safe, and every product of B > 1 vectors
  * reads M only once the kernels before the call have completed.  The B > 1
  * paths keep their digit operand in library scratch held per stream: calls on
- * different streams may run concurrently, and a buffer grows only when a call needs more than any
- * earlier call on that stream, which must not happen while the stream is being
- * captured (a buffer that a captured call was given stays valid for its graph,
- * and is never given back). */
+ * different streams may run concurrently, and a buffer grows (with a
+ * synchronisation of the stream) only when a call needs more than any earlier
+ * call on that stream, which must not happen while the stream is being
+ * captured.  A buffer that a captured call was given stays valid for its graph
+ * and is never given back. */
 int pvmvmd_server_mvm(const int8_t *W_dev, int m, int K, const uint32_t *Xhat_dev, int B,
                       uint32_t *Yhat_dev, void *stream);
 
@@ -206,7 +207,8 @@ int pvmvmd_server_mvm_grouped(const pvmvmd_mvm_batch_job *jobs, int count, void 
  * memory is reserved up front by its own allocator or pool (a cudaMalloc
  * from inside the library could fail or fragment that pool), or a
  * latency-critical loop that cannot afford the regular call's first-use
- * allocation, or that of replacing an outgrown buffer.  It always runs the tensor-core digit product (also for B = 1),
+ * allocation, or the synchronisation of replacing an outgrown buffer.  It
+ * always runs the tensor-core digit product (also for B = 1),
  * whose fp16 digit tiles then live in one file-scope __device__ array of
  * PVMVMD_NOALLOC_SCRATCH_BYTES (16 MiB) that every GPU which loads the
  * library holds until the process exits.  The tiles take

@@ -7,20 +7,18 @@
 // it waits for the kernel before, and a call that has sized it serves every
 // smaller one, whichever of the two paths that takes.  Keying by stream lets calls on
 // different streams overlap without sharing a buffer; calls on one stream
-// are ordered, so they may share one.  A buffer that must grow is replaced by
-// one of at least twice its size and kept beside it, since kernels in flight
-// and captured graphs may still use it; the kept ones come to less than the
-// one in use.  Where memory is short those that no capture has been handed
-// are given back, after the stream has drained, for a buffer of just the size
-// that is needed; a graph may be replayed at any time, so a buffer that one was
-// handed is kept for good, and the call is refused if that leaves too little.  A
-// buffer cannot grow while the stream is being captured: make one call of the
+// are ordered, so they may share one.  A buffer that must grow is given back
+// once the stream has drained; one that a captured call was handed is kept
+// for good instead, since its graph may be replayed at any time, and then the
+// new one has at least twice its size, so that those kept come to less than the
+// one in use.  Otherwise growth is rounded up by kGrowSlack at most.  Where that
+// is not to be had the call gets just what it needs, or is refused.  A buffer
+// cannot grow while the stream is being captured: make one call of the
 // largest shape before capturing.
 #include <algorithm>
 #include <map>
 #include <mutex>
 #include <tuple>
-#include <vector>
 
 #include "launch.h"
 
@@ -30,9 +28,9 @@ namespace {
 struct Buf {
     void *ptr = nullptr;
     size_t bytes = 0;
-    bool captured = false;    // handed to a call under capture
-    std::vector<void *> old;  // outgrown, of no capture
+    bool captured = false;  // handed to a call under capture
 };
+constexpr size_t kGrowSlack = 32u << 20;
 std::mutex g_bufs_mu;
 std::map<std::tuple<int, int, cudaStream_t>, Buf> g_bufs;
 }  // namespace
@@ -56,28 +54,20 @@ cudaError_t stream_scratch(int purpose, size_t need, cudaStream_t s, void **out)
     std::lock_guard<std::mutex> lock(g_bufs_mu);
     Buf &b = g_bufs[std::make_tuple(purpose, dev, s)];
     if (b.bytes < need) {
-        size_t bytes = std::max(need, 2 * b.bytes);
+        size_t bytes = std::max(need, b.captured ? 2 * b.bytes : std::min(2 * b.bytes, b.bytes + kGrowSlack));
         void *p = nullptr;
+        if (b.ptr && !b.captured) {
+            if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
+            cudaFree(b.ptr);
+            b = Buf{};
+        }
         e = cudaMalloc(&p, bytes);
-        if (e == cudaErrorMemoryAllocation) {
+        if (e == cudaErrorMemoryAllocation && bytes > need) {
             (void)cudaGetLastError();
-            if ((b.ptr && !b.captured) || !b.old.empty()) {
-                if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
-                for (void *o : b.old) cudaFree(o);
-                b.old.clear();
-                if (!b.captured) {
-                    cudaFree(b.ptr);
-                    b.ptr = nullptr;
-                    b.bytes = 0;
-                }
-            }
             e = cudaMalloc(&p, bytes = need);
         }
         if (e != cudaSuccess) return e;
-        if (b.ptr && !b.captured) b.old.push_back(b.ptr);
-        b.ptr = p;
-        b.bytes = bytes;
-        b.captured = false;
+        b = Buf{p, bytes, false};
     }
     if (!b.captured) {
         cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
