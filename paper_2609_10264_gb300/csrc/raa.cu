@@ -1261,6 +1261,7 @@ cudaError_t launch_pdl(const void *fn, dim3 grid, dim3 block, size_t smem, cudaS
 }  // namespace
 
 // Bitmap of N bits plus 512 keystream words; covers N up to 8 * PVMVMD_MAX_K.
+// The support and suffix sums of k_syndrome_scan: t up to 25599.
 constexpr size_t kSampleMaxSmem = 200 * 1024;
 
 cudaError_t launch_sample_sparse(const pvmvmd_key &key, uint32_t tag, uint64_t idx0, uint32_t N,
@@ -1282,6 +1283,10 @@ cudaError_t launch_syndrome_scan(const uint32_t *pi2inv, const uint32_t *v2p, co
                                  cudaStream_t s) {
     if (count == 0) return cudaSuccess;
     const size_t smem = (2 * (size_t)t + 1) * sizeof(uint32_t);
+    if (smem > kSampleMaxSmem) return cudaErrorInvalidValue;
+    const cudaError_t attr = func_attr((const void *)k_syndrome_scan, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)kSampleMaxSmem);
+    if (attr != cudaSuccess) return attr;
     const unsigned grid = count * scan_tiles(N);
     const DebugWait dbg = debug_wait();
     const bool inject = dbg.site == PVMVMD_DEBUG_WAIT_SCAN;

@@ -275,6 +275,32 @@ def test_boost_mode_matches_standard_mode(pv, wl, m, K, B):
     ctx.destroy()
 
 
+@pytest.mark.parametrize("t2", [256, 257, 6143, 6144, 7000])
+def test_batch_verification_secondary_sparsity(pv, t2):
+    """Secondary challenges on both sides of the tiles' longest support and of the
+    shared memory that a kernel has without asking for more."""
+    rng = np.random.default_rng(t2)
+    B, m, n = 3, 8, 300
+    Ws = rng.integers(-128, 128, size=(B, m, n), dtype=np.int8)
+    xs = rng.integers(0, Q, size=(B, n)).astype(np.uint32)
+    ys = np.stack([oracle.server_mvm(Ws[b], xs[b]) for b in range(B)])
+    params = pv.pvmvmd_bv_params()
+    params.t2 = t2
+    ctx = pv.pvmvmd_bv_preprocess(to_dev(Ws), key=56, params=params)
+    chal = pv.pvmvmd_bv_challenge(ctx, key=57)
+    u = pv.pvmvmd_bv_server_project(ctx, chal)
+    assert pv.as_u32(pv.pvmvmd_bv_check(ctx, to_dev(xs), to_dev(ys), chal, u, key2=58)).tolist() == [1]
+    sec = pv.as_u32(pv.device_view(ctx.chal2, ctx.ell2 * 2 * t2).view(ctx.ell2, 2 * t2))
+    for j in range(ctx.ell2):
+        s_o, v_o = oracle.sample_sparse(oracle.key_from_seed(58), oracle.TAG_BV_SECONDARY, j, ctx.N2, t2)
+        assert np.array_equal(sec[j], np.concatenate([s_o, v_o]))
+    ub = u.clone()
+    tamper(pv, ub, 1, 899, 3)
+    assert pv.as_u32(pv.pvmvmd_bv_check(ctx, to_dev(xs), to_dev(ys), chal, ub, key2=58)).tolist() == [0]
+    assert pv.pvmvmd_device_status() == 0
+    ctx.destroy()
+
+
 @pytest.mark.parametrize("B,m,n", [(3, 40, 30), (4, 96, 64), (2, 700, 600)])
 def test_batch_verification_protocol2(pv, wl, B, m, n):
     """Protocol 2 on the GPU against the oracle: the preprocessed Qs and
