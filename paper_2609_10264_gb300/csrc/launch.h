@@ -105,7 +105,7 @@ cudaError_t launch_syndrome_gather(const uint32_t *pi1inv, uint32_t n, uint32_t 
                                    unsigned long long *status = nullptr, uint32_t nclear = 0);
 
 // Tiled syndrome (k_syndrome_tiles, then the gather) for `count` freshly
-// sampled vectors of sparsity t <= 256 and any N: sparse_out [count][2t] (may
+// sampled vectors of sparsity t <= 512 and any N: sparse_out [count][2t] (may
 // be null), F [count][N] scratch, status count * scan_tiles(N) words, zero at
 // the call and zero again after it.  With u non-null also
 // u[q][k] = sum_j e_{q,j} Qm[supp_{q,j}][k] for k < K.  pdl: launched as

@@ -15,11 +15,11 @@ __device__ __forceinline__ int bitlen32(uint32_t v) { return v ? 32 - __clz(v) :
 // t <= kTileMaxT without a bitmap: a draw is compared with the list itself
 // (16 bytes per shared-memory read, every lane the same address).  list is
 // 16-byte aligned and holds kTileMaxT words.
-constexpr uint32_t kTileMaxT = 256;
+constexpr uint32_t kTileMaxT = 512;
 __device__ void warp_sample_support_short(const pvmvmd_key &key, uint32_t tag, uint64_t sidx, uint32_t N,
                                           uint32_t t, uint32_t *words, uint32_t *list, int lane) {
     // unused slots hold a value no draw takes (draws are below N)
-    for (uint32_t i = lane; i < kTileMaxT; i += 32) list[i] = 0xffffffffu;
+    for (uint32_t i = lane; i < ((t + 3) & ~3u); i += 32) list[i] = 0xffffffffu;
     __syncwarp();
     if (N <= 1) {
         if (lane == 0) list[0] = 0u;
@@ -122,8 +122,11 @@ __device__ __forceinline__ void syndrome_tile(const TileArgs &A, uint32_t block)
     const uint32_t N = A.N, t = A.t, ucols = A.ucols;
     const int K = A.K;
     __shared__ __align__(16) uint32_t s_list[kTileMaxT];
-    __shared__ uint32_t s_supp[kTileMaxT], s_val[kTileMaxT], s_suf[kTileMaxT + 1];
-    __shared__ uint32_t s_words[2][512];
+    __shared__ uint32_t s_val[kTileMaxT];
+    // the keystream, then the sorted support and the suffix sums of the values
+    __shared__ uint32_t s_words[2 * kTileMaxT + 1];
+    static_assert(kTileMaxT == 512, "a draw's 512 words of keystream");
+    uint32_t *s_supp = s_words, *s_suf = s_words + kTileMaxT;
     __shared__ uint32_t s_wsum[kScanThreads / 32], s_agg, s_prefix;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int nw = kScanThreads / 32;
@@ -155,8 +158,8 @@ __device__ __forceinline__ void syndrome_tile(const TileArgs &A, uint32_t block)
 
     // ---- e: warp 0 the support, warp 1 the values
     const uint64_t vidx = A.idx0 + vec;
-    if (warp == 0) warp_sample_support_short(A.key, A.tag, 2 * vidx, N, t, s_words[0], s_list, lane);
-    else if (warp == 1) warp_sample_values(A.key, A.tag, 2 * vidx + 1, t, s_words[1], s_val, lane);
+    if (warp == 0) warp_sample_support_short(A.key, A.tag, 2 * vidx, N, t, s_words, s_list, lane);
+    else if (warp == 1) warp_sample_values(A.key, A.tag, 2 * vidx + 1, t, s_words + 512, s_val, lane);
     __syncthreads();
     if (warp == nw - 1) {  // s_suf[j] = sum_{j' >= j} e_{j'}; s_suf[t] = 0
         const uint32_t per = (t + 31) / 32;
@@ -176,8 +179,8 @@ __device__ __forceinline__ void syndrome_tile(const TileArgs &A, uint32_t block)
         }
         if (lane == 0) s_suf[t] = 0;
     }
-    if (tid < t) {  // ascending support by rank (entries distinct; unused slots are larger than all)
-        const uint32_t v = s_list[tid];
+    for (uint32_t i = tid; i < t; i += kScanThreads) {  // ascending support by rank (entries distinct, unused slots larger)
+        const uint32_t v = s_list[i];
         uint32_t rk = 0;
         for (uint32_t h = 0; h < t; h += 4) {
             const uint4 a = *reinterpret_cast<const uint4 *>(s_list + h);

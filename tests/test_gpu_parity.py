@@ -124,8 +124,12 @@ def test_small_parameters_round_trip(pv, wl):
     (300, 1025, 3, {}),                             # N_x = 8200: a last tile of 8 positions
     (683, 4101, 2, dict(rate=3)),                   # N_x = 12303, N_y = 2049: unaligned rows, a tile of 1
     (16, 1100, 30, {}), (16, 1100, 31, {}),         # 150 and 155 tiles, on both sides of one per SM
-    (40, 1030, 2, dict(t_x=256, t_y=256)),          # the longest support the tiles sort
-    (40, 1030, 2, dict(t_x=257, t_y=257)),          # one more: the paths without tiles
+    (40, 1030, 2, dict(t_x=256, t_y=256)),          # a support of one entry per thread
+    (40, 1030, 2, dict(t_x=257, t_y=257)),          # one more
+    (65, 1030, 2, dict(t_x=509, t_y=511)),          # almost, and
+    (64, 1030, 2, dict(t_x=512, t_y=512)),          # the longest support the tiles sort; all of N_y
+    (65, 1030, 2, dict(t_x=513, t_y=513)),          # one more: the paths without tiles
+    (64, 6000, 3, dict(t_x=500)),                   # a code longer than one CTA's shared memory
     (40, 1030, 2, dict(t_x=1, t_y=1, ell=3)),       # one support; an odd number of challenges
 ])
 def test_tiled_syndrome_round_trip(pv, wl, m, K, B, kw):
@@ -1006,6 +1010,7 @@ def test_small_batches_captured_after_another_call(pv):
     (1030, 1001, 310, {}),                         # unaligned rows of P^T
     (683, 64, 500, dict(rate=3, ell=3, t_y=1)),    # N_y = 2049, an odd number of challenges
     (4096, 520, 100, dict(t_y=256, ell=1)),        # 256-column CTAs
+    (300, 96, 700, dict(t_y=512)),                 # the longest challenge support
     (2048, 96, 300, dict(ell=16)),                 # the most challenges
 ])
 def test_large_decode_in_one_kernel(pv, wl, m, K, B, kw):
