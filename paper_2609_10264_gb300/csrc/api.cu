@@ -718,18 +718,34 @@ int encode_batch(pvmvmd_ctx *ctx, const uint32_t *X_dev, int B, const pvmvmd_key
     uint32_t *stp = static_cast<uint32_t *>(st_dev);
     const CodeDev &d = ctx->gx;
     const bool fits = syndrome_fused_fits(ctx->Nx, ctx->t_x);
-    // A code too long for that, and vectors enough for the SMs: a CTA per
-    // vector, two per SM.  Against the lanes, back to back and alone (one
-    // encode and a field add, about 8 us of it launches): K = 8192, B = 256: 55
-    // against 83 us and 71 against 85; B = 100: 23 / 45 and 44 / 46; B = 64: 15 /
-    // 40 but 44 / 42; K = 5700, B = 32: 7 / 36 and 36 / 37; K = 13000, B = 152:
-    // 54 / 97 and 74 / 99, B = 128: 47 / 68 but 74 / 70.  The lines keep both.
-    if (d.slices && B >= (ctx->Nx <= 48 * 1024 ? kLaneMinBatch : ctx->Nx <= 80 * 1024 ? 2 * sm_count() / 3 : sm_count())) {
+    const bool lanes = B >= kLaneMinBatch && ctx->laux && !fits;
+    const bool tiles = syndrome_tiles_eligible((uint32_t)ctx->t_x);
+    const uint32_t ntiles = scan_tiles((uint32_t)ctx->Nx);
+    // A code too long for that: a CTA per vector, two per SM, slice by slice.
+    //  * Against the lanes, back to back and alone (one encode and a field add,
+    //    about 8 us of it launches): K = 8192, B = 256: 55 against 83 us and 71
+    //    against 85; B = 100: 23 / 45 and 44 / 46; B = 64: 15 / 40 but 44 / 42;
+    //    K = 5700, B = 32: 7 / 36 and 36 / 37; K = 13000, B = 152: 54 / 97 and
+    //    74 / 99, B = 128: 47 / 68 but 74 / 70.  The lines keep both.
+    //  * Against the tiles, whose every CTA draws the whole support, so that a
+    //    call costs B N_x t_x where it costs N_x here: the line is where one call
+    //    alone takes about as long (back to back and alone): t_x = 333, B = 16:
+    //    K = 5700: 7.9 against 27 us and 50 against 46, K = 8192: 9.2 / 31 and 57 /
+    //    48, K = 10000: 12 / 49 and 70 / 71; t_x = 156, B = 31: K = 5700: 8.9 / 29
+    //    and 47 / 49, K = 8192: 11 / 36 and 55 / 51, K = 13000: 18 / 58 but 84 / 74.
+    //  * Where the scratch holds fewer vectors than the batch has, or the tiles
+    //    do not take the support: K = 8192, 16 vectors one by one 64 / 104.
+    bool sliced = false;
+    if (d.slices && lanes)
+        sliced = B >= (ctx->Nx <= 48 * 1024 ? kLaneMinBatch : ctx->Nx <= 80 * 1024 ? 2 * sm_count() / 3 : sm_count());
+    else if (d.slices)
+        sliced = !tiles || B > ctx->sb || (uint64_t)B * ctx->t_x > (uint64_t)33 * sm_count();
+    if (sliced) {
         PV_CUDA(launch_syndrome_sliced(*key, kTagMask, 0, ctx->Nx, ctx->t_x, (uint32_t)B, d.slices, d.v1m, ctx->K, stp,
                                        X_dev, Xhat_dev, s));
         return PVMVMD_OK;
     }
-    if (B >= kLaneMinBatch && ctx->laux && !fits) {
+    if (lanes) {
         // vectors as lanes: every permutation step moves whole rows (a code
         // that fits one CTA's shared memory stays on chip in the fused kernel)
         for (int b0 = 0; b0 < B; b0 += ctx->sb) {
@@ -742,16 +758,19 @@ int encode_batch(pvmvmd_ctx *ctx, const uint32_t *X_dev, int B, const pvmvmd_key
         }
         return PVMVMD_OK;
     }
-    // A code of more than four tiles and a batch of at most one tile per SM:
+    // A code of more than four tiles (more where the support is long, since each
+    // draws it by itself) and a batch of at most one tile per SM:
     // small CTAs, one per tile, finish sooner than a CTA per vector.  Measured
     // (one encode and a field add, graph replay, about 8 us of it launches):
     // K = 4096, B = 8: 16.8 against 25.2 us; K = 2560, B = 8: 17.6 against
-    // 21.4; K = 1001 (four tiles), B = 1: 13.7 and 13.7; back to back the two
+    // 21.4; K = 1001 (four tiles), B = 1: 13.7 and 13.7; t_x = 335, B = 1, alone:
+    // K = 4096 32.5 against 34, K = 2048 (eight tiles) 33 against 28; back to back the two
     // tie at one tile per SM (K = 4096, B = 8: 7.1 against 6.7 us a call) and
-    // beyond it the CTA per vector wins (B = 16: 12.1 against 6.7).
-    const bool tiles = syndrome_tiles_eligible((uint32_t)ctx->t_x);
-    const uint32_t ntiles = scan_tiles((uint32_t)ctx->Nx);
-    if (fits && !(tiles && ntiles > 4 && (uint64_t)B * ntiles <= (uint64_t)sm_count())) {
+    // beyond it the CTA per vector wins (B = 16: 12.1 against 6.7).  It needs no
+    // scratch either: a batch of more vectors than the scratch holds stays whole.
+    const bool spread = tiles && ntiles > 4 && 32 * ntiles > (uint32_t)ctx->t_x && B <= ctx->sb &&
+                        (uint64_t)B * ntiles <= (uint64_t)sm_count();
+    if (fits && !spread) {
         // sample, scan and gather in one launch per batch, no scratch
         PV_CUDA(launch_syndrome_fused(*key, kTagMask, 0, ctx->Nx, ctx->t_x, (uint32_t)B, d.pi1inv, d.pi2,
                                       d.v2m, d.v1pm, ctx->K, ctx->rate, stp, X_dev, Xhat_dev, s));

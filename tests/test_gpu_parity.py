@@ -170,6 +170,11 @@ def test_code_tables_sampled_on_device(pv, N):
     (16001, 40, dict(rate=3, t_x=1)),              # N_x = 48003: ragged tables, odd outputs, one support
     (8200, 99, {}), (8200, 110, {}),               # lanes and slices, on both sides of the rule
     (13000, 160, {}),                              # the longest codes that two CTAs per SM hold
+    (8192, 15, dict(t_x=333)), (8192, 16, dict(t_x=333)),  # tiles and slices, on both sides of the rule (152 SMs)
+    (8192, 3, dict(scratch_batch=2)),              # more vectors than the scratch holds
+    (6000, 2, dict(t_x=513)),                      # a support longer than the tiles take
+    (4096, 4, dict(scratch_batch=3)),              # a code that fits one CTA: whole, or
+    (14000, 4, dict(scratch_batch=3)),             # tiles in chunks where nothing else takes it
     (15000, 300, dict(scratch_batch=270)),         # beyond them: lanes, in chunks of 270 and 30
 ])
 def test_sliced_encode(pv, wl, K, B, kw):
