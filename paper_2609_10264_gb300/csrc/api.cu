@@ -920,6 +920,26 @@ bool overlaps(const void *a, const void *b, size_t bytes) {
     return x < y + bytes && y < x + bytes;
 }
 
+// The verification on the context's side stream, the decrypt on s, joined.
+int decode_beside(pvmvmd_ctx *ctx, const void *st_dev, const uint32_t *mask_out_dev, const uint32_t *Xhat_dev,
+                  const uint32_t *Yhat_dev, int B, const pvmvmd_key *challenge_key, uint32_t *Y_dev,
+                  int32_t *accept_dev, cudaStream_t s) {
+    const bool early = !ctx->captured && !ctx->on_caller;
+    int st = PVMVMD_OK;
+    if (early && (st = challenge_chain(ctx, challenge_key, ctx->side))) return st;
+    PV_CUDA(cudaEventRecord(ctx->fork, s));
+    PV_CUDA(cudaStreamWaitEvent(ctx->side, ctx->fork, 0));
+    if (!early && (st = challenge_chain(ctx, challenge_key, ctx->side))) return st;
+    ctx->on_caller = false;
+    PV_CUDA(launch_check(Xhat_dev, ctx->K, Yhat_dev, ctx->m, ctx->g, ctx->u, (uint32_t)ctx->ell, B, accept_dev,
+                         ctx->side));
+    PV_CUDA(launch_decrypt(ctx->PT, ctx->m, static_cast<const uint32_t *>(st_dev), ctx->t_x, (uint32_t)ctx->Nx,
+                           Yhat_dev, B, Y_dev, s, mask_out_dev));
+    PV_CUDA(cudaEventRecord(ctx->join, ctx->side));
+    PV_CUDA(cudaStreamWaitEvent(s, ctx->join, 0));
+    return PVMVMD_OK;
+}
+
 // Verify and decrypt: Y = Yhat - P e_x from st, or Y = Yhat - mask_out when
 // mask_out is given (boost mode).
 //  * A large decrypt: one kernel on the caller's stream (launch_decode).
@@ -959,26 +979,23 @@ int decode_verify_batch(pvmvmd_ctx *ctx, const void *st_dev, const uint32_t *mas
         PV_CUDA(launch_decode(c, s));
         return PVMVMD_OK;
     }
-    const cudaStream_t cs = in_place ? s : ctx->side;
-    int st = PVMVMD_OK;
     if (!in_place) {
-        const bool early = !ctx->captured && !ctx->on_caller;
-        if (early && (st = challenge_chain(ctx, challenge_key, cs))) return st;
-        PV_CUDA(cudaEventRecord(ctx->fork, s));
-        PV_CUDA(cudaStreamWaitEvent(cs, ctx->fork, 0));
-        if (!early && (st = challenge_chain(ctx, challenge_key, cs))) return st;
-        ctx->on_caller = false;
-    } else {
-        ctx->on_caller = true;
-        if ((st = challenge_chain(ctx, challenge_key, cs))) return st;
+        const int st = decode_beside(ctx, st_dev, mask_out_dev, Xhat_dev, Yhat_dev, B, challenge_key, Y_dev,
+                                     accept_dev, s);
+        // not joined: what the side stream has of the call must not run beside
+        // the next one, which may use the scratch on another stream
+        if (st != PVMVMD_OK && capture == cudaStreamCaptureStatusNone) {
+            cudaStreamSynchronize(ctx->side);
+            (void)cudaGetLastError();
+        }
+        return st;
     }
-    PV_CUDA(launch_check(Xhat_dev, ctx->K, Yhat_dev, ctx->m, ctx->g, ctx->u, (uint32_t)ctx->ell, B, accept_dev, cs));
+    ctx->on_caller = true;
+    const int st = challenge_chain(ctx, challenge_key, s);
+    if (st) return st;
+    PV_CUDA(launch_check(Xhat_dev, ctx->K, Yhat_dev, ctx->m, ctx->g, ctx->u, (uint32_t)ctx->ell, B, accept_dev, s));
     PV_CUDA(launch_decrypt(ctx->PT, ctx->m, static_cast<const uint32_t *>(st_dev), ctx->t_x, (uint32_t)ctx->Nx,
                            Yhat_dev, B, Y_dev, s, mask_out_dev));
-    if (!in_place) {
-        PV_CUDA(cudaEventRecord(ctx->join, ctx->side));
-        PV_CUDA(cudaStreamWaitEvent(s, ctx->join, 0));
-    }
     return PVMVMD_OK;
 }
 }  // namespace
