@@ -163,6 +163,10 @@ __device__ __forceinline__ void chacha20_block_dev(const pvmvmd_key &key, uint32
 }
 
 // ---------------------------------------------------------------- memory ordering
+// A kernel launched with programmatic serialisation is in place before the
+// kernels before it have written what it reads after griddepcontrol.wait. The
+// read-only path (__ldg, or const with __restrict__) is, in such a kernel, for what
+// does not change while it is there: the code tables, P^T and Q, and nothing else.
 __device__ __forceinline__ void st_release_u64(unsigned long long *p, unsigned long long v) {
     asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }

@@ -49,8 +49,7 @@ __device__ __forceinline__ uint4 ldg4(const uint32_t *p) {
 // in shared memory.
 constexpr int kVuCols = 64, kVuGroups = 4;
 __global__ void __launch_bounds__(kVuCols * kVuGroups) k_verify_u(const uint32_t *__restrict__ Qm, int K,
-                                                                 const uint32_t *__restrict__ chal, uint32_t t,
-                                                                 uint32_t *__restrict__ u) {
+                                                                 const uint32_t *chal, uint32_t t, uint32_t *u) {
     extern __shared__ uint32_t sm[];
     __shared__ uint32_t s_part[kVuGroups - 1][kVuCols];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -258,11 +257,9 @@ constexpr int kCheckBatch = 4;      // loads in flight per operand and thread
 constexpr int kCheckSlice = 2048;   // columns a CTA takes, where eight CTAs suffice
 constexpr int kCheckMaxCluster = 8;
 
-__global__ void __launch_bounds__(kCheckThreads, 4) k_check(const uint32_t *__restrict__ Xhat, int K,
-                                                           const uint32_t *__restrict__ Yhat, int m,
-                                                           const uint32_t *__restrict__ g,
-                                                           const uint32_t *__restrict__ u, uint32_t ell,
-                                                           int32_t *__restrict__ accept) {
+__global__ void __launch_bounds__(kCheckThreads, 4) k_check(const uint32_t *Xhat, int K, const uint32_t *Yhat,
+                                                           int m, const uint32_t *g, const uint32_t *u, uint32_t ell,
+                                                           int32_t *accept) {
     cg::cluster_group cluster = cg::this_cluster();
     __shared__ uint32_t s_part[4][kCheckThreads / 32];
     __shared__ uint32_t s_sum[4];

@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(kRingThreads, 2) k_gemv_ring(const __grid_cons
                 const uint4 *xp = reinterpret_cast<const uint4 *>(job.xhat + (size_t)(ct + i * T) * 16);
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    const uint4 xv = __ldg(xp + q);
+                    const uint4 xv = xp[q];  // written while this kernel was in place already: no read-only load
                     const uint32_t xs[4] = {xv.x, xv.y, xv.z, xv.w};
                     uint32_t u[4];
 #pragma unroll

@@ -77,8 +77,7 @@ struct NbArgs {
 // Digit planes of the batch, once per call: planes[j][p][v][k] (int8) is
 // digit p of centred x_hat[4j + v][k]; vectors past B are zero.  One thread
 // per four consecutive K-elements of one vector.
-__global__ void __launch_bounds__(256) k_nb_planes(const uint32_t *__restrict__ Xhat, int B, int K, int Bp,
-                                                  uint32_t *__restrict__ planes) {
+__global__ void __launch_bounds__(256) k_nb_planes(const uint32_t *Xhat, int B, int K, int Bp, uint32_t *planes) {
     // x_hat comes from the kernel before, and M may: the product, which reads M
     // without a wait of its own, may start only after it
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -89,7 +88,7 @@ __global__ void __launch_bounds__(256) k_nb_planes(const uint32_t *__restrict__ 
     const int b = (int)(gid / per_vec), q4 = (int)(gid % per_vec);
     uint32_t p[4] = {0u, 0u, 0u, 0u};
     if (b < B) {
-        const uint4 xv = __ldg(reinterpret_cast<const uint4 *>(Xhat + (size_t)b * K) + q4);
+        const uint4 xv = reinterpret_cast<const uint4 *>(Xhat + (size_t)b * K)[q4];
         const uint32_t xs[4] = {xv.x, xv.y, xv.z, xv.w};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
@@ -165,7 +164,7 @@ __global__ void __launch_bounds__(kMultiThreads, 2) k_gemv_nb(const __grid_const
                 uint4 t[8];
 #pragma unroll
                 for (int r = 0; r < 8; ++r)
-                    t[r] = __ldg(reinterpret_cast<const uint4 *>(job.planes + (size_t)(8 * h + r) * job.ldp) + c);
+                    t[r] = reinterpret_cast<const uint4 *>(job.planes + (size_t)(8 * h + r) * job.ldp)[c];
 #pragma unroll
                 for (int r = 0; r < 8; ++r) s_planes[(8 * h + r) * kNbStride + c] = t[r];
             }

@@ -1002,13 +1002,12 @@ __global__ void __launch_bounds__(128) k_lane_sample(pvmvmd_key key, uint32_t ta
 // C[pi2(k)][b] = v2_k (A e_b)_k: a thread walks kExpandSpan positions k of
 // four lanes in order with a pointer per lane into the sorted support, and
 // writes the four lanes of row pi2(k) with one 16-byte store.
-__global__ void __launch_bounds__(kLaneCta) k_lane_expand(const uint32_t *__restrict__ st,
-                                                         const uint32_t *__restrict__ S,
-                                                         const uint16_t *__restrict__ first, uint32_t t,
+__global__ void __launch_bounds__(kLaneCta) k_lane_expand(const uint32_t *st, const uint32_t *S,
+                                                         const uint16_t *first, uint32_t t,
                                                          uint32_t N, uint32_t L,
                                                          const uint32_t *__restrict__ pi2,
                                                          const uint32_t *__restrict__ v2m,
-                                                         uint4 *__restrict__ C) {
+                                                         uint4 *C) {
     asm volatile("griddepcontrol.wait;" ::: "memory");  // inputs come from the kernel before
     const uint32_t cols = lane_cols(L), Lq = lane_pad(L) / 4;
     const uint32_t g = blockIdx.y * cols + threadIdx.x % cols;
@@ -1026,15 +1025,15 @@ __global__ void __launch_bounds__(kLaneCta) k_lane_expand(const uint32_t *__rest
             // first support index with s_j >= k0: from the bucket of k0, then
             // past the few supports between the bucket's start and k0
             const uint32_t *supp = st + (size_t)b * 2 * t;
-            uint32_t lo = __ldg(first + (size_t)b * kLaneBuckets + (k0 >> lane_bshift(N)));
-            uint32_t nx = lo < t ? __ldg(supp + lo) : 0xffffffffu;
+            uint32_t lo = first[(size_t)b * kLaneBuckets + (k0 >> lane_bshift(N))];
+            uint32_t nx = lo < t ? supp[lo] : 0xffffffffu;
             while (nx < k0) {
                 ++lo;
-                nx = lo < t ? __ldg(supp + lo) : 0xffffffffu;
+                nx = lo < t ? supp[lo] : 0xffffffffu;
             }
             j[q] = lo;
             next[q] = nx;
-            cur[q] = __ldg(S + (size_t)b * (t + 1) + lo);
+            cur[q] = S[(size_t)b * (t + 1) + lo];
         }
     }
     for (uint32_t kb = k0; kb < k1; kb += 4) {  // k0 is a multiple of 4: 16-byte table loads
@@ -1061,8 +1060,8 @@ __global__ void __launch_bounds__(kLaneCta) k_lane_expand(const uint32_t *__rest
                 const uint32_t b = 4 * g + q;
                 while (next[q] < k) {
                     ++j[q];
-                    next[q] = j[q] < t ? __ldg(st + (size_t)b * 2 * t + j[q]) : 0xffffffffu;
-                    cur[q] = __ldg(S + (size_t)b * (t + 1) + j[q]);
+                    next[q] = j[q] < t ? st[(size_t)b * 2 * t + j[q]] : 0xffffffffu;
+                    cur[q] = S[(size_t)b * (t + 1) + j[q]];
                 }
                 o[q] = fmul_mont(cur[q], vk[u]);
             }
@@ -1072,8 +1071,8 @@ __global__ void __launch_bounds__(kLaneCta) k_lane_expand(const uint32_t *__rest
 }
 
 // agg[tau][b] = sum over the tile's positions of C[i][b].
-__global__ void __launch_bounds__(kLaneCta) k_lane_tile_sum(const uint4 *__restrict__ C, uint32_t N, uint32_t tile,
-                                                           uint32_t L, uint4 *__restrict__ agg) {
+__global__ void __launch_bounds__(kLaneCta) k_lane_tile_sum(const uint4 *C, uint32_t N, uint32_t tile, uint32_t L,
+                                                           uint4 *agg) {
     asm volatile("griddepcontrol.wait;" ::: "memory");  // inputs come from the kernel before
     const uint32_t cols = lane_cols(L), Lq = lane_pad(L) / 4, ntiles = (N + tile - 1) / tile;
     const uint32_t g = blockIdx.y * cols + threadIdx.x % cols;
@@ -1104,8 +1103,8 @@ __device__ __forceinline__ uint4 shfl_down4(uint4 v, int o) {
 __device__ __forceinline__ uint4 fsub4(uint4 a, uint4 b) {
     return make_uint4(fsub(a.x, b.x), fsub(a.y, b.y), fsub(a.z, b.z), fsub(a.w, b.w));
 }
-__global__ void __launch_bounds__(kCarryThreads) k_lane_carry(const uint4 *__restrict__ agg, uint32_t ntiles,
-                                                             uint32_t Lq, uint4 *__restrict__ carry) {
+__global__ void __launch_bounds__(kCarryThreads) k_lane_carry(const uint4 *agg, uint32_t ntiles, uint32_t Lq,
+                                                             uint4 *carry) {
     asm volatile("griddepcontrol.wait;" ::: "memory");  // inputs come from the kernel before
     __shared__ uint4 wsum[kCarryThreads / 32];
     const uint32_t g = blockIdx.x, c = threadIdx.x, lane = c & 31, warp = c >> 5;
@@ -1160,8 +1159,8 @@ __global__ void __launch_bounds__(kCarryThreads) k_lane_carry(const uint4 *__res
 
 // In place: C[i][b] <- v1_i (carry[tau][b] + sum_{i' >= i in tile tau} C[i'][b]),
 // with v1m = v1 R (Montgomery, R = 2^32) so that each product is one REDC.
-__global__ void __launch_bounds__(kLaneCta, 4) k_lane_scan(uint4 *__restrict__ C, uint32_t N, uint32_t tile, uint32_t L,
-                                                       const uint4 *__restrict__ carry,
+__global__ void __launch_bounds__(kLaneCta, 4) k_lane_scan(uint4 *C, uint32_t N, uint32_t tile, uint32_t L,
+                                                       const uint4 *carry,
                                                        const uint32_t *__restrict__ v1m) {
     asm volatile("griddepcontrol.wait;" ::: "memory");  // inputs come from the kernel before
     const uint32_t cols = lane_cols(L), Lq = lane_pad(L) / 4, ntiles = (N + tile - 1) / tile;
@@ -1192,7 +1191,7 @@ __global__ void __launch_bounds__(kLaneCta, 4) k_lane_scan(uint4 *__restrict__ C
 // out[b][j] = addend[b][j] + sum_{c<r} C[pi1^-1(r j + c)][b] for kGatherJ
 // outputs and the CTA's lanes, transposed through shared memory so that out
 // rows are written 128 bytes at a time.  addend may be null or alias out.
-__global__ void __launch_bounds__(kLaneCta, 4) k_lane_gather(const uint4 *__restrict__ C,
+__global__ void __launch_bounds__(kLaneCta, 4) k_lane_gather(const uint4 *C,
                                                          const uint32_t *__restrict__ pi1inv,
                                                          uint32_t r, uint32_t n, uint32_t L,
                                                          const uint32_t *addend, uint32_t *out) {

@@ -29,7 +29,7 @@ __global__ void k_lift_i16(const int16_t *__restrict__ W, size_t n, uint32_t *__
 // y = 256 y + y_lo over F_q (y holds y_hi on entry).  Launched beside the
 // product that writes them, which it waits for (a 4096 x 2560 product of 8
 // vectors 12.8 -> 12.4 us, its round trip 46.4 -> 45.0).
-__global__ void k_combine_256(uint32_t *__restrict__ y, const uint32_t *__restrict__ ylo, size_t n) {
+__global__ void k_combine_256(uint32_t *y, const uint32_t *ylo, size_t n) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (i >= n) return;

@@ -156,3 +156,21 @@ def test_operand_kernels_wait_before_they_signal():
         body = re.search(r"__global__[^;{]*\b" + kernel + r"\(.*?\n}\n", text, flags=re.S).group(0)
         wait, signal = body.find("griddepcontrol.wait;"), body.find("griddepcontrol.launch_dependents;")
         assert 0 <= wait < signal, kernel
+
+
+@pytest.mark.parametrize("name,kernel,written", [
+    ("gemv.cu", "k_gemv_ring", ["xhat", "xp"]), ("gemv_small.cu", "k_nb_planes", ["Xhat"]),
+    ("gemv_small.cu", "k_gemv_nb", ["planes"]), ("weights16.cu", "k_combine_256", ["y", "ylo"]),
+    ("decode.cu", "k_verify_u", ["chal"]), ("decode.cu", "k_check", ["Xhat", "Yhat", "g", "u"]),
+    ("raa.cu", "k_syndrome_gather", ["F", "addend"]), ("raa.cu", "k_lane_expand", ["st", "S", "first"]),
+    ("raa.cu", "k_lane_tile_sum", ["C"]), ("raa.cu", "k_lane_carry", ["agg"]), ("raa.cu", "k_lane_scan", ["C", "carry"]),
+    ("raa.cu", "k_lane_gather", ["C", "addend"]), ("raa.cu", "k_syndrome_fused", ["addend"]),
+    ("raa.cu", "k_syndrome_sliced", ["addend"])])
+def test_early_kernels_read_what_is_being_written_coherently(name, kernel, written):
+    """Kernels launched before the kernel before them has finished do not read its
+    output through the read-only path."""
+    text = open(os.path.join(ROOT, "paper_2609_10264_gb300", "csrc", name)).read()
+    head, body = re.search(r"\b" + kernel + r"\(([^;{]*?)\) ?{(.*?)\n}\n", text, flags=re.S).groups()
+    for w in written:
+        assert not re.search(r"__restrict__ " + w + r"\b", head), w
+        assert not re.search(r"__ldg\((reinterpret_cast<[^>]*>\()?(\w+\.)?" + w + r"\b", body), w
