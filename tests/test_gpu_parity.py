@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 
 import oracle
-from gpu_util import (Q, assert_equal_report, ctx_tables, exact_product, field, pt_columns, q_columns,
+from gpu_util import (Q, assert_equal_report, ctx_tables, exact_product, field, key_bound_error, pt_columns, q_columns,
                       sample_rows, tamper,
                       to_dev)
 
@@ -1070,7 +1070,9 @@ def test_decodes_of_every_route_in_turn(pv, wl):
     """Decodes of one context that take the side stream, the caller's stream (Y
     over Y_hat), one kernel (a large batch), boost mode and a captured graph,
     queued one after the other without a wait: the challenges' shared scratch
-    is handed from one to the next, and every output and verdict is exact."""
+    is handed from one to the next, and every output and verdict is exact.  A
+    verdict that rests on another call's challenges shows: vectors 2 and 3 are
+    wrong in ways that the challenges of one key each cannot see."""
     import torch
     m, K, B = 600, 520, 400
     W = wl.weights_uniform(m, K, 81)
@@ -1081,6 +1083,11 @@ def test_decodes_of_every_route_in_turn(pv, wl):
     Yh = pv.pvmvmd_server_mvm(Wd, Xh)
     bad = Yh.clone()
     tamper(pv, bad, 1, 17, 5)
+    keys, at = (201, 202, 203), (5, 300, 599)
+    for b, key in ((2, keys[0]), (3, keys[1])):
+        for i, err in zip(at, key_bound_error(83, m, key, at)):
+            tamper(pv, bad, b, i, err)
+    verdict = lambda k, key: [[1, 0, int(key == keys[0]), int(key == keys[1])][b] if b < 4 else 1 for b in range(k)]
     mask_in, mask_out, _ = pv.pvmvmd_boost_prepare(ctx, B, key=84)
     exp = to_dev(field(exact_product(W, x)))
     exp_bad = pv.pvmvmd_decode_verify(ctx, st, Xh, bad, 85)[0]
@@ -1092,28 +1099,29 @@ def test_decodes_of_every_route_in_turn(pv, wl):
     for turn in range(3):
         got = []
         for i in range(40):
-            key = 100 + 50 * turn + i
+            key = keys[i % 3]
             if i % 5 == 0:
-                got.append((4, *pv.pvmvmd_decode_verify(ctx, *small, key)))
+                got.append((4, key, *pv.pvmvmd_decode_verify(ctx, *small, key)))
             elif i % 5 == 1:
                 Yip = small[2].clone()
-                got.append((4, *pv.pvmvmd_decode_verify(ctx, *small, key, Y=Yip)) if i % 2 else
-                           (4, Yip, pv.pvmvmd_decode_verify(ctx, small[0], small[1], Yip, key, Y=Yip)[1]))
+                got.append((4, key, *pv.pvmvmd_decode_verify(ctx, *small, key, Y=Yip)) if i % 2 else
+                           (4, key, Yip, pv.pvmvmd_decode_verify(ctx, small[0], small[1], Yip, key, Y=Yip)[1]))
             elif i % 5 == 2:
-                got.append((B, *pv.pvmvmd_decode_verify(ctx, st, Xh, bad, key)))
+                got.append((B, key, *pv.pvmvmd_decode_verify(ctx, st, Xh, bad, key)))
             elif i % 5 == 3:
-                got.append((4, *pv.pvmvmd_boost_decode_verify(ctx, mask_out[:4].contiguous(), small[1], small[2], key)))
+                got.append((4, key, *pv.pvmvmd_boost_decode_verify(ctx, mask_out[:4].contiguous(), small[1], small[2],
+                                                                   key)))
             elif graph is not None:
                 graph.replay()
-                got.append((4, Yg.clone(), ag.clone()))
+                got.append((4, keys[1], Yg.clone(), ag.clone()))
         torch.cuda.synchronize()
-        for k, Y, acc in got:
+        for i, (k, key, Y, acc) in enumerate(got):
             assert torch.equal(Y, exp_bad[:k]) and torch.equal(Y[0], exp[0])
-            assert acc.tolist() == [0 if b == 1 else 1 for b in range(k)]
+            assert acc.tolist() == verdict(k, key), (turn, i, key)
         if turn == 0:  # from the second turn on with a captured call among them
             graph = torch.cuda.CUDAGraph()
             with torch.cuda.graph(graph, stream=s):
-                pv.pvmvmd_decode_verify(ctx, *small, 77, Y=Yg, accept=ag, stream=s)
+                pv.pvmvmd_decode_verify(ctx, *small, keys[1], Y=Yg, accept=ag, stream=s)
     assert pv.pvmvmd_device_status() == 0
     ctx.destroy()
 
