@@ -1,6 +1,7 @@
 // C ABI of the pvMVMD library (include/pvmvmd.h): parameter resolution, the
-// host-side sampling of the public RAA codes, context management, and the
-// ordering of the device kernels for each protocol call.
+// host's sampler of the public RAA codes (contexts sample theirs on the
+// device), context management, and the ordering of the device kernels for each
+// protocol call.
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>

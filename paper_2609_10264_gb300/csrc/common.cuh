@@ -75,10 +75,6 @@ __host__ __device__ __forceinline__ uint32_t fmul_mont(uint32_t a, uint32_t b_m)
     return u >= kQ ? u - kQ : u;
 #endif
 }
-// b -> b R mod q (host table preparation).
-__host__ __device__ __forceinline__ uint32_t to_mont(uint32_t b) {
-    return (uint32_t)(((uint64_t)b << 32) % kQ);
-}
 
 // Signed 64-bit integer -> canonical representative.
 __host__ __device__ __forceinline__ uint32_t fred_signed(int64_t v) {
@@ -90,9 +86,6 @@ __host__ __device__ __forceinline__ uint32_t fred_signed(int64_t v) {
     int64_t r = v % (int64_t)kQ;
     return (uint32_t)(r < 0 ? r + (int64_t)kQ : r);
 #endif
-}
-__host__ __device__ __forceinline__ uint32_t flift_i8(int8_t w) {
-    return w < 0 ? kQ + (uint32_t)(int32_t)w : (uint32_t)w;
 }
 
 // Canonical x in [0, q) -> centred c in [-(q-1)/2, (q-1)/2] -> four signed
@@ -185,15 +178,11 @@ __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long
     asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
 }
-__device__ __forceinline__ void st_release_u32(uint32_t *p, uint32_t v) {
-    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
 __device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t *p) {
     uint32_t v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
-__device__ __forceinline__ uint32_t ld_cg_u32(const uint32_t *p) { return __ldcg(p); }
 
 __device__ __forceinline__ void record_error(uint32_t *err, uint32_t bit) {
     if (err) atomicOr(err, bit);

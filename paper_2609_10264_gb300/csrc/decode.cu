@@ -347,14 +347,15 @@ __global__ void __launch_bounds__(kCheckThreads, 4) k_check(const uint32_t *Xhat
 //   the decrypt, all but its last wave of resident CTAs,
 //   the check of one vector each, from u and g,
 //   the rest of the decrypt.
-// A CTA waits only for CTAs of lower index, which the GPU starts first; the
-// verification is done while P^T streams, and nothing is left between two
-// decodes but one launch (a side stream for the verification, forked and
-// joined by events, kept them 6 to 10 us apart).  sync: the finished tiles of
-// each challenge, the finished CTAs of u and g, the CTAs of the verification
-// that are through; all zero at launch, and set back, with the tiles' status
-// words, by the last of those.  A wait that runs out lets its CTA go on, so
-// only a count of all of them says that none will use the words again.
+// A CTA waits only for CTAs of lower index (started first, as in
+// syndrome_tile); the verification is done while P^T streams, and nothing is
+// left between two decodes but one launch (a side stream for the verification,
+// forked and joined by events, kept them 6 to 10 us apart).  sync: the finished
+// tiles of each challenge, the finished CTAs of u and g, the CTAs of the
+// verification that are through; all zero at launch, and set back, with the
+// tiles' status words, by the last of those.  A wait that runs out lets its CTA
+// go on, so only a count of all of them says that none will use the words again
+// (4096 x 4096, 100 vectors 41.6 -> 41.8 us against a count of the checks).
 // ---------------------------------------------------------------------------
 constexpr int kSyncReady = 16, kSyncFinished = 17;
 static_assert(kSyncFinished < kDecodeSyncWords, "sync words");

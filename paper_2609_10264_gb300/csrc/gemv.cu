@@ -434,8 +434,10 @@ cudaError_t run_gemv_ring(const MvmJob *jobs, int count, cudaStream_t s) {
     // to back 346 -> 336).  Below the line the rings hold much of the share
     // and the overlap is worth more (dependent single calls, two CTAs against
     // one: 8192 x 4096 8.3 and 6.8 us, 6144 x 6144 8.0 and 7.6; above it
-    // 4096 x 14336 12.0 and 10.9, 8192 x 8192 11.0 and 11.6, gate and up of
-    // 14336 x 4096 17.3 and 18.7; 100 requests 249 and 237).
+    // 8192 x 8192 11.0 and 11.6, gate and up of 14336 x 4096 17.3 and 18.7;
+    // 100 requests 249 and 237).  4096 x 14336 pays 1.1 us for the even
+    // placement that the gate and up after it depend on (12.0 and 10.9): its
+    // 13 rows of 14 KiB a CTA leave a ring of two chunks little to run on.
     const long long total = args.base[count];
     const long long slots = count <= kRingFewJobs && total >= sms * kRingPairBytes ? 2LL * sms : sms;
     const int grid = (int)std::max(1LL, std::min({slots, rows, total / kRingMinBytes}));

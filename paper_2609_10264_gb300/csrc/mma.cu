@@ -760,7 +760,7 @@ cudaError_t batched_launch(const int8_t *W, int m, int K, const uint32_t *Xhat, 
 // of that, from one lane, had held the loads up.
 // One 8B-class layer for 64 vectors 84.7 -> 79.5 us, for 16 vectors 59.4 ->
 // 46.4; one 70B-class layer for 256 vectors 1092 -> 1020 us (1.72 PFLOP/s of
-// the four digits, at the power cap; a plain bf16 GEMM sustains 1.73).  Tiles of
+// the four digits, at the power cap; a plain bf16 GEMM sustains 1.69).  Tiles of
 // two K-blocks (128-byte rows) in the raw ring measured the same.
 // ---------------------------------------------------------------------------
 constexpr int kMaxGroupJobs = 8;

@@ -741,7 +741,8 @@ __global__ void __launch_bounds__(1024) k_slice_tables(const uint32_t *__restric
 // holds a state in its high half (1: the tile's own sum, 2: the inclusive
 // prefix through the tile) and the value in its low half, so a reader gets
 // state and value in one load and no fence or block barrier is needed.
-// A tile's predecessors are CTAs of lower index, which the GPU starts first.  (The earlier form, one flag per
+// A tile's predecessors are CTAs of lower index (started first, as in
+// syndrome_tile; with a ticket a launch took as long).  (The earlier form, one flag per
 // tile and the lanes' values in separate arrays behind a fence and block
 // barriers, with warp 0 reading 32 flags at a time, took 0.755 ms per
 // 4096 x 4096 encoding.)  At 32 positions per tile the kernel is held to 64

@@ -88,8 +88,10 @@ __device__ void warp_sample_values(const pvmvmd_key &key, uint32_t tag, uint64_t
 // fit beside a decrypt's.  The tables of a tile are requested before the
 // draw.  Tile sums are chained by a look-back over the tiles after it: their
 // own sums only, 32 at a time by one warp, since all of them are published
-// at about the same time.  A tile waits only for CTAs of lower index, which
-// the GPU starts first.  status holds one 64-bit word per (vector, tile)
+// at about the same time.  A tile waits only for CTAs of lower index: GPUs start
+// blocks in that order, though CUDA does not promise it, and where one did
+// not, the bounded waits would run out and be reported (a ticket per CTA would
+// cost each call an atomic's latency).  status holds one 64-bit word per (vector, tile)
 // (1 << 32 | sum), zero at launch; the gather kernel that follows clears it.
 //
 // Latency-bound.  Against one cluster of 2 to 8 CTAs of 1024 threads per
