@@ -841,13 +841,14 @@ def test_code_encode_lanes(pv, wl, m, K, which, L):
     ctx.destroy()
 
 
-def test_long_code_uses_three_kernel_path(pv, wl):
-    """K = 50000 gives N_x = 400000, too long for one cluster's shared memory,
-    so encode takes the sample / look-back scan / gather kernels; the result
-    must still equal the oracle."""
-    W = wl.weights_uniform(16, 50000, 9)
-    x = wl.int8_vectors(2, 50000, 10)
-    _full_round_trip(pv, W, x, seeds=(31, 32, 33))
+@pytest.mark.parametrize("m,K,kw", [(16, 50000, {}), (300, 14000, dict(t_x=513, t_y=600))])
+def test_long_code_uses_three_kernel_path(pv, wl, m, K, kw):
+    """Codes beyond one CTA's shared memory and the slices: N_x = 400000, by tiles,
+    and N_x = 112000 with supports that the tiles do not take, by the sample,
+    look-back scan and gather kernels (the challenges over two tiles too)."""
+    W = wl.weights_uniform(m, K, 9)
+    x = wl.int8_vectors(2, K, 10)
+    _full_round_trip(pv, W, x, seeds=(31, 32, 33), **(dict(params=_params(pv, **kw), oracle_kw=kw) if kw else {}))
 
 
 @pytest.mark.parametrize("layer,B", [("8b", 64), ("70b", 256)])
