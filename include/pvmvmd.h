@@ -21,8 +21,11 @@
  *  - Pointers named *_dev are CUDA device pointers on the current device;
  *    the caller owns them.  The library owns only what a context holds.
  *  - `stream` is a cudaStream_t passed as void* (NULL = legacy default
- *    stream).  Every call only enqueues work on that stream and returns;
- *    results are valid once the stream has been synchronised.  Calls that use
+ *    stream).  Every call only enqueues work and returns; results are valid
+ *    once the stream has been synchronised, and what a call reads and writes
+ *    of the caller's is read and written in that stream's order.  (A decode
+ *    may form its challenges, from the key and the context alone, on the
+ *    context's own stream before the caller's gets to it.)  Calls that use
  *    one context must be ordered on one stream (a context's internal scratch
  *    is shared by its calls), with one exception: an encode
  *    (pvmvmd_encode, pvmvmd_boost_prepare) and a decode
@@ -114,7 +117,10 @@ int pvmvmd_params_resolve(const pvmvmd_params *in, int m, int K, pvmvmd_params *
  * returning.  The context also owns one CUDA stream, created at the device's
  * highest stream priority, on which pvmvmd_decode_verify runs its short
  * verification kernels beside the decrypt (large calls run one kernel on the
- * caller's stream instead).  On error *out is NULL. */
+ * caller's stream instead).  The challenges start there without waiting for the
+ * caller's stream, but for a context that has been used under stream capture,
+ * since its graph may be replayed at any time, and after a verification on a
+ * caller's stream.  On error *out is NULL. */
 int pvmvmd_preprocess(const int8_t *W_dev, int m, int K, const pvmvmd_params *params,
                       const pvmvmd_key *key, void *stream, pvmvmd_ctx **out);
 
